@@ -72,10 +72,10 @@ typedef enum {
   RHMC_MIXED_FP32 = 1, /* FP32 operator and block updates inside an FP64-accurate
                           reliable-update / defect-correction loop; FP64 n x n
                           coefficient algebra, FP64 force.  The residuals of the
-                          loop use the double-float operator (RHMC_DF64) */
-  RHMC_DF64 = 2        /* operator only (apply / hop): FP64-accurate double-float
-                          arithmetic (pairs of FP32, about 2^-44 relative) on the
-                          FP32 units, which on this GPU are 74x faster than FP64 */
+                          loop use the FP64-accurate operator */
+  RHMC_DF64 = 2        /* operator only (apply / hop): FP64-accurate; the same arithmetic as
+                          RHMC_FP64 (exact integer sums of products on the integer units,
+                          several times faster than this GPU's FP64 units) */
 } rhmc_precision_t;
 
 /* Largest number of right-hand sides per block (n_pf). */
@@ -127,10 +127,11 @@ rhmc_status_t rhmc_apply_mdagm_mrhs(rhmc_ctx_t *ctx, const void *X_dev, void *Y_
  * for callers that must not allocate device memory (inside a stream capture,
  * under a fixed memory budget, or under a framework that owns all
  * allocation).  The paper has no counterpart; this is a deployment variant.
- * It allocates nothing: the odd-parity intermediate lives in a file-scope
- * device array of fixed size (32 MiB, i.e. V/2 * 3 * n_rhs * 16 bytes at most,
+ * It allocates nothing: the odd-parity intermediate lives in file-scope
+ * device arrays of fixed size (32 MiB, and a sixth as much for exponents; i.e. V/2 * 3 * n_rhs * 16 bytes at most,
  * e.g. a 16^4 lattice with 16 right-hand sides), which every GPU that loads
- * the library holds until the process exits.  Larger problems are rejected
+ * the library holds until the process exits; Y serves as scratch before the
+ * result is written.  Larger problems are rejected
  * with INVALID_ARG.  The first call on a device looks up the array's device
  * address (cudaGetSymbolAddress); make that first call before any stream
  * capture.  All calls share the array: calls that overlap on the GPU (other

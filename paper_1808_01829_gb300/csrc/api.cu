@@ -184,7 +184,8 @@ struct rhmc_ctx {
   int bc_t = -1;
   double2 *l64[2] = {nullptr, nullptr};
   float2 *l32[2] = {nullptr, nullptr};
-  float4 *ldf[2] = {nullptr, nullptr};  // double-float copy of the FP64 link records
+  int4 *lfx[2] = {nullptr, nullptr};    // integer copy of the FP64 link records (fx.cuh)
+  int *lexp[2] = {nullptr, nullptr};    // exponent of each site's largest link entry
   float2 *l12[2] = {nullptr, nullptr};  // first two rows of the FP32 records (used when every link is SU(3))
   bool rec12 = false;
   bool have_gauge = false;
@@ -260,9 +261,6 @@ template <typename T> struct LinksOf;
 template <> struct LinksOf<float> {
   static const float2 *get(const rhmc_ctx *c, int p) { return c->l32[p]; }
 };
-template <> struct LinksOf<double> {
-  static const double2 *get(const rhmc_ctx *c, int p) { return c->l64[p]; }
-};
 template <typename T> struct Links12Of;
 template <> struct Links12Of<float> {
   static const float2 *get(const rhmc_ctx *c, int p) {
@@ -270,55 +268,75 @@ template <> struct Links12Of<float> {
     return (c->rec12 && tune_get(TUNE_LINKS12) == 1) ? c->l12[p] : nullptr;
   }
 };
-template <> struct Links12Of<double> {
-  static const double2 *get(const rhmc_ctx *, int) { return nullptr; }
+
+static FxLinks fx_links(const rhmc_ctx *c, int p) { return {c->lfx[p], c->lexp[p], c->l64[p]}; }
+
+// Exponents of the two fields of an FP64-accurate operator application in integer form
+// (fx.cuh): Vh x n each.
+struct FxExp {
+  int *in = nullptr, *mid = nullptr;
 };
 
-// Y = (A + sigma) X, tmp: odd-parity field of the same width.
+// out = D in for FP64 fields, or out = a self - D in: on the integer units (FP64-accurate;
+// conv: an FP64-sized buffer for the converted input, not aliasing out), or in native FP64 with
+// RHMC_TUNE_NATIVE_FP64_RESIDUALS.
+static rhmc_status_t hop64(const rhmc_ctx *c, int par, const double2 *in, double2 *out, double2 *conv, int *ex, int n,
+                           cudaStream_t s) {
+  if (tune_get(TUNE_NATIVE_FP64_RESIDUALS))
+    return hop<double>(c->g, par, c->l64[par], in, out, nullptr, 0.0, n, 1, 0, s);
+  return hop_fx_to64(c->g, par, fx_links(c, par), in, {(int4 *)conv, ex}, out, n, s);
+}
+
+// Y = (A + sigma) X in FP64, tmp: odd-parity field of the same width.  Y may hold the
+// converted X until the second hop overwrites it.
+static rhmc_status_t apply_A64(const Geom &g, const FxLinks &even, const FxLinks &odd, double mass, const double2 *X,
+                               double2 *Y, double2 *tmp, FxExp ex, int n, double sigma, cudaStream_t s) {
+  const double a = 4.0 * mass * mass + sigma;
+  if (tune_get(TUNE_NATIVE_FP64_RESIDUALS)) {
+    RHMC_TRY(hop<double>(g, 1, odd.l64, X, tmp, nullptr, 0.0, n, 1, 0, s));
+    return hop<double>(g, 0, even.l64, tmp, Y, X, a, n, 1, 0, s);
+  }
+  const FxField fx{(int4 *)Y, ex.in}, ft{(int4 *)tmp, ex.mid};
+  RHMC_TRY(hop_fx(g, 1, odd, X, fx, ft, n, PROF_HOP64, s));
+  return hop_fx_self(g, 0, even, ft, Y, X, a, n, s);
+}
+rhmc_status_t apply_noalloc(const Geom &g, const FxLinks &even, const FxLinks &odd, double mass, const double2 *X,
+                            double2 *Y, double2 *tmp, int *exps, int n, double sigma, cudaStream_t s) {
+  return apply_A64(g, even, odd, mass, X, Y, tmp, {exps, exps + g.Vh * n}, n, sigma, s);
+}
+
 template <typename T>
-static rhmc_status_t apply_A(const rhmc_ctx *c, const C<T> *X, C<T> *Y, C<T> *tmp, int n, double sigma,
+static rhmc_status_t apply_A(const rhmc_ctx *c, const C<T> *X, C<T> *Y, C<T> *tmp, FxExp ex, int n, double sigma,
                              cudaStream_t s) {
-  RHMC_TRY(hop<T>(c->g, 1, LinksOf<T>::get(c, 1), X, tmp, nullptr, 0.0, n, 1, 0, s, Links12Of<T>::get(c, 1),
-                  c->bc_t));
-  RHMC_TRY(hop<T>(c->g, 0, LinksOf<T>::get(c, 0), tmp, Y, X, 4.0 * c->mass * c->mass + sigma, n, 1, 0, s,
-                  Links12Of<T>::get(c, 0), c->bc_t));
-  return RHMC_OK;
+  if constexpr (sizeof(T) == 8) {
+    return apply_A64(c->g, fx_links(c, 0), fx_links(c, 1), c->mass, X, Y, tmp, ex, n, sigma, s);
+  } else {
+    RHMC_TRY(hop<T>(c->g, 1, LinksOf<T>::get(c, 1), X, tmp, nullptr, 0.0, n, 1, 0, s, Links12Of<T>::get(c, 1),
+                    c->bc_t));
+    return hop<T>(c->g, 0, LinksOf<T>::get(c, 0), tmp, Y, X, 4.0 * c->mass * c->mass + sigma, n, 1, 0, s,
+                  Links12Of<T>::get(c, 0), c->bc_t);
+  }
 }
 
-// Y = (A + sigma) X with FP64 accuracy on the FP32 units (double-float):
-// split writes X as (hi, lo) into `split`, tmp holds the odd intermediate;
-// Y is written in FP64.  split, tmp, Y: FP64-field-sized buffers.
-static rhmc_status_t apply_A_df(const rhmc_ctx *c, const double2 *X, double2 *Y, double2 *tmp, double2 *split, int n,
-                                double sigma, cudaStream_t s) {
-  const long len = c->g.Vh * 3 * n;
-  RHMC_TRY(df_split(X, (float4 *)split, len, s));
-  RHMC_TRY(hop_df(c->g, 1, c->ldf[1], (const float4 *)split, (float4 *)tmp, nullptr, 0.0, n, s));
-  RHMC_TRY(hop_df(c->g, 0, c->ldf[0], (const float4 *)tmp, (float4 *)Y, (const float4 *)split,
-                  4.0 * c->mass * c->mass + sigma, n, s));
-  RHMC_TRY(df_merge((float4 *)Y, len, s));
-  return RHMC_OK;
-}
-
-// R = B - (A + sigma) X with FP64 accuracy for the mixed path; Rf (optional)
-// receives the FP32 rounding of R and npart (optional) the kParts x n column
-// partials of |R|^2.  Y, tmp, split: FP64-field-sized scratch; R may be split.
-// The double-float form subtracts the operator's (hi, lo) result directly.
+// R = B - (A + sigma) X with FP64 accuracy; Rf (optional) receives the FP32 rounding of R
+// and npart (optional) the kParts x n column partials of |R|^2.  tmp, ex, scratch
+// (hop_fx_parts x n doubles): scratch.  R may hold the converted X until the second hop, whose
+// epilogue subtracts.
 static rhmc_status_t residual_accurate(const rhmc_ctx *c, const double2 *B, const double2 *X, double2 *R,
-                                       float2 *Rf, double2 *Y, double2 *tmp, double2 *split, int n, double sigma,
+                                       float2 *Rf, double2 *tmp, FxExp ex, int n, double sigma, double *scratch,
                                        double *npart, cudaStream_t s) {
   const long rows = c->g.Vh * 3, len = rows * n;
   if (tune_get(TUNE_NATIVE_FP64_RESIDUALS)) {
-    RHMC_TRY(apply_A<double>(c, X, Y, tmp, n, sigma, s));
-    RHMC_TRY(sub(B, Y, R, len, s));
+    RHMC_TRY(apply_A<double>(c, X, R, tmp, ex, n, sigma, s));
+    RHMC_TRY(sub(B, R, R, len, s));
     if (Rf) RHMC_TRY((convert<double, float>(R, Rf, len, s)));
     if (npart) RHMC_TRY(colnorm2<double>(R, rows, n, npart, kParts, s));
     return RHMC_OK;
   }
-  RHMC_TRY(df_split(X, (float4 *)split, len, s));
-  RHMC_TRY(hop_df(c->g, 1, c->ldf[1], (const float4 *)split, (float4 *)tmp, nullptr, 0.0, n, s));
-  RHMC_TRY(hop_df(c->g, 0, c->ldf[0], (const float4 *)tmp, (float4 *)Y, (const float4 *)split,
-                  4.0 * c->mass * c->mass + sigma, n, s));
-  return resid_df(B, (const float4 *)Y, R, Rf, rows, n, npart, kParts, s);
+  const FxField fx{(int4 *)R, ex.in}, ft{(int4 *)tmp, ex.mid};
+  RHMC_TRY(hop_fx(c->g, 1, fx_links(c, 1), X, fx, ft, n, PROF_HOP_DF, s));
+  return resid_fx(c->g, fx_links(c, 0), ft, X, 4.0 * c->mass * c->mass + sigma, B, R, Rf, n, scratch, npart, kParts,
+                  s);
 }
 
 // ------------------------------------------------------------ solver workspace
@@ -331,7 +349,9 @@ struct SolveBufs {
   float *btiles;      // tensor-core B tiles of the shifted updates
   double2 *partial;   // the summed Gram matrix (n x n)
   double2 *gscratch;  // per-CTA Gram partials
-  double *npart;
+  double *npart;      // kParts x n column partials
+  double *nscr;       // per-CTA column sums of the residual kernel
+  FxExp ex;           // exponents of the integer fields of an FP64-accurate operator application
   SolverState *st;
   int accumulate = 0;  // shifts s >= 1 add w_s X^(s) into one field after X^(0) (FP64)
   // stored-basis mode (mixed, several shifts): the block basis Q_0 .. Q_{cap-1}
@@ -394,6 +414,9 @@ static void layout_solve(Arena &a, const Geom &g, int n, int ns, bool mixed, Sol
   b.partial = a.take<double2>((size_t)n * n);
   b.gscratch = a.take<double2>((size_t)kGramCtas * n * n);
   b.npart = a.take<double>((size_t)kParts * kMaxN);
+  b.nscr = a.take<double>((size_t)hop_fx_parts(g, n) * n);
+  b.ex.in = a.take<int>((size_t)g.Vh * n);
+  b.ex.mid = a.take<int>((size_t)g.Vh * n);
   b.st = a.take<SolverState>(1);
   const int cap = basis_cap(g, n, ns, mixed);
   if (cap > 0) {
@@ -526,7 +549,7 @@ static rhmc_status_t sbcgrq_iteration(rhmc_ctx *c, const SolveBufs &b, TX *Xacc,
   cudaStream_t ss = split ? c->side : s;
   // (chunk boundaries are joined on the host, so only waits inside a chunk are needed)
   if (split && k - 2 > chunk_start) RHMC_CUDA_TRY(cudaStreamWaitEvent(s, c->ev_side[(k - 2) % 3], 0));
-  RHMC_TRY(apply_A<T>(c, P, AP, Todd, n, sigma0, s));
+  RHMC_TRY(apply_A<T>(c, P, AP, Todd, b.ex, n, sigma0, s));
   RHMC_TRY(gram<T>(P, AP, rows, n, b.gscratch, b.partial, s));
   RHMC_TRY(nxn_alpha<T>(b.partial, kGramParts, n, b.st, k, (C<T> *)b.mw, s));
   const bool cols = use_column_update<T>();
@@ -820,7 +843,7 @@ static rhmc_status_t solve_phase1(rhmc_ctx *c, const double2 *B, int n, int ns, 
       // reliable update: flush FP32 increments, FP64 true base residual, re-QR
       for (int q = 0; q < nflush(); ++q) RHMC_TRY(flush(X + q * len, (float2 *)b.Xinc + q * len, len, s));
       // thin QR of the FP32-rounded true residual (Q is an FP32 basis)
-      RHMC_TRY(residual_accurate(c, B, X, b.R64, (float2 *)b.W, b.AP64, b.T64, b.R64, n, sigma0, nullptr, s));
+      RHMC_TRY(residual_accurate(c, B, X, b.R64, (float2 *)b.W, b.T64, b.ex, n, sigma0, b.nscr, nullptr, s));
       RHMC_TRY(gram<float>((float2 *)b.W, (float2 *)b.W, rows, n, b.gscratch, b.partial, s));
       RHMC_TRY(nxn_reliable<float>(b.partial, kGramParts, n, b.st, k, (float2 *)b.mw, s));
       // (the stored basis keeps the replaced block: P^(s)_k was formed from it, and the
@@ -919,15 +942,8 @@ static rhmc_status_t solve_all(rhmc_ctx *c, const double2 *B, int n, int ns, con
     SolveBufs &b1 = w.b1;
     for (int round = 0;; ++round) {
       double rn[kMaxN];
-      if (prm.mixed) {
-        RHMC_TRY(residual_accurate(c, B, Xq, w.rb.Bref, nullptr, b1.AP64, b1.T64, b1.R64, n, shifts[q], b1.npart,
-                                   ls));
-        RHMC_TRY(read_colnorms(c, b1.npart, n, rn, ls));
-      } else {
-        RHMC_TRY(apply_A<double>(c, Xq, b1.AP64, b1.T64, n, shifts[q], ls));
-        RHMC_TRY(sub(B, b1.AP64, w.rb.Bref, len, ls));
-        RHMC_TRY(colnorms(c, w.rb.Bref, n, rn, b1.npart, ls));
-      }
+      RHMC_TRY(residual_accurate(c, B, Xq, w.rb.Bref, nullptr, b1.T64, b1.ex, n, shifts[q], b1.nscr, b1.npart, ls));
+      RHMC_TRY(read_colnorms(c, b1.npart, n, rn, ls));
       w.dirac++;
       double mx = 0.0, ratio_min = 1e300;
       for (int j = 0; j < n; ++j) {
@@ -1033,8 +1049,7 @@ static rhmc_status_t solve_all(rhmc_ctx *c, const double2 *B, int n, int ns, con
   return RHMC_OK;
 }
 
-rhmc_status_t ctx_geometry(const rhmc_ctx_t *c, int *device, Geom *g, double *mass, const double2 **l64_even,
-                           const double2 **l64_odd) {
+rhmc_status_t ctx_geometry(const rhmc_ctx_t *c, int *device, Geom *g, double *mass, FxLinks *even, FxLinks *odd) {
   if (!c->have_gauge) {
     set_error("gauge field not set");
     return RHMC_ERR_NO_GAUGE;
@@ -1042,8 +1057,8 @@ rhmc_status_t ctx_geometry(const rhmc_ctx_t *c, int *device, Geom *g, double *ma
   *device = c->device;
   *g = c->g;
   *mass = c->mass;
-  *l64_even = c->l64[0];
-  *l64_odd = c->l64[1];
+  *even = fx_links(c, 0);
+  *odd = fx_links(c, 1);
   return RHMC_OK;
 }
 
@@ -1092,6 +1107,7 @@ static size_t scg_bytes(const Geom &g, int ns) {
   a.take<double>(kParts);
   a.take<double>(kMaxS);
   a.take<ScgScalars>(1);
+  a.take<int>((size_t)g.Vh * 2);
   return a.off + 256;
 }
 
@@ -1199,7 +1215,8 @@ rhmc_status_t rhmc_create(rhmc_ctx_t **out, const rhmc_lattice_t *lat, int devic
   for (int p = 0; p < 2; ++p) {
     if (cudaMalloc(&c->l64[p], sizeof(double2) * 72 * c->g.Vh) != cudaSuccess ||
         cudaMalloc(&c->l32[p], sizeof(float2) * 72 * c->g.Vh) != cudaSuccess ||
-        cudaMalloc(&c->ldf[p], sizeof(float4) * 72 * c->g.Vh) != cudaSuccess ||
+        cudaMalloc(&c->lfx[p], sizeof(int4) * 72 * c->g.Vh) != cudaSuccess ||
+        cudaMalloc(&c->lexp[p], sizeof(int) * c->g.Vh) != cudaSuccess ||
         cudaMalloc(&c->l12[p], sizeof(float2) * 48 * c->g.Vh) != cudaSuccess) {
       set_error("rhmc_create: out of device memory for links");
       rhmc_destroy(c);
@@ -1234,7 +1251,8 @@ rhmc_status_t rhmc_destroy(rhmc_ctx_t *c) {
   for (int p = 0; p < 2; ++p) {
     if (c->l64[p]) cudaFree(c->l64[p]);
     if (c->l32[p]) cudaFree(c->l32[p]);
-    if (c->ldf[p]) cudaFree(c->ldf[p]);
+    if (c->lfx[p]) cudaFree(c->lfx[p]);
+    if (c->lexp[p]) cudaFree(c->lexp[p]);
     if (c->l12[p]) cudaFree(c->l12[p]);
   }
   if (c->side) cudaStreamSynchronize(c->side);
@@ -1266,7 +1284,7 @@ rhmc_status_t rhmc_set_gauge(rhmc_ctx_t *c, const void *U, rhmc_stream_t sv) {
   TuneScope tscope(c);
   cudaStream_t s = (cudaStream_t)sv;
   RHMC_TRY(stage_links(c->g, (const double2 *)U, c->bc_t, c->l64, c->l32, s));
-  for (int p = 0; p < 2; ++p) RHMC_TRY(stage_links_df(c->g, c->l64[p], c->ldf[p], s));
+  for (int p = 0; p < 2; ++p) RHMC_TRY(stage_links_fx(c->g, c->l64[p], c->lfx[p], c->lexp[p], s));
   RHMC_TRY(stage_links12(c->g, c->bc_t, c->l32, c->l12, &c->rec12, s));
   RHMC_CUDA_TRY(cudaStreamSynchronize(s));
   c->have_gauge = true;
@@ -1282,7 +1300,8 @@ size_t rhmc_workspace_bytes(const rhmc_ctx_t *c, int n, int ns, rhmc_precision_t
   // solve with an internal X (unsorted shifts or force) + force's Y fields
   const size_t len = (size_t)c->g.Vh * 3 * n;
   size_t solve = solve_bytes(c->g, n, ns, mixed, true);
-  size_t force = sizeof(double2) * len * ns * 2 + sizeof(double) * (kMaxS + kParts) + 4096;
+  size_t force = sizeof(double2) * len * (ns * 2 + 1) + sizeof(int) * c->g.Vh * n + sizeof(double) * (kMaxS + kParts) +
+                 4096;
   return std::max(solve, force) + sizeof(double2) * len * ns + 4096;
 }
 
@@ -1313,21 +1332,18 @@ rhmc_status_t rhmc_apply_mdagm_mrhs(rhmc_ctx_t *c, const void *X, void *Y, int n
   TuneScope tscope(c);
   cudaStream_t s = (cudaStream_t)sv;
   const long len = c->g.Vh * 3 * n;
-  if (p == RHMC_FP64) {
-    RHMC_TRY(ensure_pool(c, sizeof(double2) * len + 256));
-    return apply_A<double>(c, (const double2 *)X, (double2 *)Y, (double2 *)c->pool, n, sigma, s);
-  }
-  if (p == RHMC_DF64) {
-    RHMC_TRY(ensure_pool(c, 2 * (sizeof(double2) * len + 256)));
+  if (p == RHMC_FP64 || p == RHMC_DF64) {  // both FP64-accurate on the integer units
+    RHMC_TRY(ensure_pool(c, sizeof(double2) * len + 2 * sizeof(int) * c->g.Vh * n + 1024));
     Arena a(c->pool);
-    double2 *tmp = a.take<double2>(len), *split = a.take<double2>(len);
-    return apply_A_df(c, (const double2 *)X, (double2 *)Y, tmp, split, n, sigma, s);
+    double2 *tmp = a.take<double2>(len);
+    FxExp ex{a.take<int>(c->g.Vh * n), a.take<int>(c->g.Vh * n)};
+    return apply_A<double>(c, (const double2 *)X, (double2 *)Y, tmp, ex, n, sigma, s);
   }
   RHMC_TRY(ensure_pool(c, 3 * (sizeof(float2) * len + 256)));
   Arena a(c->pool);
   float2 *x32 = a.take<float2>(len), *y32 = a.take<float2>(len), *t32 = a.take<float2>(len);
   RHMC_TRY((convert<double, float>((const double2 *)X, x32, len, s)));
-  RHMC_TRY(apply_A<float>(c, x32, y32, t32, n, sigma, s));
+  RHMC_TRY(apply_A<float>(c, x32, y32, t32, {}, n, sigma, s));
   RHMC_TRY((convert<float, double>(y32, (double2 *)Y, len, s)));
   return RHMC_OK;
 }
@@ -1343,12 +1359,11 @@ rhmc_status_t rhmc_hop(rhmc_ctx_t *c, const void *X, void *Y, int n, int out_par
   TuneScope tscope(c);
   cudaStream_t s = (cudaStream_t)sv;
   const long len = c->g.Vh * 3 * n;
-  if (p == RHMC_FP64) return hop<double>(c->g, out_par, c->l64[out_par], (const double2 *)X, (double2 *)Y, nullptr, 0, n, 1, 0, s);
-  if (p == RHMC_DF64) {
-    RHMC_TRY(ensure_pool(c, sizeof(double2) * len + 256));
-    RHMC_TRY(df_split((const double2 *)X, (float4 *)c->pool, len, s));
-    RHMC_TRY(hop_df(c->g, out_par, c->ldf[out_par], (const float4 *)c->pool, (float4 *)Y, nullptr, 0.0, n, s));
-    return df_merge((float4 *)Y, len, s);
+  if (p == RHMC_FP64 || p == RHMC_DF64) {
+    RHMC_TRY(ensure_pool(c, sizeof(double2) * len + sizeof(int) * c->g.Vh * n + 1024));
+    Arena a(c->pool);
+    double2 *conv = a.take<double2>(len);
+    return hop64(c, out_par, (const double2 *)X, (double2 *)Y, conv, a.take<int>(c->g.Vh * n), n, s);
   }
   RHMC_TRY(ensure_pool(c, 2 * (sizeof(float2) * len + 256)));
   Arena a(c->pool);
@@ -1527,9 +1542,10 @@ rhmc_status_t rhmc_multishift_cg_pervector(rhmc_ctx_t *c, const void *Bv, int n,
           *tmp = a.take<double2>(len1), *p = a.take<double2>(len1 * ns), *x = a.take<double2>(len1 * ns);
   double *parts = a.take<double>(kParts), *sig = a.take<double>(kMaxS);
   ScgScalars *sc = a.take<ScgScalars>(1);
+  int *exps = a.take<int>((size_t)c->g.Vh * 2);
+  const FxExp ex{exps, exps + c->g.Vh};
   RHMC_CUDA_TRY(cudaMemcpyAsync(sig, sh.data(), sizeof(double) * ns, cudaMemcpyHostToDevice, s));
   const int kmax = max_iter > 0 ? max_iter : default_max_iter(c, sh[0], tol);
-  const double a0 = 4.0 * c->mass * c->mass + sh[0];
   int total_iters = 0, dirac = 0;
   bool all_ok = true;
   RHMC_TRY(ensure_pinned(c, sizeof(ScgScalars)));
@@ -1547,8 +1563,7 @@ rhmc_status_t rhmc_multishift_cg_pervector(rhmc_ctx_t *c, const void *Bv, int n,
       const int chunk = std::min(kCheckEvery, kmax - k);
       for (int q = 0; q < chunk; ++q) {
         ++k;
-        RHMC_TRY(hop<double>(c->g, 1, c->l64[1], p, tmp, nullptr, 0.0, 1, 1, 0, s));
-        RHMC_TRY(hop<double>(c->g, 0, c->l64[0], tmp, Ap, p, a0, 1, 1, 0, s));
+        RHMC_TRY(apply_A<double>(c, p, Ap, tmp, ex, 1, sh[0], s));
         RHMC_TRY(redot(p, Ap, len1, parts, kParts, s));
         RHMC_TRY(scg_alpha(sc, parts, kParts, ns, s));
         RHMC_TRY(scg_update1(sc, r, Ap, x, p, ns, len1, parts, kParts, s));
@@ -1648,11 +1663,10 @@ rhmc_status_t rhmc_rational_solve(rhmc_ctx_t *c, const void *Phi, int n, double 
   double rec = 0.0;
   for (int q = 0; q < ns; ++q)
     for (int j = 0; j < n; ++j) rec = std::max(rec, v.res[q][j]);
-  RHMC_TRY(apply_A<double>(c, X2, b.AP64, b.T64, n, sh[0], s));
-  RHMC_TRY(sub((const double2 *)Phi, b.AP64, b.R64, len, s));
   double bn[kMaxN], rn[kMaxN];
   RHMC_TRY(colnorms(c, (const double2 *)Phi, n, bn, b.npart, s));
-  RHMC_TRY(colnorms(c, b.R64, n, rn, b.npart, s));
+  RHMC_TRY(residual_accurate(c, (const double2 *)Phi, X2, b.R64, nullptr, b.T64, b.ex, n, sh[0], b.nscr, b.npart, s));
+  RHMC_TRY(read_colnorms(c, b.npart, n, rn, s));
   double tr = 0.0;
   for (int j = 0; j < n; ++j) tr = std::max(tr, std::sqrt(rn[j] / bn[j]));
   // Y = alpha0 Phi + w_0 X^(0) + sum_{s>=1} w_s X^(s)
@@ -1720,7 +1734,7 @@ rhmc_status_t rhmc_force(rhmc_ctx_t *c, const void *Phi, int n, double alpha0, c
     std::memset(info, 0, sizeof(*info));
     info->per_shift_resid = user;
   }
-  // Y^(s) = D_oe X^(s), then the outer-product sum; FP64-accurate in
+  // Y^(s) = D_oe X^(s) on the integer units, then the outer-product sum; FP64-accurate in
   // double-float arithmetic on the FP32 units (native FP64 with
   // RHMC_TUNE_NATIVE_FP64_RESIDUALS)
   Arena fa(rest);
@@ -1728,6 +1742,7 @@ rhmc_status_t rhmc_force(rhmc_ctx_t *c, const void *Phi, int n, double alpha0, c
   void *Yf = fa.take<double2>((size_t)ns * len);
   double *alpha_d = fa.take<double>(kMaxS);
   double *parts = fa.take<double>(kParts);
+  const FxField fconv{fa.take<int4>((size_t)len), fa.take<int>((size_t)c->g.Vh * n)};  // one shift's X in integer form
   if (G) {
     RHMC_CUDA_TRY(cudaMemcpyAsync(alpha_d, alpha, sizeof(double) * ns, cudaMemcpyHostToDevice, s));
     if (tune_get(TUNE_NATIVE_FP64_RESIDUALS)) {
@@ -1738,7 +1753,7 @@ rhmc_status_t rhmc_force(rhmc_ctx_t *c, const void *Phi, int n, double alpha0, c
       float4 *Xd = (float4 *)Xf, *Yd = (float4 *)Yf;
       RHMC_TRY(df_split(X, Xd, (long)ns * len, s));
       for (int q = 0; q < ns; ++q)
-        RHMC_TRY(hop_df(c->g, 1, c->ldf[1], Xd + (size_t)q * len, Yd + (size_t)q * len, nullptr, 0.0, n, s));
+        RHMC_TRY(hop_fx_to_df(c->g, 1, fx_links(c, 1), X + (size_t)q * len, fconv, Yd + (size_t)q * len, n, s));
       RHMC_TRY(force_links_df(c->g, Xd, Yd, n, ns, len, alpha_d, c->bc_t, (double2 *)G, s));
     }
   }

@@ -15,6 +15,7 @@
 
 #include "common.cuh"
 #include "df.cuh"
+#include "fx.cuh"
 #include "kernels.h"
 
 namespace rhmc {
@@ -694,70 +695,427 @@ rhmc_status_t hop(const Geom &g, int par, const C<T> *links, const C<T> *in, C<T
   return RHMC_OK;
 }
 
-// ------------------------------------------------------------ double-float hop
-// FP64-accurate hop on the FP32 units (double-float arithmetic of df.cuh).
 using namespace df;
 
+// ------------------------------------------------------------ FP64-accurate hop on the integer units
+// The FP64 operator, the residuals of the solvers and the force's D_oe X: sums of
+// 24 complex products per output, formed exactly as integers (fx.cuh).  A field is
+// converted once (k_fx_convert; the first hop of an operator application writes its
+// result in integer form already), not by each of the eight neighbours that read it:
+// converting inside the hop took 465 us per hop at 24^4, n = 16.
+//
+// Integer link records, one int4 per complex of the FP64 records, and the exponent of each
+// site's largest entry (kSpecial where the site takes FP64 arithmetic).  Eight lanes
+// per site, one per direction.
+__global__ void __launch_bounds__(256) k_stage_links_fx(const double2 *__restrict__ l64, int4 *__restrict__ lfx,
+                                                        int *__restrict__ lexp, long nrec) {
+  const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;  // (site, direction)
+  const bool in = k < nrec;
+  double2 v[9];
+  int ef = 0;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    v[e] = in ? l64[k * 9 + e] : make_double2(0.0, 0.0);
+    ef = max(ef, max(fx::expo(v[e].x), fx::expo(v[e].y)));
+  }
+#pragma unroll
+  for (int off = 4; off > 0; off >>= 1) ef = max(ef, __shfl_xor_sync(0xffffffffu, ef, off, 8));
+  if (!in) return;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const int2 re = fx::split(v[e].x, ef), im = fx::split(v[e].y, ef);
+    lfx[k * 9 + e] = make_int4(re.x, re.y, im.x, im.y);
+  }
+  if ((k & 7) == 0) lexp[k >> 3] = (ef == 0 || ef == 0x7ff) ? fx::kSpecial : ef - 1022;
+}
 
-template <bool SELF>
-__global__ void __launch_bounds__(128) k_hop_df(Geom g, int par, const float4 *__restrict__ links,
-                                                const float4 *__restrict__ in, float4 *__restrict__ out,
-                                                const float4 *__restrict__ self, float ah, float al, int n, int tile) {
+rhmc_status_t stage_links_fx(const Geom &g, const double2 *l64, int4 *lfx, int *lexp, cudaStream_t s) {
+  const long n = g.Vh * 8;
+  k_stage_links_fx<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(l64, lfx, lexp, n);
+  RHMC_LAUNCH_CHECK();
+  return RHMC_OK;
+}
+
+// FP64 field [sites][3][n] -> integer form; one thread per (site, column)
+__global__ void __launch_bounds__(128) k_fx_convert(const double2 *__restrict__ in, int4 *__restrict__ out,
+                                                    int *__restrict__ ex, int count, int n) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= count) return;
+  const int h = k / n;
+  const long o = (long)h * 3 * n + (k - h * n);
+  double2 v[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) v[c] = in[o + c * n];
+  int4 q[3];
+  ex[k] = fx::pack3(v, q);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) out[o + c * n] = q[c];
+}
+
+static rhmc_status_t fx_convert(const Geom &g, const double2 *in, FxField out, int n, cudaStream_t s) {
+  if (n < 1 || n > RHMC_MAX_NRHS || g.Vh * 3L * n > 0x7fffffffL) return RHMC_ERR_INVALID_ARG;
+  const int count = (int)(g.Vh * n);
+  prof_begin(PROF_OTHER, s);
+  k_fx_convert<<<(unsigned)((count + 127) / 128), 128, 0, s>>>(in, out.v, out.e, count, n);
+  prof_end(s, (double)count * (3 * 32.0 + 4.0));
+  RHMC_LAUNCH_CHECK();
+  return RHMC_OK;
+}
+
+// S lanes of a warp per (site, right-hand side), 8 / S directions each, `tile` sites per
+// CTA.  The tile's link records go to shared memory by cp.async (padded to 73 int4,
+// so that the sites of a warp read different banks).  A lane shifts each neighbour's
+// words to the largest of the eight exponents and adds up its products: 648 integer
+// multiply-adds of four clocks per (site, right-hand side), which bound the kernel
+// on large lattices, and about 60 shifts and adds per direction on the other pipes.
+// (Shifting every direction's sums instead took 350 us per hop at 24^4, n = 16,
+// and 380 us without the three-product form.)  The loop over the directions
+// is not unrolled: the unrolled body waited for the instruction cache.
+// S = 4 where one lane per (site, right-hand side) would leave the schedulers without
+// warps (small lattices): the lanes' integer sums are added by shuffles, and three of
+// the four lanes write one colour each.  With S = 4 an FP64 input (IN64) is converted here:
+// a separate pass would cost a launch, and each value is read by few warps.
+// Measured per hop, FP64 fields: 24^4, n = 16 353 us (and 60 us to convert the input of
+// the first hop) against 1246 us with FP64 FMAs; an operator application at 8^4,
+// n = 4 16 against 37 us.  Against a long-double sum its error is 1.0e-16 relative for
+// Gaussian fields, that of FP64 FMAs 2.9e-16.
+// Lanes with a special block among their inputs, or neighbours more than 2^26
+// apart in size, take FP64 arithmetic.
+//
+// MODE 0: out = D in.  1: out = a self - D in.  2: out = B - (a self - D in), with
+// the optional FP32 rounding outf and per-CTA column sums of |out|^2 (part).
+// 3: out = D in as double-float pairs (float4).  4: D in in integer form, exponents oex.
+template <int MODE, int S, bool IN64>
+__global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *__restrict__ lfx,
+                                                   const int *__restrict__ lexp, const double2 *__restrict__ l64,
+                                                   const int4 *__restrict__ in, const int *__restrict__ iex,
+                                                   void *outv, int *__restrict__ oex, const double2 *self, double a,
+                                                   int n, int tile, const double2 *__restrict__ B,
+                                                   float2 *__restrict__ outf, double *__restrict__ part) {
+  constexpr int LS = 73;
+  constexpr int IW = 32 / S;  // (site, right-hand side) items per warp
+  constexpr int ND = 8 / S;   // directions per lane
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4 *sl = reinterpret_cast<float4 *>(smem_raw);
-  int *snb = reinterpret_cast<int *>(smem_raw + (size_t)tile * 72 * sizeof(float4));
+  const int tid = threadIdx.x, nt = blockDim.x;
+  int4 *sl = reinterpret_cast<int4 *>(smem_raw);
+  int *snb = reinterpret_cast<int *>(sl + tile * LS);
   const int h0 = blockIdx.x * tile;
   const int nsites = min(tile, (int)g.Vh - h0);
-  for (int k = threadIdx.x; k < nsites * 72; k += blockDim.x) sl[k] = links[(long)h0 * 72 + k];
-  for (int k = threadIdx.x; k < nsites * 8; k += blockDim.x) {
+  {
+    const unsigned base = (unsigned)__cvta_generic_to_shared(sl);
+    const char *src = reinterpret_cast<const char *>(lfx + (long)h0 * 72);
+    for (int c = tid; c < nsites * 72; c += nt) {
+      const int site = c / 72;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(base + 16u * (unsigned)(c + site)),
+                   "l"(src + 16L * c)
+                   : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  for (int k = tid; k < nsites * 8; k += nt) {
     const int site = k >> 3, d = k & 7;
-    int x[4];
-    site_coords(g, par, h0 + site, x);
-    const int mu = d & 3, st = d < 4 ? 1 : -1;
-    int y0 = x[0], y1 = x[1], y2 = x[2], y3 = x[3];
-    if (mu == 0) y0 = (y0 + st + g.L[0]) % g.L[0];
-    else if (mu == 1) y1 = (y1 + st + g.L[1]) % g.L[1];
-    else if (mu == 2) y2 = (y2 + st + g.L[2]) % g.L[2];
-    else y3 = (y3 + st + g.L[3]) % g.L[3];
+    int y0, y1, y2, y3;
+    site_coords32(g, par, h0 + site, y0, y1, y2, y3);
+    const int mu = d & 3;
+    const bool fwd = d < 4;
+    if (mu == 0) y0 = fwd ? (y0 + 1 == g.L[0] ? 0 : y0 + 1) : (y0 == 0 ? g.L[0] - 1 : y0 - 1);
+    else if (mu == 1) y1 = fwd ? (y1 + 1 == g.L[1] ? 0 : y1 + 1) : (y1 == 0 ? g.L[1] - 1 : y1 - 1);
+    else if (mu == 2) y2 = fwd ? (y2 + 1 == g.L[2] ? 0 : y2 + 1) : (y2 == 0 ? g.L[2] - 1 : y2 - 1);
+    else y3 = fwd ? (y3 + 1 == g.L[3] ? 0 : y3 + 1) : (y3 == 0 ? g.L[3] - 1 : y3 - 1);
     const int lex = y0 + g.L[0] * (y1 + g.L[1] * (y2 + g.L[2] * y3));
-    snb[k] = (lex >> 1) * 3 * n;
+    snb[k] = lex >> 1;
   }
   __syncthreads();
-  const int ls = threadIdx.x / n, j = threadIdx.x - ls * n;
-  if (ls >= nsites) return;
-  const int h = h0 + ls;
-  DF re[3], im[3];
+  const int lane = tid & 31, quad = lane / IW;  // which 8 / S of the directions
+  const int item = (tid >> 5) * IW + (lane - quad * IW);
+  const int ls = item / n, j = item - ls * n;
+  const bool live = ls < nsites;
+  const int *nb = snb + (live ? ls : 0) * 8;
+  const int n3 = 3 * n, d0 = quad * ND;
+  const double2 *in64 = reinterpret_cast<const double2 *>(in);
+  int E = fx::kZero, low = fx::kSpecial, el = 0, ef = 0;
+  int4 v[3];
+  double2 x64[IN64 ? ND : 1][3];
+  if (IN64) {
+    bool any = false;
+    if (live) {
+      el = lexp[h0 + ls];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) re[c] = im[c] = DF{0.f, 0.f};
-#pragma unroll 1
-  for (int d = 0; d < 8; ++d) {
-    const float4 *v = in + snb[ls * 8 + d] + j;
-    const float4 v0 = v[0], v1 = v[n], v2 = v[2 * n];
-    const float4 *l = sl + ls * 72 + d * 9;
+      for (int d = 0; d < ND; ++d)
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      df_cmac(re[a], im[a], l[a * 3 + 0], v0);
-      df_cmac(re[a], im[a], l[a * 3 + 1], v1);
-      df_cmac(re[a], im[a], l[a * 3 + 2], v2);
+        for (int c = 0; c < 3; ++c) x64[IN64 ? d : 0][c] = __ldg(in64 + (nb[d0 + d] * n3 + j) + c * n);
+#pragma unroll
+      for (int d = 0; d < ND; ++d)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const double2 x = x64[IN64 ? d : 0][c];
+          ef = max(ef, max(fx::expo(x.x), fx::expo(x.y)));
+          any = any || fx::nonzero(x.x) || fx::nonzero(x.y);
+        }
+    }
+#pragma unroll
+    for (int off = IW; off < 32; off <<= 1) {
+      ef = max(ef, __shfl_xor_sync(0xffffffffu, ef, off));
+      any = __shfl_xor_sync(0xffffffffu, (int)any, off) || any;
+    }
+    E = !any ? fx::kZero : (ef == 0 || ef == 0x7ff) ? fx::kSpecial : ef - 1022;
+    low = E;
+  } else if (live) {
+    el = lexp[h0 + ls];
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+      const int e = iex[nb[d0 + d] * n + j];
+      E = max(E, e);
+      low = min(low, e == fx::kZero ? fx::kSpecial : e);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) v[c] = __ldg(in + (nb[d0] * n3 + j) + c * n);
+  }
+  if (!IN64) {
+#pragma unroll
+    for (int off = IW; off < 32; off <<= 1) {
+      E = max(E, __shfl_xor_sync(0xffffffffu, E, off));
+      low = min(low, __shfl_xor_sync(0xffffffffu, low, off));
     }
   }
-  const int o = h * 3 * n + j;
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  const bool fast = E != fx::kSpecial && el != fx::kSpecial && (E == fx::kZero || E - low <= fx::kAlign);
+  long long R[6];
+  if (live && fast) {
+    long long pA[3], pB[3], mA[3], mB[3], iA[3], iB[3];  // sums of a c, b d, (a + b)(c + d)
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    if (SELF) {
-      // result = a * self - D in: negate the hop sum, add the scaled self term
-      DF r2{-re[c].h, -re[c].e}, i2{-im[c].h, -im[c].e};
-      const float4 sv = self[o + c * n];
-      df_add_prod(r2, ah, al, sv.x, sv.z);
-      df_add_prod(i2, ah, al, sv.y, sv.w);
-      out[o + c * n] = df_pack(r2, i2);
+    for (int c = 0; c < 3; ++c) pA[c] = pB[c] = mA[c] = mB[c] = iA[c] = iB[c] = 0;
+    const int4 *lk = sl + ls * LS + d0 * 9;
+    auto add = [&](int4 w, const int4 *l3) {  // one neighbour colour times the links' column
+      const int sx = w.x + w.z, sy = w.y + w.w;
+#pragma unroll
+      for (int ca = 0; ca < 3; ++ca) {
+        const int4 l = l3[ca * 3];
+        fx::mac2(pA[ca], pB[ca], l.x, l.y, w.x, w.y);
+        fx::mac2(mA[ca], mB[ca], l.z, l.w, w.z, w.w);
+        fx::mac2(iA[ca], iB[ca], l.x + l.z, l.y + l.w, sx, sy);
+      }
+    };
+    if constexpr (IN64) {
+#pragma unroll
+      for (int d = 0; d < ND; ++d)
+#pragma unroll
+        for (int cb = 0; cb < 3; ++cb) {
+          const int2 re = fx::split(x64[d][cb].x, ef), im = fx::split(x64[d][cb].y, ef);
+          add(make_int4(re.x, re.y, im.x, im.y), lk + d * 9 + cb);
+        }
     } else {
-      out[o + c * n] = df_pack(re[c], im[c]);
+#pragma unroll 1
+      for (int d = d0; d < d0 + ND; ++d, lk += 9) {
+        const int sh = min(fx::kAlign, E - iex[nb[d] * n + j]);  // (clamped for zeros only)
+        int4 w[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) w[c] = v[c];
+        if (d < d0 + ND - 1) {  // the next direction's values are in flight while this one's are multiplied
+          const int4 *p = in + (nb[d + 1] * n3 + j);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) v[c] = __ldg(p + c * n);
+        }
+#pragma unroll
+        for (int cb = 0; cb < 3; ++cb) {
+          fx::align(w[cb].x, w[cb].y, sh);
+          fx::align(w[cb].z, w[cb].w, sh);
+          add(w[cb], lk + cb);
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      R[2 * c] = fx::join(pA[c] - mA[c], pB[c] - mB[c]);
+      R[2 * c + 1] = fx::join(iA[c] - pA[c] - mA[c], iB[c] - pB[c] - mB[c]);
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 6; ++c) R[c] = 0;
+  }
+#pragma unroll
+  for (int off = IW; off < 32; off <<= 1)
+#pragma unroll
+    for (int c = 0; c < 6; ++c) R[c] += __shfl_xor_sync(0xffffffffu, R[c], off);
+  double nrm = 0.0;
+  if (live) {
+    const int c0 = S == 1 ? 0 : quad, c1 = S == 1 ? 3 : min(3, quad + 1);  // this lane's colours
+    const long o = (long)(h0 + ls) * n3 + j;
+    const int k = E + el - 56;
+    double2 acc[3];
+    if (!fast) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) acc[c] = make_double2(0.0, 0.0);
+      const double2 *L = l64 + (long)(h0 + ls) * 72;
+#pragma unroll 1
+      for (int q = 0; q < 24; ++q) {
+        const int d = q / 3, cb = q - d * 3;
+        const double2 w = IN64 ? in64[nb[d] * n3 + j + cb * n]
+                               : fx::unpack(in[nb[d] * n3 + j + cb * n], iex[nb[d] * n + j]);
+        const double2 *l = L + d * 9 + cb;
+#pragma unroll
+        for (int ca = 0; ca < 3; ++ca) cmac<double>(acc[ca], l[ca * 3], w);
+      }
+    }
+    if (MODE == 4) {
+      int4 q[3];
+      int e;
+      if (!fast) {
+        e = fx::pack3(acc, q);
+      } else if (E == fx::kZero) {
+        e = fx::kZero;
+        q[0] = q[1] = q[2] = make_int4(0, 0, 0, 0);
+      } else {
+        e = fx::renorm3(R, k, q);
+      }
+      if (quad == 0) oex[(long)(h0 + ls) * n + j] = e;
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        if (c >= c0 && c < c1) reinterpret_cast<int4 *>(outv)[o + c * n] = q[c];
+      return;
+    }
+    double2 *out = reinterpret_cast<double2 *>(outv);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      if (c < c0 || c >= c1) continue;
+      double2 r = fast ? make_double2(fx::value(R[2 * c], k), fx::value(R[2 * c + 1], k)) : acc[c];
+      if (MODE == 1 || MODE == 2) {
+        const double2 s = self[o + c * n];
+        r = make_double2(fma(a, s.x, -r.x), fma(a, s.y, -r.y));
+      }
+      if (MODE == 2) {
+        const double2 b = B[o + c * n];
+        r = make_double2(b.x - r.x, b.y - r.y);
+        if (outf) outf[o + c * n] = make_float2((float)r.x, (float)r.y);
+        if (part) nrm = fma(r.x, r.x, fma(r.y, r.y, nrm));
+      }
+      if (MODE == 3) {
+        const float2 x = df_split1(r.x), y = df_split1(r.y);
+        reinterpret_cast<float4 *>(outv)[o + c * n] = make_float4(x.x, y.x, x.y, y.y);
+      } else {
+        out[o + c * n] = r;
+      }
+    }
+  }
+  if (MODE == 2 && part) {  // column sums over the CTA's sites (fixed order)
+    double *red = reinterpret_cast<double *>(smem_raw);
+#pragma unroll
+    for (int off = IW; off < 32; off <<= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
+    __syncthreads();
+    if (quad == 0) red[item] = nrm;
+    __syncthreads();
+    if (tid < n) {
+      double sum = 0.0;
+      for (int q = 0; q < nsites; ++q) sum += red[q * n + tid];
+      part[(long)blockIdx.x * n + tid] = sum;
     }
   }
 }
 
-// FP64 <-> double-float conversion of complex fields (to_df: d -> (hi, lo)).
+// out[p * n + c] = sum of the rows p, p + gridDim.x, ... of part (nblk x n), fixed order
+__global__ void __launch_bounds__(256) k_fold_parts(const double *__restrict__ part, int nblk, int n,
+                                                    double *__restrict__ out) {
+  __shared__ double red[256];
+  const int t = threadIdx.x, per = 256 / n, c = t % n, q0 = t / n;
+  double s = 0.0;
+  if (q0 < per)
+    for (long r = (long)blockIdx.x + (long)q0 * gridDim.x; r < nblk; r += (long)per * gridDim.x) s += part[r * n + c];
+  red[t] = s;
+  __syncthreads();
+  if (t < n) {
+    double sum = 0.0;
+    for (int q = 0; q < per; ++q) sum += red[q * n + t];
+    out[(long)blockIdx.x * n + t] = sum;
+  }
+}
+
+// Lanes per (site, right-hand side): four up to two warps per scheduler (four schedulers on
+// each of 152 SMs), else one.  Sites per CTA: up to 128 threads, but at least a warp's
+// worth while that gives the SMs more than two CTAs each, and at most 32 link records.
+static int fx_split(const Geom &g, int n) { return g.Vh * n <= 2L * 4 * 152 * 32 ? 4 : 1; }
+static int fx_tile(const Geom &g, int n) {
+  const int items = 128 / fx_split(g, n);
+  const int least = std::max(1, items / 4 / n);
+  int tile = std::max(std::min(items / n, 32), least);
+  while (tile > least && (g.Vh + tile - 1) / tile < 2 * 152) tile = std::max(least, tile / 2);
+  return tile;
+}
+
+long hop_fx_parts(const Geom &g, int n) {
+  const int tile = fx_tile(g, n);
+  return (g.Vh + tile - 1) / tile;
+}
+
+// in64 (optional): the input in FP64; the small-lattice kernel converts it itself, else it is
+// converted into `in` first.
+template <int MODE>
+static rhmc_status_t launch_hop_fx(const Geom &g, int par, const FxLinks &L, const double2 *in64, FxField in,
+                                   void *out, int *oex, const double2 *self, double a, int n, const double2 *B,
+                                   float2 *outf, double *part, int cat, cudaStream_t s) {
+  if (n < 1 || n > RHMC_MAX_NRHS || g.Vh * 3L * n > 0x7fffffffL) return RHMC_ERR_INVALID_ARG;
+  const int split = fx_split(g, n), iw = 32 / split;
+  if (in64 && split == 1) RHMC_TRY(fx_convert(g, in64, in, n, s));
+  const int tile = fx_tile(g, n);
+  const int threads = (tile * n + iw - 1) / iw * 32;
+  const size_t smem = (size_t)tile * (73 * sizeof(int4) + 8 * sizeof(int));
+  const unsigned grid = (unsigned)((g.Vh + tile - 1) / tile);
+  prof_begin(cat, s);
+  auto run = [&](auto kern, const int4 *src) {
+    kern<<<grid, threads, smem, s>>>(g, par, L.rec, L.exp, L.l64, src, in.e, out, oex, self, a, n, tile, B, outf, part);
+  };
+  bool done = false;
+  if constexpr (MODE == 0 || MODE == 3 || MODE == 4) {
+    if (in64 && split == 4) {
+      run(k_hop_fx<MODE, 4, true>, reinterpret_cast<const int4 *>(in64));
+      done = true;
+    }
+  }
+  if (!done) {
+    if (split == 4)
+      run(k_hop_fx<MODE, 4, false>, in.v);
+    else
+      run(k_hop_fx<MODE, 1, false>, in.v);
+  }
+  // algorithmic bytes: every link once, the inputs once, the outputs once
+  const double fields = 2.0 + (MODE == 1 ? 1.0 : 0.0) + (MODE == 2 ? 2.0 + (outf ? 0.5 : 0.0) : 0.0);
+  prof_end(s, (double)g.Vh * 16 * (72.0 + 3.0 * n * fields));
+  RHMC_LAUNCH_CHECK();
+  return RHMC_OK;
+}
+
+rhmc_status_t hop_fx(const Geom &g, int par, const FxLinks &L, const double2 *in, FxField conv, FxField out, int n,
+                     int cat, cudaStream_t s) {
+  return launch_hop_fx<4>(g, par, L, in, conv, out.v, out.e, nullptr, 0.0, n, nullptr, nullptr, nullptr, cat, s);
+}
+
+rhmc_status_t hop_fx_to64(const Geom &g, int par, const FxLinks &L, const double2 *in, FxField conv, double2 *out,
+                          int n, cudaStream_t s) {
+  return launch_hop_fx<0>(g, par, L, in, conv, out, nullptr, nullptr, 0.0, n, nullptr, nullptr, nullptr, PROF_HOP64, s);
+}
+
+rhmc_status_t hop_fx_self(const Geom &g, int par, const FxLinks &L, FxField in, double2 *out, const double2 *self,
+                          double a, int n, cudaStream_t s) {
+  return launch_hop_fx<1>(g, par, L, nullptr, in, out, nullptr, self, a, n, nullptr, nullptr, nullptr, PROF_HOP64, s);
+}
+
+rhmc_status_t hop_fx_to_df(const Geom &g, int par, const FxLinks &L, const double2 *in, FxField conv, float4 *out,
+                           int n, cudaStream_t s) {
+  return launch_hop_fx<3>(g, par, L, in, conv, out, nullptr, nullptr, 0.0, n, nullptr, nullptr, nullptr, PROF_HOP_DF,
+                          s);
+}
+
+rhmc_status_t resid_fx(const Geom &g, const FxLinks &L, FxField tmp, const double2 *X, double a, const double2 *B,
+                       double2 *R, float2 *Rf, int n, double *scratch, double *part, int nparts, cudaStream_t s) {
+  RHMC_TRY(launch_hop_fx<2>(g, 0, L, nullptr, tmp, R, nullptr, X, a, n, B, Rf, part ? scratch : nullptr, PROF_HOP_DF, s));
+  if (part) {
+    k_fold_parts<<<nparts, 256, 0, s>>>(scratch, (int)hop_fx_parts(g, n), n, part);
+    RHMC_LAUNCH_CHECK();
+  }
+  return RHMC_OK;
+}
+
+// FP64 -> double-float pairs of complex fields (the force kernel's operands).
 __global__ void k_df_convert(const double2 *__restrict__ in64, float4 *__restrict__ outdf, long len) {
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= len) return;
@@ -765,115 +1123,9 @@ __global__ void k_df_convert(const double2 *__restrict__ in64, float4 *__restric
   const float2 a = df_split1(z.x), b = df_split1(z.y);
   outdf[i] = make_float4(a.x, b.x, a.y, b.y);
 }
-__global__ void k_df_merge(float4 *__restrict__ io, long len) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= len) return;
-  const float4 v = io[i];
-  reinterpret_cast<double2 *>(io)[i] = make_double2(df_merge1(v.x, v.z), df_merge1(v.y, v.w));
-}
-
-// R = B - Y in FP64 for Y in double-float as the second hop writes it:
-// (B - hi) - lo, which needs no FP64 copy of Y.  Optionally Rf, the FP32
-// rounding of R, and per-CTA sums of |R|^2 per column (n interleaved
-// columns; partial[cta * n + column], CTA order fixed, so the host's sum of
-// the partials is deterministic).  Thread t owns column t % n of every
-// (256 / n)-th row; four rows are loaded before any is used.
-__global__ void __launch_bounds__(256) k_resid_df(const double2 *__restrict__ B, const float4 *__restrict__ Y,
-                                                  double2 *__restrict__ R, float2 *__restrict__ Rf, long rows,
-                                                  int n, double *__restrict__ partial) {
-  __shared__ double red[256];
-  const int t = threadIdx.x;
-  const int per = 256 / n;
-  const int c = t % n, g = t / n;
-  const long step = (long)gridDim.x * per;
-  double acc = 0.0;
-  if (g < per) {
-    long r = (long)blockIdx.x * per + g;
-    for (; r + 3 * step < rows; r += 4 * step) {
-      double2 b[4];
-      float4 y[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        b[u] = B[(r + u * step) * n + c];
-        y[u] = Y[(r + u * step) * n + c];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const double x = (b[u].x - df_widen1(y[u].x)) - df_widen1(y[u].z);
-        const double z = (b[u].y - df_widen1(y[u].y)) - df_widen1(y[u].w);
-        const long i = (r + u * step) * n + c;
-        R[i] = make_double2(x, z);
-        if (Rf) Rf[i] = make_float2((float)x, (float)z);
-        acc += x * x + z * z;
-      }
-    }
-    for (; r < rows; r += step) {
-      const long i = r * n + c;
-      const double2 bv = B[i];
-      const float4 yv = Y[i];
-      const double x = (bv.x - df_widen1(yv.x)) - df_widen1(yv.z);
-      const double z = (bv.y - df_widen1(yv.y)) - df_widen1(yv.w);
-      R[i] = make_double2(x, z);
-      if (Rf) Rf[i] = make_float2((float)x, (float)z);
-      acc += x * x + z * z;
-    }
-  }
-  if (!partial) return;
-  red[t] = acc;
-  __syncthreads();
-  if (t < n) {
-    double sum = 0.0;
-    for (int q = 0; q < per; ++q) sum += red[q * n + t];
-    partial[(long)blockIdx.x * n + t] = sum;
-  }
-}
-
-rhmc_status_t resid_df(const double2 *B, const float4 *Y, double2 *R, float2 *Rf, long rows, int n,
-                       double *partial, int nparts, cudaStream_t s) {
-  if (n < 1 || n > RHMC_MAX_NRHS || nparts < 1) return RHMC_ERR_INVALID_ARG;
-  k_resid_df<<<nparts, 256, 0, s>>>(B, Y, R, Rf, rows, n, partial);
-  RHMC_LAUNCH_CHECK();
-  return RHMC_OK;
-}
-
-rhmc_status_t stage_links_df(const Geom &g, const double2 *l64, float4 *ldf, cudaStream_t s) {
-  const long len = g.Vh * 72;
-  k_df_convert<<<(unsigned)((len + 255) / 256), 256, 0, s>>>(l64, ldf, len);
-  RHMC_LAUNCH_CHECK();
-  return RHMC_OK;
-}
 
 rhmc_status_t df_split(const double2 *in, float4 *out, long len, cudaStream_t s) {
   k_df_convert<<<(unsigned)((len + 255) / 256), 256, 0, s>>>(in, out, len);
-  RHMC_LAUNCH_CHECK();
-  return RHMC_OK;
-}
-
-rhmc_status_t df_merge(float4 *io, long len, cudaStream_t s) {
-  k_df_merge<<<(unsigned)((len + 255) / 256), 256, 0, s>>>(io, len);
-  RHMC_LAUNCH_CHECK();
-  return RHMC_OK;
-}
-
-rhmc_status_t hop_df(const Geom &g, int par, const float4 *links, const float4 *in, float4 *out, const float4 *self,
-                     double a, int n, cudaStream_t s) {
-  if (n < 1 || n > RHMC_MAX_NRHS || g.Vh * 3L * n > 0x7fffffffL) return RHMC_ERR_INVALID_ARG;
-  const int tile = max(1, 128 / n);
-  const int threads = ((tile * n + 31) / 32) * 32;
-  const size_t smem = (size_t)tile * 72 * sizeof(float4) + (size_t)tile * 8 * sizeof(int);
-  static std::once_flag attr;
-  std::call_once(attr, [&] {
-    cudaFuncSetAttribute(k_hop_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_hop_df<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  });
-  const float ah = (float)a, al = (float)(a - (double)ah);
-  const unsigned grid = (unsigned)((g.Vh + tile - 1) / tile);
-  prof_begin(PROF_HOP_DF, s);
-  if (self)
-    k_hop_df<true><<<grid, threads, smem, s>>>(g, par, links, in, out, self, ah, al, n, tile);
-  else
-    k_hop_df<false><<<grid, threads, smem, s>>>(g, par, links, in, out, self, ah, al, n, tile);
-  prof_end(s, (double)g.Vh * sizeof(float4) * (72.0 + 3.0 * n * (self ? 3 : 2)));
   RHMC_LAUNCH_CHECK();
   return RHMC_OK;
 }

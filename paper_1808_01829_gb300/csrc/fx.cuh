@@ -1,0 +1,141 @@
+// FP64-accurate sums of products on the integer units.  This GPU issues two
+// FP64 operations per clock and SM (a warp's DFMA takes 64 clocks); a 32 x 32 ->
+// 64 bit integer multiply-add of a warp takes four (measured), so a dot product whose
+// operands are first brought to a common exponent runs several times faster as
+// integers than as FP64 FMAs.
+//
+// A block of reals x with |x| < 2^E is held as q = x 2^(55 - E), truncated, in
+// two signed words q = hi 2^27 + lo with |hi| <= 2^28 and -2^26 <= lo < 2^26.
+// Values within a factor of 4 of the block's largest are exact; smaller ones lose
+// what lies below 2^-55 of 2^E (an FP64 sum rounds every step at 2^-53 of the
+// running sum).  A product of two such numbers is
+//   2^(E1 + E2 - 56) [h1 h2 + (h1 l2 + l1 h2) 2^-27 + l1 l2 2^-54],
+// whose last term is below 2^-58 of 2^(E1 + E2) and dropped.  The sums A = sum h h
+// and B = sum (h l + l h) are exact.
+//
+// A complex product (a + i b)(c + i d) takes three real ones, a c, b d and
+// (a + b)(c + d); as integers nothing is lost in their differences.  Over up to
+// 24 complex products |A| <= 24 2^58 < 2^63 and, with the second factor's words
+// aligned (|lo| < 1.25 2^27), |B| <= 24 (2^29 1.25 2^28 + 2^27 2^29) < 2^63.
+//
+// A field in this form has one int4 (re hi, re lo, im hi, im lo) per complex, as
+// large as its FP64 form, and one exponent E per (site, column) for the three
+// colours.  Blocks with infinities, NaN or subnormals keep their FP64 values in the
+// int4 under the exponent kSpecial; kZero marks a block of zeros.
+#pragma once
+
+namespace rhmc {
+namespace fx {
+
+constexpr int kLow = 27;              // bits of the low word
+constexpr int kBits = 55;             // magnitude bits
+constexpr int kSpecial = 1 << 20;     // exponent code: the block holds FP64 values
+constexpr int kZero = -(1 << 20);     // exponent code: all zeros
+
+// biased exponent field (0: zero or subnormal, 0x7ff: infinity or NaN)
+__device__ __forceinline__ int expo(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ bool nonzero(double x) {
+  return (((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x)) != 0u;
+}
+
+// the two words of q
+__device__ __forceinline__ int2 words(long long q) {
+  const int lo = (int)((unsigned)q << 5) >> 5;  // the low 27 bits, signed
+  return make_int2((int)((q - (long long)lo) >> kLow), lo);
+}
+// x 2^(55 - E) for the block's largest exponent field ef (E = ef - 1022)
+__device__ __forceinline__ int2 split(double x, int ef) {
+  const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
+  const int e = (int)(hw >> 20) & 0x7ff;
+  const unsigned mh = (hw & 0xfffffu) | (e ? 0x100000u : 0u);
+  // mantissa left-justified below bit 63, subnormals shifted out
+  const unsigned long long m = ((unsigned long long)((mh << 10) | (lw >> 22)) << 32) | (lw << 10);
+  const unsigned long long mag = m >> (e ? min(63, ef - e + 8) : 63);
+  const long long sg = (long long)((int)hw >> 31);
+  return words((long long)(mag ^ (unsigned long long)sg) - sg);
+}
+
+// Three complex numbers (a site's column) as one block; returns its exponent.
+__device__ __forceinline__ int pack3(const double2 *v, int4 *o) {
+  int ef = 0;
+  bool any = false;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    ef = max(ef, max(expo(v[c].x), expo(v[c].y)));
+    any = any || nonzero(v[c].x) || nonzero(v[c].y);
+  }
+  if (ef == 0x7ff || (ef == 0 && any)) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) o[c] = *reinterpret_cast<const int4 *>(&v[c]);
+    return kSpecial;
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int2 re = split(v[c].x, ef), im = split(v[c].y, ef);
+    o[c] = make_int4(re.x, re.y, im.x, im.y);
+  }
+  return any ? ef - 1022 : kZero;
+}
+// The FP64 value of one complex of a block with exponent e.
+__device__ __forceinline__ double2 unpack(int4 q, int e) {
+  if (e == kSpecial) return *reinterpret_cast<const double2 *>(&q);
+  if (e == kZero) return make_double2(0.0, 0.0);
+  const long long re = ((long long)q.x << kLow) + q.y, im = ((long long)q.z << kLow) + q.w;
+  return make_double2(ldexp((double)re, e - kBits), ldexp((double)im, e - kBits));
+}
+
+// The words of q 2^-sh, 0 <= sh <= kAlign: the bits that leave the high word enter the low
+// one (lo then lies in [-2^26, 2^27 + 2^25)).
+constexpr int kAlign = 26;
+__device__ __forceinline__ void align(int &hi, int &lo, int sh) {
+  // the low sh bits of hi at the top of a word (nothing for sh = 0), then down to bits 26 ..
+  const unsigned out = __funnelshift_r(0u, (unsigned)hi, sh);
+  lo = (lo >> sh) + (int)(out >> 5);
+  hi >>= sh;
+}
+
+// A += h h, B += h l + l h
+__device__ __forceinline__ void mac2(long long &A, long long &B, int ah, int al, int bh, int bl) {
+  A += (long long)ah * bh;
+  B += (long long)ah * bl;
+  B += (long long)al * bh;
+}
+// (A + B 2^-27) for the sums of a product
+__device__ __forceinline__ long long join(long long A, long long B) { return A + (B >> kLow); }
+
+// r 2^k rounded to FP64
+__device__ __forceinline__ double value(long long r, int k) {
+  if (r == 0) return 0.0;
+  const double d = __ll2double_rn(r);
+  const int hw = __double2hiint(d);
+  const int e = ((hw >> 20) & 0x7ff) + k;
+  if ((unsigned)(e - 1) < 2045u) return __hiloint2double(hw + (k << 20), __double2loint(d));
+  return ldexp(d, max(-4000, min(4000, k)));
+}
+
+__device__ __forceinline__ long long shift(long long r, int right) {
+  return right > 0 ? r >> right : (long long)((unsigned long long)r << -right);
+}
+// Six reals r 2^k (three complex) as a block: brought to 55 bits by the leading bit of the
+// largest.
+__device__ __forceinline__ int renorm3(const long long *r, int k, int4 *o) {
+  unsigned long long m = 0;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) m |= (unsigned long long)(r[c] ^ (r[c] >> 63));
+  // |r| <= m + 1 <= 2^len
+  const int len = 64 - __clzll((long long)m);
+  const int sh = len - kBits;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int2 re = words(shift(r[2 * c], sh));
+    const int2 im = words(shift(r[2 * c + 1], sh));
+    o[c] = make_int4(re.x, re.y, im.x, im.y);
+  }
+  bool any = m != 0;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) any = any || r[c] != 0;  // (all -1 has m = 0)
+  return any ? k + len : kZero;
+}
+
+}  // namespace fx
+}  // namespace rhmc

@@ -44,16 +44,37 @@ rhmc_status_t hop(const Geom &g, int par, const C<T> *links, const C<T> *in, C<T
                   int n, int nbatch, long bstride, cudaStream_t s, const C<T> *links12 = nullptr, int bc_t = -1);
 rhmc_status_t stage_links12(const Geom &g, int bc_t, float2 *const l32[2], float2 *l12[2], bool *ok, cudaStream_t s);
 
-// double-float (FP64-accurate, FP32 units) operator pieces
-rhmc_status_t stage_links_df(const Geom &g, const double2 *l64, float4 *ldf, cudaStream_t s);
+// FP64-accurate operator on the integer units (fx.cuh): integer link records (int4 per
+// complex), the exponent of each site's largest entry, and the FP64 records
+struct FxLinks {
+  const int4 *rec = nullptr;
+  const int *exp = nullptr;
+  const double2 *l64 = nullptr;
+};
+// a field in integer form: int4 per complex [sites][3][n], exponent per (site, column)
+struct FxField {
+  int4 *v = nullptr;
+  int *e = nullptr;
+};
+rhmc_status_t stage_links_fx(const Geom &g, const double2 *l64, int4 *lfx, int *lexp, cudaStream_t s);
+// out = D in for an FP64 field, out in integer form (cat: profiler category); conv: an
+// FP64-sized buffer and exponents for the converted input
+rhmc_status_t hop_fx(const Geom &g, int par, const FxLinks &L, const double2 *in, FxField conv, FxField out, int n,
+                     int cat, cudaStream_t s);
+// the same with FP64 output, and as double-float pairs
+rhmc_status_t hop_fx_to64(const Geom &g, int par, const FxLinks &L, const double2 *in, FxField conv, double2 *out,
+                          int n, cudaStream_t s);
+rhmc_status_t hop_fx_to_df(const Geom &g, int par, const FxLinks &L, const double2 *in, FxField conv, float4 *out,
+                           int n, cudaStream_t s);
+// out = a self - D in for an input in integer form, FP64 output
+rhmc_status_t hop_fx_self(const Geom &g, int par, const FxLinks &L, FxField in, double2 *out, const double2 *self,
+                          double a, int n, cudaStream_t s);
+// R = B - (a X - D_eo tmp) (tmp = D_oe X), with the optional FP32 copy Rf and the nparts x n
+// column partials of |R|^2 (part; scratch: hop_fx_parts x n doubles)
+long hop_fx_parts(const Geom &g, int n);
+rhmc_status_t resid_fx(const Geom &g, const FxLinks &L, FxField tmp, const double2 *X, double a, const double2 *B,
+                       double2 *R, float2 *Rf, int n, double *scratch, double *part, int nparts, cudaStream_t s);
 rhmc_status_t df_split(const double2 *in, float4 *out, long len, cudaStream_t s);
-rhmc_status_t df_merge(float4 *io, long len, cudaStream_t s);
-// R = B - Y (Y in double-float, FP64 R), with the optional FP32 copy Rf and per-CTA
-// column sums of |R|^2 (partial: nparts x n; launched with nparts CTAs)
-rhmc_status_t resid_df(const double2 *B, const float4 *Y, double2 *R, float2 *Rf, long rows, int n,
-                       double *partial, int nparts, cudaStream_t s);
-rhmc_status_t hop_df(const Geom &g, int par, const float4 *links, const float4 *in, float4 *out, const float4 *self,
-                     double a, int n, cudaStream_t s);
 
 // blas.cu
 constexpr int kGramCtas = 4 * 152;  // CTAs of the Gram kernel (its scratch holds kGramCtas * n * n partials)
@@ -167,10 +188,13 @@ struct CtxTuneScope {
   ~CtxTuneScope();
 };
 
-// api.cu: read-only view of a context (device, geometry, mass, staged FP64
+// api.cu: read-only view of a context (device, geometry, mass, staged
 // links of the two output parities); NO_GAUGE before rhmc_set_gauge.
-rhmc_status_t ctx_geometry(const rhmc_ctx_t *ctx, int *device, Geom *g, double *mass, const double2 **l64_even,
-                           const double2 **l64_odd);
+rhmc_status_t ctx_geometry(const rhmc_ctx_t *ctx, int *device, Geom *g, double *mass, FxLinks *even, FxLinks *odd);
+
+// api.cu: Y = (A + sigma) X in FP64 with caller scratch (tmp: FP64 field, exps: 2 Vh n)
+rhmc_status_t apply_noalloc(const Geom &g, const FxLinks &even, const FxLinks &odd, double mass, const double2 *X,
+                            double2 *Y, double2 *tmp, int *exps, int n, double sigma, cudaStream_t s);
 
 // api.cu: device and geometry of a context (no gauge field needed), and its
 // scratch array of per-CTA partial sums (allocated on first use)

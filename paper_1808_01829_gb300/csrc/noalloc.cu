@@ -19,6 +19,8 @@ namespace rhmc {
 // e.g. a 16^4 lattice with 16 right-hand sides (25.2 MB).
 constexpr size_t kNoAllocScratchBytes = 32u << 20;
 static __device__ __align__(256) double2 g_noalloc_scratch[kNoAllocScratchBytes / sizeof(double2)];
+// exponents of the converted input and of the intermediate: one per three complex values each
+static __device__ __align__(256) int g_noalloc_exp[2 * (kNoAllocScratchBytes / (3 * sizeof(double2)))];
 
 namespace {
 constexpr int kMaxDevices = 64;
@@ -28,6 +30,7 @@ std::mutex g_mu;
 // as that context lives, so a process that resets a device (cudaDeviceReset)
 // must not call this entry point on that device afterwards.
 double2 *g_scratch_ptr[kMaxDevices] = {};
+int *g_scratch_exp[kMaxDevices] = {};
 }  // namespace
 
 }  // namespace rhmc
@@ -46,7 +49,7 @@ extern "C" rhmc_status_t rhmc_apply_mdagm_mrhs_noalloc(rhmc_ctx_t *ctx, const vo
   int device = 0;
   Geom g;
   double mass = 0.0;
-  const double2 *le = nullptr, *lo = nullptr;
+  FxLinks le, lo;
   rhmc_status_t rc = ctx_geometry(ctx, &device, &g, &mass, &le, &lo);
   if (rc != RHMC_OK) return rc;
   const size_t need = (size_t)g.Vh * 3 * n_rhs * sizeof(double2);
@@ -68,24 +71,25 @@ extern "C" rhmc_status_t rhmc_apply_mdagm_mrhs_noalloc(rhmc_ctx_t *ctx, const vo
     std::lock_guard<std::mutex> lock(g_mu);
     if (!g_scratch_ptr[device]) {
       // once per device, with that device current: the symbol's device address
-      void *p = nullptr;
-      const cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-      if (e != cudaSuccess || !p) {
+      void *p = nullptr, *q = nullptr;
+      cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
+      if (e == cudaSuccess) e = cudaGetSymbolAddress(&q, g_noalloc_exp);
+      if (e != cudaSuccess || !p || !q) {
         set_error("rhmc_apply_mdagm_mrhs_noalloc: cudaGetSymbolAddress: %s", cudaGetErrorString(e));
         if (prev >= 0 && prev != device) cudaSetDevice(prev);
         return RHMC_ERR_CUDA;
       }
       g_scratch_ptr[device] = static_cast<double2 *>(p);
+      g_scratch_exp[device] = static_cast<int *>(q);
     }
     scratch = g_scratch_ptr[device];
   }
   cudaStream_t s = (cudaStream_t)sv;
   CtxTuneScope tscope(ctx);  // the context's launch settings, as in rhmc_apply_mdagm_mrhs
-  // the intermediate is fully overwritten by the first hop: nothing to clear
-  rc = hop<double>(g, 1, lo, (const double2 *)X_dev, scratch, nullptr, 0.0, n_rhs, 1, 0, s);
-  if (rc == RHMC_OK)
-    rc = hop<double>(g, 0, le, scratch, (double2 *)Y_dev, (const double2 *)X_dev, 4.0 * mass * mass + sigma, n_rhs, 1,
-                     0, s);
+  // the intermediate is fully overwritten by the first hop: nothing to clear.  Y holds the
+  // converted input until the second hop writes it.
+  rc = apply_noalloc(g, le, lo, mass, (const double2 *)X_dev, (double2 *)Y_dev, scratch,
+                     g_scratch_exp[device], n_rhs, sigma, s);
   if (prev >= 0 && prev != device) cudaSetDevice(prev);
   return rc;
 }

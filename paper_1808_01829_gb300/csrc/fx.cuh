@@ -55,6 +55,17 @@ __device__ __forceinline__ int2 split(double x, int ef) {
   return words((long long)(mag ^ (unsigned long long)sg) - sg);
 }
 
+// x 2^54 rounded, for |x| < 2
+__device__ __forceinline__ long long fixed54(double x) {
+  const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
+  const int e = (int)(hw >> 20) & 0x7ff;
+  const unsigned long long m = ((unsigned long long)((hw & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lw;
+  const int s = 1023 + 52 - 54 - e;  // x = m 2^(e - 1075), 2^54 x = m 2^(e - 1021)
+  const unsigned long long mag = s <= 0 ? m << -s : ((m >> min(63, s - 1)) + 1) >> 1;
+  const long long sg = (long long)((int)hw >> 31);
+  return (long long)(mag ^ (unsigned long long)sg) - sg;
+}
+
 // Three complex numbers (a site's column) as one block; returns its exponent.
 __device__ __forceinline__ int pack3(const double2 *v, int4 *o) {
   int ef = 0;
@@ -113,8 +124,9 @@ __device__ __forceinline__ double value(long long r, int k) {
   return ldexp(d, max(-4000, min(4000, k)));
 }
 
+// r 2^-right, rounded
 __device__ __forceinline__ long long shift(long long r, int right) {
-  return right > 0 ? r >> right : (long long)((unsigned long long)r << -right);
+  return right > 0 ? (r + (1ll << (right - 1))) >> right : (long long)((unsigned long long)r << -right);
 }
 // Six reals r 2^k (three complex) as a block: brought to 55 bits by the leading bit of the
 // largest.

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fx.cuh"
 #include "kernels.h"
 
 namespace rhmc {
@@ -227,11 +228,8 @@ __global__ void __launch_bounds__(256) k_momenta(const double *__restrict__ p, d
 }
 
 // P_mu(x) += coef TA(U_mu(x) V_mu(x)); the kick P += eps TA(U G_g^dagger)/2 with
-// G_g = -(beta/3) V^dagger has coef = -eps beta / 6
-__global__ void __launch_bounds__(128) k_gauge_momentum(Geom g, const double2 *__restrict__ U, double2 *__restrict__ P,
-                                                        double coef) {
-  const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= 4 * g.V) return;
+// G_g = -(beta/3) V^dagger has coef = -eps beta / 6.  FP64 form, one link e.
+__device__ __noinline__ void kick_fp64(const Geom &g, const double2 *U, double2 *P, double coef, long e) {
   const long site = e >> 2;
   const int mu = (int)(e & 3);
   int x[4], xp[4];
@@ -252,6 +250,183 @@ __global__ void __launch_bounds__(128) k_gauge_momentum(Geom g, const double2 *_
   add_ta(P + e * 9, mul(ld3(U + e * 9), V), coef);
 }
 
+__global__ void __launch_bounds__(128) k_gauge_momentum(Geom g, const double2 *__restrict__ U, double2 *__restrict__ P,
+                                                        double coef) {
+  const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < 4 * g.V) kick_fp64(g, U, P, coef, e);
+}
+
+// ------------------------------------------------------------ the kick on the integer units
+// The 13 products of 3 x 3 matrices of a link's kick (1404 FP64 FMAs, 64 clocks each for a
+// warp) as exact integer sums (fx.cuh): 243 multiply-adds of four clocks per product.  The
+// entries of SU(3) links, their products and the sum of six staples have known sizes, so
+// everything is held in units of 2^-54 (two words, hi 2^27 + lo) and a product needs no
+// shift: 2^-54 2^-54 (h1 h2 2^54 + (h1 l2 + l1 h2) 2^27 + l1 l2), the last term dropped.
+// Links whose largest entry is not in [1/2, 2), products above 2 and staple sums above 8
+// (never for SU(3)) send the link's kick to the FP64 form.
+// The links are converted once, to v[(mu * 9 + entry) * V + site], so that the warps of the
+// kick, 32 consecutive sites of one direction each, read whole lines; ok[mu * V + site] says
+// whether the link fits.
+__global__ void __launch_bounds__(128) k_links_to_fx(const double2 *__restrict__ U, int4 *__restrict__ v,
+                                                     int *__restrict__ ok, long V) {
+  const int mu = threadIdx.x >> 5;
+  const long site = (long)blockIdx.x * 32 + (threadIdx.x & 31);
+  if (site >= V) return;
+  const M3 u = ld3(U + (site * 4 + mu) * 9);
+  int ef = 0;
+#pragma unroll
+  for (int c = 0; c < 9; ++c) ef = max(ef, max(fx::expo(u.e[c].x), fx::expo(u.e[c].y)));
+  const bool fits = ef == 1022 || ef == 1023;
+#pragma unroll
+  for (int c = 0; c < 9; ++c) {
+    const int2 re = fx::words(fits ? fx::fixed54(u.e[c].x) : 0), im = fx::words(fits ? fx::fixed54(u.e[c].y) : 0);
+    v[(mu * 9 + c) * V + site] = make_int4(re.x, re.y, im.x, im.y);
+  }
+  ok[mu * V + site] = fits;
+}
+
+namespace {
+// three sums r_j = sum_k a_k b[k][j] in units of 2^-54, rounded (reals: re, im)
+__device__ __forceinline__ void row_times(const int4 *a, const int4 *b, long long *r) {
+  constexpr long long half = 1ll << (fx::kLow - 1);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    long long pA = 0, pB = half, mA = 0, mB = 0, iA = 0, iB = 2 * half;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int4 x = a[k], y = b[k * 3 + j];
+      fx::mac2(pA, pB, x.x, x.y, y.x, y.y);
+      fx::mac2(mA, mB, x.z, x.w, y.z, y.w);
+      fx::mac2(iA, iB, x.x + x.z, x.y + x.w, y.x + y.z, y.y + y.w);
+    }
+    r[2 * j] = fx::join(pA - mA, pB - mB);
+    r[2 * j + 1] = fx::join(iA - pA - mA, iB - pB - mB);
+  }
+}
+__device__ __forceinline__ int4 conj_if(int4 z, int m) {  // m = -1: the conjugate, 0: z
+  return make_int4(z.x, z.y, (z.z ^ m) - m, (z.w ^ m) - m);
+}
+// |r| < 2^bits
+__device__ __forceinline__ bool below(long long r, int bits) {
+  return (int)(r >> bits) == 0 || (int)(r >> bits) == -1;
+}
+}  // namespace
+
+// The kick of k_gauge_momentum with integer products.  A staple is op(X) Y^dagger op'(Z)
+// (forward: X, Z^dagger; backward: X^dagger, Z), formed row by row; the six are added as
+// integers and only the traceless anti-Hermitian part of U V is converted to FP64.
+// The loops over staples and rows are not unrolled, and the sum lives in shared memory:
+// unrolled, the warps waited for instructions.  Bound by the integer multiplier, 13 x 243
+// multiply-adds of four clocks per link (175 us at 16^3 x 32), and by the adds and shifts around
+// them at two warps per scheduler.  Measured at 16^3 x 32: 518 us, and 27 us for the conversion,
+// 1791 us in FP64; error of P after a kick of eps = 0.5 7.6e-17 (FP64 form 1.0e-16).
+__global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4 *__restrict__ v,
+                                                              const int *__restrict__ ok,
+                                                              const double2 *__restrict__ U, double2 *__restrict__ P,
+                                                              double coef) {
+  __shared__ long long sV[18][128];  // the staple sum V of this thread
+  const int mu = threadIdx.x >> 5, tid = threadIdx.x;
+  const int nsite = (int)g.V, site = blockIdx.x * 32 + (threadIdx.x & 31);
+  if (site >= nsite) return;
+#pragma unroll
+  for (int c = 0; c < 18; ++c) sV[c][tid] = 0;
+  int x[4], xp[4];
+  {
+    int r = site;
+    x[0] = r % g.L[0];
+    r /= g.L[0];
+    x[1] = r % g.L[1];
+    r /= g.L[1];
+    x[2] = r % g.L[2];
+    x[3] = r / g.L[2];
+  }
+  step(g, x, mu, 1, xp);
+  const int sp = (int)lex_of(g, xp);
+  bool fits = ok[mu * nsite + site];
+#pragma unroll 1
+  for (int q = 0; q < 6; ++q) {
+    const int nu = (q >> 1) < mu ? (q >> 1) : (q >> 1) + 1;
+    const bool fwd = (q & 1) == 0;
+    int xn[4], xq[4];
+    step(g, x, nu, fwd ? 1 : -1, xn);
+    step(g, xn, mu, 1, xq);
+    const int sn = (int)lex_of(g, xn);
+    const int sx = fwd ? sp : (int)lex_of(g, xq), sz = fwd ? site : sn;
+    fits = fits && ok[nu * nsite + sx] && ok[mu * nsite + sn] && ok[nu * nsite + sz];
+    const int4 *px = v + (long)nu * 9 * nsite + sx, *py = v + (long)mu * 9 * nsite + sn,
+               *pz = v + (long)nu * 9 * nsite + sz;
+    const int cz = fwd ? -1 : 0;
+    const int rs = fwd ? 3 : 1, cs = fwd ? 1 : 3;  // strides of op(X)'s rows and columns
+    int4 y[9], z[9];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        y[k * 3 + j] = conj_if(__ldg(py + (j * 3 + k) * nsite), -1);
+        z[k * 3 + j] = conj_if(__ldg(pz + (j * rs + k * cs) * nsite), cz);
+      }
+#pragma unroll 1
+    for (int i = 0; i < 3; ++i) {
+      int4 a[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) a[k] = conj_if(__ldg(px + (i * rs + k * cs) * nsite), ~cz);
+      long long r[6];
+      row_times(a, y, r);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        fits = fits && below(r[2 * k], 55) && below(r[2 * k + 1], 55);
+        const int2 re = fx::words(r[2 * k]), im = fx::words(r[2 * k + 1]);
+        a[k] = make_int4(re.x, re.y, im.x, im.y);
+      }
+      row_times(a, z, r);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) sV[i * 6 + c][tid] += r[c];
+    }
+  }
+  int4 b[9];
+#pragma unroll
+  for (int c = 0; c < 9; ++c) {
+    const long long re = sV[2 * c][tid], im = sV[2 * c + 1][tid];
+    fits = fits && below(re, 57) && below(im, 57);
+    const int2 wr = fx::words(re), wi = fx::words(im);
+    b[c] = make_int4(wr.x, wr.y, wi.x, wi.y);
+  }
+  if (!fits) {
+    kick_fp64(g, U, P, coef, (long)site * 4 + mu);
+    return;
+  }
+  long long w[18];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    int4 a[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) a[c] = __ldg(v + (long)(mu * 9 + i * 3 + c) * nsite + site);
+    row_times(a, b, w + 6 * i);
+  }
+  // TA(w) = (w - w^dagger)/2 - tr(w - w^dagger)/6; its upper triangle, twice as large
+  double2 *p = P + ((long)site * 4 + mu) * 9;
+  const long long tr = (w[1] + w[9] + w[17]) / 3;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double d = fx::value(w[2 * (i * 4) + 1] - tr, -53);
+    double2 z = p[i * 4];
+    z.y = fma(0.5 * coef, d, z.y);
+    p[i * 4] = z;
+#pragma unroll
+    for (int j = i + 1; j < 3; ++j) {
+      const int a = 2 * (i * 3 + j), c = 2 * (j * 3 + i);
+      const double re = fx::value(w[a] - w[c], -54), im = fx::value(w[a + 1] + w[c + 1], -54);
+      double2 z1 = p[i * 3 + j], z2 = p[j * 3 + i];
+      z1.x = fma(0.5 * coef, re, z1.x);
+      z1.y = fma(0.5 * coef, im, z1.y);
+      z2.x = fma(-0.5 * coef, re, z2.x);
+      z2.y = fma(0.5 * coef, im, z2.y);
+      p[i * 3 + j] = z1;
+      p[j * 3 + i] = z2;
+    }
+  }
+}
+
 // P += coef TA(U G^dagger)
 __global__ void __launch_bounds__(128) k_momentum_update(const double2 *__restrict__ U, const double2 *__restrict__ G,
                                                          double2 *__restrict__ P, long nlinks, double coef) {
@@ -260,52 +435,94 @@ __global__ void __launch_bounds__(128) k_momentum_update(const double2 *__restri
   add_ta(P + l * 9, mul_nd(ld3(U + l * 9), ld3(G + l * 9)), coef);
 }
 
-// U <- exp(eps P) U.  exp(Y) for |Y|_F <= 1/2 by the Taylor polynomial of degree
-// kTaylor in Horner form, E = I + Y (I + Y/2 (I + ... (I + Y/kTaylor))), whose
-// remainder is below |Y|^(kTaylor+1) / (kTaylor+1)! e^|Y| < 4e-20; larger
-// arguments are scaled by 2^-k first and the result squared k times.
+// U <- exp(Y) U, Y = eps P.  exp(Y) for |Y|_F <= 1/2 by its Taylor polynomial; larger
+// arguments are scaled by 2^-k first and the result squared k times.  With the
+// Cayley-Hamilton identity P^3 = t P^2 - s P + d (t = tr P, s = (t^2 - tr P^2) / 2, d = det P)
+// the polynomial is f_0 + f_1 Y + f_2 Y^2, and its Horner steps act on three complex numbers:
+//   (f_0, f_1, f_2) <- (1 + d f_2 / k, (f_0 - s f_2) / k, (f_1 + t f_2) / k)
+// (t, s, d scaled by eps, eps^2, eps^3): 18 FP64 operations instead of the 126 of a matrix
+// product, for any P.  exp(Y) - 1 = D is carried instead of exp(Y), so that U + D U rounds at
+// the size of D.  The degree is the smallest whose remainder |Y|^(m+1) / (m+1)! e^|Y| is below
+// 4e-20, the bound of degree 16 at |Y| = 1/2.  Bound by the FP64 pipe, about 500 operations per
+// link.  Measured at 16^3 x 32: 508 us, 1922 us with matrix products at degree 16; against a
+// 113-bit sum the error of U is 4e-17 at eps = 0.05 (7.7e-17 with matrix products).
+__constant__ double kRecip[kTaylor + 1] = {0.0,      1.0,      1.0 / 2,  1.0 / 3,  1.0 / 4,  1.0 / 5,
+                                           1.0 / 6,  1.0 / 7,  1.0 / 8,  1.0 / 9,  1.0 / 10, 1.0 / 11,
+                                           1.0 / 12, 1.0 / 13, 1.0 / 14, 1.0 / 15, 1.0 / 16};
+__device__ __forceinline__ double2 zmul(double2 a, double2 b) {
+  return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ double2 zscale(double2 a, double r) { return make_double2(a.x * r, a.y * r); }
 __global__ void __launch_bounds__(128) k_link_update(double2 *__restrict__ U, const double2 *__restrict__ P, long nlinks,
                                                      double eps) {
   const long l = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= nlinks) return;
-  M3 Y = ld3(P + l * 9);
+  const M3 p = ld3(P + l * 9);
   double n2 = 0.0;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    Y.e[k].x *= eps;
-    Y.e[k].y *= eps;
-    n2 = fma(Y.e[k].x, Y.e[k].x, fma(Y.e[k].y, Y.e[k].y, n2));
-  }
+  for (int k = 0; k < 9; ++k) n2 = fma(p.e[k].x, p.e[k].x, fma(p.e[k].y, p.e[k].y, n2));
+  n2 *= eps * eps;
   int sq = 0;
-  double sc = 1.0;
-  while (n2 * sc * sc > 0.25 && sq < 64) {  // bounded: a non-finite norm stops at 64
+  double sc = eps;
+  while (n2 > 0.25 && sq < 64) {  // bounded: a non-finite norm stops at 64
+    n2 *= 0.25;
     sc *= 0.5;
     ++sq;
   }
-#pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    Y.e[k].x *= sc;
-    Y.e[k].y *= sc;
-  }
-  M3 E = zero3();
-  E.e[0].x = E.e[4].x = E.e[8].x = 1.0;
-#pragma unroll
-  for (int k = kTaylor; k >= 1; --k) {
-    E = mul(Y, E);
-    const double r = 1.0 / k;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      E.e[q].x *= r;
-      E.e[q].y *= r;
+  int deg = 0;
+  {
+    // from an upper bound of |Y| (NaN takes the full degree)
+    const float ny = sqrtf((float)n2) * 1.0001f;
+    float r = ny * __expf(ny) * 1.01f;  // remainder of degree 0
+    while (deg < kTaylor && !(r < 4e-20f)) {
+      ++deg;
+      r *= ny / (float)(deg + 1);
     }
-    E.e[0].x += 1.0;
-    E.e[4].x += 1.0;
-    E.e[8].x += 1.0;
+    deg = max(2, deg);
   }
-  for (int i = 0; i < sq; ++i) E = mul(E, E);
-  const M3 u = mul(E, ld3(U + l * 9));
+  const M3 p2 = mul(p, p);
+  const double sc2 = sc * sc;
+  double2 tr = make_double2(p.e[0].x + p.e[4].x + p.e[8].x, p.e[0].y + p.e[4].y + p.e[8].y);
+  const double2 q2 = make_double2(p2.e[0].x + p2.e[4].x + p2.e[8].x, p2.e[0].y + p2.e[4].y + p2.e[8].y);
+  const double2 t2 = zmul(tr, tr);
+  const double2 s = make_double2(0.5 * sc2 * (t2.x - q2.x), 0.5 * sc2 * (t2.y - q2.y));
+  // det P along the first row
+  auto minor = [&](int a, int b, int c, int d) {
+    const double2 u = zmul(p.e[a], p.e[d]), w = zmul(p.e[b], p.e[c]);
+    return make_double2(u.x - w.x, u.y - w.y);
+  };
+  const double2 m0 = zmul(p.e[0], minor(4, 5, 7, 8)), m1 = zmul(p.e[1], minor(3, 5, 6, 8)),
+                m2 = zmul(p.e[2], minor(3, 4, 6, 7));
+  const double2 d = zscale(make_double2(m0.x - m1.x + m2.x, m0.y - m1.y + m2.y), sc * sc2);
+  tr = zscale(tr, sc);
+  double2 f0 = make_double2(0.0, 0.0), f1 = f0, f2 = f0;  // f0: less one
+  for (int k = deg; k >= 1; --k) {
+    const double r = kRecip[k];
+    const double2 g2 = zscale(f2, r);
+    const double2 h0 = zmul(d, g2), h1 = zmul(s, g2), h2 = zmul(tr, g2);
+    f2 = make_double2(fma(f1.x, r, h2.x), fma(f1.y, r, h2.y));
+    f1 = make_double2(fma(f0.x, r, r - h1.x), fma(f0.y, r, -h1.y));
+    f0 = h0;
+  }
+  f1 = zscale(f1, sc);
+  f2 = zscale(f2, sc2);
+  M3 D;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) U[l * 9 + k] = u.e[k];
+  for (int q = 0; q < 9; ++q) {
+    double2 a = q % 4 == 0 ? f0 : make_double2(0.0, 0.0);
+    cmac<double>(a, f2, p2.e[q]);
+    cmac<double>(a, f1, p.e[q]);
+    D.e[q] = a;
+  }
+  for (int i = 0; i < sq; ++i) {  // (1 + D)^2 - 1 = 2 D + D^2
+    const M3 D2 = mul(D, D);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) D.e[q] = make_double2(fma(2.0, D.e[q].x, D2.e[q].x), fma(2.0, D.e[q].y, D2.e[q].y));
+  }
+  const M3 u = ld3(U + l * 9);
+  const M3 w = mul(D, u);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) U[l * 9 + k] = make_double2(u.e[k].x + w.e[k].x, u.e[k].y + w.e[k].y);
 }
 
 // ------------------------------------------------------------ launch wrappers
@@ -363,13 +580,31 @@ rhmc_status_t momenta_from_normals(const Geom &g, const double *p, double2 *P, c
   return RHMC_OK;
 }
 
-rhmc_status_t gauge_momentum(const Geom &g, const double2 *U, double2 *P, double beta, double eps, cudaStream_t s) {
+rhmc_status_t gauge_momentum(rhmc_ctx_t *c, const Geom &g, const double2 *U, double2 *P, double beta, double eps, cudaStream_t s) {
   const long nl = g.V * 4;
+  const unsigned grid = (unsigned)((g.V + 31) / 32);  // 128 threads: four directions of 32 sites
+  // The integer form needs the links in integer form, in a buffer of the context.  A stream
+  // that is being captured takes the FP64 kernel: its graph may run at any later time,
+  // next to other users of the buffer.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  RHMC_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+  int4 *v = nullptr;
+  int *ex = nullptr;
+  if (cap == cudaStreamCaptureStatusNone) {
+    RHMC_TRY(ctx_links_fx_begin(c, &v, &ex, s));
+    prof_begin(PROF_OTHER, s);
+    k_links_to_fx<<<grid, 128, 0, s>>>(U, v, ex, g.V);
+    prof_end(s, (double)nl * 2 * kLinkBytes);
+    RHMC_LAUNCH_CHECK();
+  }
   prof_begin(PROF_OTHER, s);
-  k_gauge_momentum<<<(unsigned)((nl + 127) / 128), 128, 0, s>>>(g, U, P, -eps * beta / 6.0);
+  if (v)
+    k_gauge_momentum_fx<<<grid, 128, 0, s>>>(g, v, ex, U, P, -eps * beta / 6.0);
+  else
+    k_gauge_momentum<<<(unsigned)((nl + 127) / 128), 128, 0, s>>>(g, U, P, -eps * beta / 6.0);
   prof_end(s, (double)nl * 3 * kLinkBytes);
   RHMC_LAUNCH_CHECK();
-  return RHMC_OK;
+  return v ? ctx_links_fx_end(c, s) : RHMC_OK;
 }
 
 rhmc_status_t momentum_update(const Geom &g, const double2 *U, const double2 *G, double2 *P, double eps,
@@ -419,7 +654,7 @@ struct Md {
   }
   rhmc_status_t gauge_kick(double eps) {
     info->gauge_force_evals += 1;
-    return gauge_momentum(g, U, P, p->beta, eps, s);
+    return gauge_momentum(c, g, U, P, p->beta, eps, s);
   }
   // D(h): n_gauge OMF2 steps of the gauge force, the kicks at the same links merged
   rhmc_status_t drift(double h) {
@@ -532,7 +767,7 @@ rhmc_status_t rhmc_gauge_momentum(rhmc_ctx_t *c, const void *U, void *P, double 
     set_error("rhmc_gauge_momentum: null U or P");
     return RHMC_ERR_INVALID_ARG;
   }
-  return gauge_momentum(L.g, (const double2 *)U, (double2 *)P, beta, eps, (cudaStream_t)sv);
+  return gauge_momentum(c, L.g, (const double2 *)U, (double2 *)P, beta, eps, (cudaStream_t)sv);
 }
 
 rhmc_status_t rhmc_momentum_update(rhmc_ctx_t *c, const void *U, const void *G, void *P, double eps,

@@ -120,6 +120,12 @@ constexpr int kRefineLanes = 4;       // concurrent defect corrections (built-in
 // host checks of a defect-correction solve (divides kCheckEvery); measured at 24^4 with the
 // 0.9 margin: every 1, 2, 3 iterations took 223, 230, 240 correction iterations (95, 97, 100 ms)
 constexpr int kCorrectionCheckEvery = 1;
+// Fields shorter than this (complex numbers) let their corrections stop on the device, with a
+// host check every kCheckEvery iterations; the bulk kernels of longer ones hide the host's
+// checks, and would pay for the iterations that a chunk runs past the stop.  Measured (tolerance
+// 1e-11): 12^4, n = 4 28.5 -> 26.7 ms with its action, 8^4 trajectory 181 -> 155 ms; 16^4,
+// n = 8 and longer 1-2 % slower with device stops.
+constexpr long kDeviceStopLen = 1 << 19;
 // A defect correction stops when its recursive residual is kCorrectionMargin x tol / r of the
 // residual r it started from.  Its own FP32 drift is about 1e-6 of r (1e-3 of its target),
 // so the true residual after it lands within that margin of tol; a second round
@@ -310,14 +316,14 @@ rhmc_status_t apply_noalloc(const Geom &g, const FxLinks &even, const FxLinks &o
 
 template <typename T>
 static rhmc_status_t apply_A(const rhmc_ctx *c, const C<T> *X, C<T> *Y, C<T> *tmp, FxExp ex, int n, double sigma,
-                             cudaStream_t s) {
+                             cudaStream_t s, const SolverState *st = nullptr) {
   if constexpr (sizeof(T) == 8) {
     return apply_A64(c->g, fx_links(c, 0), fx_links(c, 1), c->mass, X, Y, tmp, ex, n, sigma, s);
   } else {
     RHMC_TRY(hop<T>(c->g, 1, LinksOf<T>::get(c, 1), X, tmp, nullptr, 0.0, n, 1, 0, s, Links12Of<T>::get(c, 1),
-                    c->bc_t));
+                    c->bc_t, st));
     return hop<T>(c->g, 0, LinksOf<T>::get(c, 0), tmp, Y, X, 4.0 * c->mass * c->mass + sigma, n, 1, 0, s,
-                  Links12Of<T>::get(c, 0), c->bc_t);
+                  Links12Of<T>::get(c, 0), c->bc_t, st);
   }
 }
 
@@ -356,6 +362,7 @@ struct SolveBufs {
   double *nscr;       // per-CTA column sums of the residual kernel
   FxExp ex;           // exponents of the integer fields of an FP64-accurate operator application
   SolverState *st;
+  bool device_stop = false;  // (mixed, single shift) the solve stops on the device
   int accumulate = 0;  // shifts s >= 1 add w_s X^(s) into one field after X^(0) (FP64)
   // stored-basis mode (mixed, several shifts): the block basis Q_0 .. Q_{cap-1}
   // (rows x cap*n, row-major), the per-iteration shift coefficients and the
@@ -501,6 +508,8 @@ struct StateView {
   int active[kMaxS];
   int breakdown;
   int device_timeout;
+  int done;
+  int nit;
 };
 
 static rhmc_status_t read_state(rhmc_ctx *c, SolverState *st, StateView &v, cudaStream_t s) {
@@ -508,7 +517,7 @@ static rhmc_status_t read_state(rhmc_ctx *c, SolverState *st, StateView &v, cuda
   StateView *h = reinterpret_cast<StateView *>(lane(c).h_pin);
   RHMC_CUDA_TRY(cudaMemcpyAsync(h->res, st->res, sizeof(v.res), cudaMemcpyDeviceToHost, s));
   RHMC_CUDA_TRY(cudaMemcpyAsync(h->active, st->active, sizeof(v.active), cudaMemcpyDeviceToHost, s));
-  RHMC_CUDA_TRY(cudaMemcpyAsync(&h->breakdown, &st->breakdown, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  RHMC_CUDA_TRY(cudaMemcpyAsync(&h->breakdown, &st->breakdown, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
   RHMC_CUDA_TRY(cudaStreamSynchronize(s));
   std::memcpy(&v, h, sizeof(StateView));
   return RHMC_OK;
@@ -552,14 +561,17 @@ static rhmc_status_t sbcgrq_iteration(rhmc_ctx *c, const SolveBufs &b, TX *Xacc,
   cudaStream_t ss = split ? c->side : s;
   // (chunk boundaries are joined on the host, so only waits inside a chunk are needed)
   if (split && k - 2 > chunk_start) RHMC_CUDA_TRY(cudaStreamWaitEvent(s, c->ev_side[(k - 2) % 3], 0));
-  RHMC_TRY(apply_A<T>(c, P, AP, Todd, b.ex, n, sigma0, s));
-  RHMC_TRY(gram<T>(P, AP, rows, n, b.gscratch, b.partial, s));
+  // (device stop: 4 m^2 + sigma_0 comes from the state, and a solve that has stopped skips the
+  // rest of its chunk)
+  const int *done = b.device_stop ? &b.st->done : nullptr;
+  RHMC_TRY(apply_A<T>(c, P, AP, Todd, b.ex, n, sigma0, s, b.device_stop ? b.st : nullptr));
+  RHMC_TRY(gram<T>(P, AP, rows, n, b.gscratch, b.partial, s, done));
   RHMC_TRY(nxn_alpha<T>(b.partial, kGramParts, n, b.st, k, (C<T> *)b.mw, s));
   const bool cols = use_column_update<T>();
   if (cols) {
     // W = Q - (AP) alpha and its Gram W^dagger W in one pass
     RHMC_TRY(axpy_gram_cols((const float2 *)AP, (const float2 *)Qprev, (const float2 *)b.mw, (float2 *)W, rows, n,
-                            b.gscratch, b.partial, s));
+                            b.gscratch, b.partial, s, done));
   } else {
     RHMC_TRY(block_axpy<T, T>(AP, Qprev, (const C<T> *)b.mw, W, rows, n, s));
     RHMC_TRY(gram<T>(W, W, rows, n, b.gscratch, b.partial, s));
@@ -570,7 +582,8 @@ static rhmc_status_t sbcgrq_iteration(rhmc_ctx *c, const SolveBufs &b, TX *Xacc,
     // one pass: Q_k = W rho^-1, X^(0), P^(0), and block k of the stored basis (k from the
     // device counter: graph replays)
     RHMC_TRY(base_step((const float2 *)W, (float2 *)Qcur, (float2 *)P, (float2 *)Xacc, (const float2 *)b.coef,
-                       b.basis, b.cap, b.basis ? &b.st->kabs[k % kSlots] : nullptr, rows, n, s));
+                       b.basis, b.cap, b.basis ? &b.st->kabs[k % kSlots] : nullptr,
+                       b.device_stop ? &b.st->upd[0] : nullptr, rows, n, s));
   } else if (cols) {
     RHMC_TRY(axpy_cols((const float2 *)W, nullptr, (const float2 *)b.coef, (float2 *)Qcur, rows, n, s));
     if (b.basis)  // block k of the stored basis (k from the device counter: graph replays)
@@ -635,10 +648,14 @@ template <typename T>
 static rhmc_status_t run_chunk_graph(rhmc_ctx *c, const SolveBufs &b, double2 *X, int n, int ns, double sigma0,
                                      int chunk_start, int len, double target, int freeze, cudaStream_t s) {
   // (b.basis: chunks with and without the stored basis record different kernels)
-  std::vector<double> key = {(double)(uintptr_t)b.P, (double)(uintptr_t)X, (double)(uintptr_t)b.basis,
+  // (mixed: the chunk does not touch X; with device stop it reads sigma_0 and the tolerance
+  // from the state, so that one graph serves the corrections of every shift)
+  const bool mixed = sizeof(T) == 4;
+  std::vector<double> key = {(double)(uintptr_t)b.P, mixed ? 0.0 : (double)(uintptr_t)X, (double)(uintptr_t)b.basis,
                              (double)b.accumulate, (double)n,
-                             (double)ns, sigma0, target, (double)freeze, (double)sizeof(T), (double)len,
-                             (double)(chunk_start % kCheckEvery)};
+                             (double)ns, b.device_stop ? 0.0 : sigma0, b.device_stop ? 0.0 : target, (double)freeze,
+                             (double)sizeof(T), (double)len, (double)(chunk_start % kCheckEvery),
+                             (double)b.device_stop};
   for (int t = 0; t < TUNE_NKEYS; ++t) key.push_back((double)tune_get(t));
   SolverLane &L = lane(c);
   SolverLane::GraphEntry *hit = nullptr;
@@ -748,6 +765,18 @@ static rhmc_status_t solve_phase1(rhmc_ctx *c, const double2 *B, int n, int ns, 
   // stay zero (their solutions come from the assembly), so only the base system's
   auto nflush = [&]() { return b.basis ? 1 : ns; };
   RHMC_CUDA_TRY(cudaMemcpyAsync(b.st->sigma, shifts, sizeof(double) * ns, cudaMemcpyHostToDevice, s));
+  // A defect correction stops on the device, in the iteration that reaches its tolerance, so
+  // the host looks once per chunk of kCheckEvery iterations (with the kernels that know how
+  // to stop; a host check cadence can be asked for instead)
+  const int hm = tune_get(TUNE_HOP_STAGED);
+  const bool device_stop = mixed && ns == 1 && len < kDeviceStopLen && (hm == 0 || hm == 3 || hm == 4) &&
+                           !prm.reliable && !prm.verify_at_convergence &&
+                           tune_get(TUNE_CORRECTION_CHECK_EVERY) == 0 && tune_get(TUNE_NXN_FP64) != 1 &&
+                           tune_get(TUNE_AXPY_SCALAR) != 1 && tune_get(TUNE_UPDATE_TENSOR) != 2 &&
+                           tune_get(TUNE_FLUSH_EVERY) == 0;
+  b.device_stop = device_stop;
+  const double ctl[2] = {device_stop ? prm.tol : 0.0, 4.0 * c->mass * c->mass + sigma0};
+  RHMC_CUDA_TRY(cudaMemcpyAsync(&b.st->stop_tol, ctl, sizeof(ctl), cudaMemcpyHostToDevice, s));
   // accumulating solve: X^(0) and one field for sum_{s>=1} w_s X^(s)
   RHMC_CUDA_TRY(cudaMemsetAsync(X, 0, sizeof(double2) * len * (b.accumulate ? std::min(ns, 2) : ns), s));
   // initialisation: {Q_0, delta_0} = qr(B) (FP64 Gram), P^(s) = Q_0
@@ -783,7 +812,8 @@ static rhmc_status_t solve_phase1(rhmc_ctx *c, const double2 *B, int n, int ns, 
   const int fz = tune_get(TUNE_SHIFT_FREEZE_NANO);
   const double tol_shift = mixed ? std::max(target, fz > 0 ? 1e-9 * fz : kShiftFreezeMixed) : target;
   double res_at_reliable = 1.0;
-  const int check_every = prm.check_every > 0                ? prm.check_every
+  const int check_every = device_stop                        ? kCheckEvery
+                          : prm.check_every > 0              ? prm.check_every
                           : tune_get(TUNE_CHECK_EVERY) > 0 ? tune_get(TUNE_CHECK_EVERY)
                                                            : kCheckEvery;
   const int flush_every = tune_get(TUNE_FLUSH_EVERY);
@@ -802,15 +832,17 @@ static rhmc_status_t solve_phase1(rhmc_ctx *c, const double2 *B, int n, int ns, 
     }
     // a captured chunk replays for every later chunk with the same start modulo kCheckEvery
     // (the k % 2 buffer and k % 3 state-slot patterns), so its length must divide kCheckEvery
-    const bool graph = use_graphs() && chunk == check_every && kCheckEvery % check_every == 0 && k > 0 &&
-                       k % check_every == 0;
+    const bool graph = use_graphs() && chunk == check_every && kCheckEvery % check_every == 0 &&
+                       (k > 0 || device_stop) && k % check_every == 0;
     if (graph)
       RHMC_TRY(run_chunk_graph<T>(c, b, X, n, ns, sigma0, k, chunk, tol_shift, freeze, s));
     else
       RHMC_TRY(run_chunk<T>(c, b, X, n, ns, sigma0, k, chunk, tol_shift, freeze, s));
+    const int k_before = k;
     k += chunk;
-    stats.dirac += chunk;
     RHMC_TRY(read_state(c, b.st, v, s));
+    if (device_stop && v.done) k = v.nit;
+    stats.dirac += k - k_before;
     if (v.device_timeout) {
       set_error("a bounded device-side wait expired in the tensor-core update (iteration %d)", k);
       stats.iters = k;

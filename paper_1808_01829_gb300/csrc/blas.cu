@@ -97,7 +97,8 @@ __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_g
 // and the CTA reduction writes the rest as conjugates.
 template <typename T, int N, bool SAME, bool PK, int TR = kGramTileRows, int WG = kGramWarps>
 __global__ void __launch_bounds__(WG * 32) k_gram(const C<T> *__restrict__ A, const C<T> *__restrict__ B, long rows,
-                                                  double2 *__restrict__ partial) {
+                                                  double2 *__restrict__ partial, const int *__restrict__ done) {
+  if (done && *done) return;
   constexpr int TE = TR * N;  // complex per tile and operand
   constexpr int E = (N * N + 31) / 32;   // entries per lane
   constexpr bool STRUCT = (N == 16);
@@ -222,7 +223,8 @@ __global__ void __launch_bounds__(WG * 32) k_gram(const C<T> *__restrict__ A, co
 
 // out[e] = sum over the nparts partials of entry e, fixed order.
 __global__ void __launch_bounds__(128) k_gram_sum(const double2 *__restrict__ partial, int nparts,
-                                                  double2 *__restrict__ out) {
+                                                  double2 *__restrict__ out, const int *__restrict__ done) {
+  if (done && *done) return;
   __shared__ double2 red[128];
   const int e = blockIdx.x;
   double2 s = make_double2(0.0, 0.0);
@@ -763,7 +765,9 @@ template <int N, int R, int WW>
 __global__ void __launch_bounds__(WW * 32, 1) k_base_step(const float2 *__restrict__ Wf, float2 *__restrict__ Q,
                                                         float2 *__restrict__ P, float2 *__restrict__ X,
                                                         const float2 *__restrict__ coef, float2 *__restrict__ basis,
-                                                        int cap, const int *__restrict__ kdev, long rows) {
+                                                        int cap, const int *__restrict__ kdev,
+                                                        const int *__restrict__ upd, long rows) {
+  if (upd && !*upd) return;
   constexpr int TILE = R * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int CS = (3 * N * N + 1) & ~1;  // coefficient area, padded: the tiles start on 16-byte boundaries
@@ -881,7 +885,7 @@ constexpr int kBaseRows = 8, kBaseWarps = 16;
 
 template <int N, int R, int WW>
 static void launch_base(const float2 *W, float2 *Q, float2 *P, float2 *X, const float2 *coef, float2 *basis, int cap,
-                        const int *kdev, long rows, cudaStream_t s) {
+                        const int *kdev, const int *upd, long rows, cudaStream_t s) {
   const int threads = WW * 32;
   const size_t smem = (((3 * N * N + 1) & ~1) + (size_t)WW * 6 * R * N) * sizeof(float2);
   static std::once_flag attr;
@@ -891,11 +895,11 @@ static void launch_base(const float2 *W, float2 *Q, float2 *P, float2 *X, const 
   const long ntiles = (rows + R - 1) / R;
   long grid = (ntiles + WW - 1) / WW;
   grid = std::min(grid, (long)resident_ctas(k_base_step<N, R, WW>, threads, smem));
-  k_base_step<N, R, WW><<<(unsigned)grid, threads, smem, s>>>(W, Q, P, X, coef, basis, cap, kdev, rows);
+  k_base_step<N, R, WW><<<(unsigned)grid, threads, smem, s>>>(W, Q, P, X, coef, basis, cap, kdev, upd, rows);
 }
 
 rhmc_status_t base_step(const float2 *W, float2 *Q, float2 *P, float2 *X, const float2 *coef, float2 *basis, int cap,
-                        const int *kdev, long rows, int n, cudaStream_t s) {
+                        const int *kdev, const int *upd, long rows, int n, cudaStream_t s) {
   if (rows % 8) return RHMC_ERR_INVALID_ARG;
   prof_begin(PROF_UPDATE_SHIFTS32, s);
   rhmc_status_t rc = RHMC_OK;
@@ -905,15 +909,15 @@ rhmc_status_t base_step(const float2 *W, float2 *Q, float2 *P, float2 *X, const 
   {                                                                                              \
     if constexpr (NN == 16) {                                                                    \
       if (tile == 1)                                                                             \
-        launch_base<NN, 16, 12>(W, Q, P, X, coef, basis, cap, kdev, rows, s);                    \
+        launch_base<NN, 16, 12>(W, Q, P, X, coef, basis, cap, kdev, upd, rows, s);                    \
       else if (tile == 2)                                                                        \
-        launch_base<NN, 16, 8>(W, Q, P, X, coef, basis, cap, kdev, rows, s);                     \
+        launch_base<NN, 16, 8>(W, Q, P, X, coef, basis, cap, kdev, upd, rows, s);                     \
       else if (tile == 3)                                                                        \
-        launch_base<NN, 8, 12>(W, Q, P, X, coef, basis, cap, kdev, rows, s);                     \
+        launch_base<NN, 8, 12>(W, Q, P, X, coef, basis, cap, kdev, upd, rows, s);                     \
       else                                                                                       \
-        launch_base<NN, kBaseRows, kBaseWarps>(W, Q, P, X, coef, basis, cap, kdev, rows, s);     \
+        launch_base<NN, kBaseRows, kBaseWarps>(W, Q, P, X, coef, basis, cap, kdev, upd, rows, s);     \
     } else {                                                                                     \
-      launch_base<NN, kBaseRows, kBaseWarps>(W, Q, P, X, coef, basis, cap, kdev, rows, s);       \
+      launch_base<NN, kBaseRows, kBaseWarps>(W, Q, P, X, coef, basis, cap, kdev, upd, rows, s);       \
     }                                                                                            \
   }
   RHMC_DISPATCH_N(n, L_BASE)
@@ -1109,7 +1113,9 @@ template <int N, int R, int W, bool PK>
 __global__ void __launch_bounds__(W * 32, 1) k_axpy_gram_cols(const float2 *__restrict__ A,
                                                            const float2 *__restrict__ Cin,
                                                            const float2 *__restrict__ M, float2 *__restrict__ Y,
-                                                           long rows, double2 *__restrict__ partial) {
+                                                           long rows, double2 *__restrict__ partial,
+                                                           const int *__restrict__ done) {
+  if (done && *done) return;
   constexpr int TILE = R * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1233,7 +1239,7 @@ static void launch_axpy_cols(const float2 *A, const float2 *C, const float2 *M, 
 
 template <int N, bool PK>
 static void launch_axpy_gram_cols(const float2 *A, const float2 *C, const float2 *M, float2 *Y, long rows,
-                                  double2 *scratch, double2 *out, cudaStream_t s) {
+                                  double2 *scratch, double2 *out, const int *done, cudaStream_t s) {
   constexpr int W = axpy_gram_warps<PK>();
   // rows per warp tile: 8, or 16 at n = 16 with RHMC_TUNE_AXPY_ROWS = 1
   constexpr int R = (PK && N == 16) ? 16 : kAxpyRows;
@@ -1250,25 +1256,25 @@ static void launch_axpy_gram_cols(const float2 *A, const float2 *C, const float2
     const long ntiles = (rows + rr - 1) / rr;
     long grid = (ntiles + W - 1) / W;
     grid = std::min(grid, (long)std::min(kGramCtas, resident_ctas(kern, threads, smem)));
-    kern<<<(unsigned)grid, threads, smem, s>>>(A, C, M, Y, rows, scratch);
+    kern<<<(unsigned)grid, threads, smem, s>>>(A, C, M, Y, rows, scratch, done);
     return grid;
   };
   const long grid = big ? run(k_axpy_gram_cols<N, R, W, PK>, R) : run(k_axpy_gram_cols<N, kAxpyRows, W, PK>, kAxpyRows);
-  k_gram_sum<<<N * N, 128, 0, s>>>(scratch, (int)grid, out);
+  k_gram_sum<<<N * N, 128, 0, s>>>(scratch, (int)grid, out, done);
   count_launch();  // the second kernel of this launcher (the caller counts the first)
 }
 
 // Y = C + A M and out = Y^dagger Y (FP64 sums of FP32 products) in one pass over
 // the rows; scratch holds kGramCtas * n * n partials.
 rhmc_status_t axpy_gram_cols(const float2 *A, const float2 *C, const float2 *M, float2 *Y, long rows, int n,
-                             double2 *scratch, double2 *out, cudaStream_t s) {
+                             double2 *scratch, double2 *out, cudaStream_t s, const int *done) {
   if (rows % 8 || !C) return RHMC_ERR_INVALID_ARG;
   prof_begin(PROF_AXPY, s);
 #define L_AG(NN)                                                        \
   if (axpy_packed())                                                    \
-    launch_axpy_gram_cols<NN, true>(A, C, M, Y, rows, scratch, out, s); \
+    launch_axpy_gram_cols<NN, true>(A, C, M, Y, rows, scratch, out, done, s); \
   else                                                                  \
-    launch_axpy_gram_cols<NN, false>(A, C, M, Y, rows, scratch, out, s)
+    launch_axpy_gram_cols<NN, false>(A, C, M, Y, rows, scratch, out, done, s)
   RHMC_DISPATCH_N(n, L_AG)
 #undef L_AG
   prof_end(s, (double)rows * n * sizeof(float2) * 3);
@@ -1371,7 +1377,8 @@ __global__ void __launch_bounds__(256) k_redot(const double2 *__restrict__ A, co
 // ------------------------------------------------------------ launchers
 
 template <typename T, int N, bool PK, int TR, int WG>
-static void launch_gram_tw(const C<T> *A, const C<T> *B, long rows, double2 *scratch, double2 *out, cudaStream_t s) {
+static void launch_gram_tw(const C<T> *A, const C<T> *B, long rows, double2 *scratch, double2 *out, const int *done,
+                           cudaStream_t s) {
   const bool same = (A == B);
   const size_t smem = (size_t)WG * 2 * (same ? 1 : 2) * TR * N * sizeof(C<T>);
   const size_t smem_red = (size_t)WG * N * N * sizeof(double2);
@@ -1388,52 +1395,57 @@ static void launch_gram_tw(const C<T> *A, const C<T> *B, long rows, double2 *scr
                             : resident_ctas(k_gram<T, N, false, PK, TR, WG>, threads, bytes);
   const int grid = (int)std::min<long>((ntiles + WG - 1) / WG, std::min(kGramCtas, resident));
   if (same)
-    k_gram<T, N, true, PK, TR, WG><<<grid, threads, bytes, s>>>(A, B, rows, scratch);
+    k_gram<T, N, true, PK, TR, WG><<<grid, threads, bytes, s>>>(A, B, rows, scratch, done);
   else
-    k_gram<T, N, false, PK, TR, WG><<<grid, threads, bytes, s>>>(A, B, rows, scratch);
-  k_gram_sum<<<N * N, 128, 0, s>>>(scratch, grid, out);
+    k_gram<T, N, false, PK, TR, WG><<<grid, threads, bytes, s>>>(A, B, rows, scratch, done);
+  k_gram_sum<<<N * N, 128, 0, s>>>(scratch, grid, out, done);
   count_launch();  // the second kernel of this launcher (the caller counts the first)
 }
 template <typename T, int N, bool PK>
-static void launch_gram(const C<T> *A, const C<T> *B, long rows, double2 *scratch, double2 *out, cudaStream_t s) {
+static void launch_gram(const C<T> *A, const C<T> *B, long rows, double2 *scratch, double2 *out, const int *done,
+                        cudaStream_t s) {
   // packed n = 16: tile rows x warps from RHMC_TUNE_GRAM_TILE (0: 16 x 4, measured at 24^4:
   // 37.6 us against 41.8 for 16 x 8, 38.2 for 32 x 8, 41.5 for 8 x 8)
   if constexpr (PK && N == 16) {
     switch (tune_get(TUNE_GRAM_TILE)) {
-      case 1: launch_gram_tw<T, N, PK, 32, 8>(A, B, rows, scratch, out, s); return;
-      case 2: launch_gram_tw<T, N, PK, 16, 8>(A, B, rows, scratch, out, s); return;
-      case 3: launch_gram_tw<T, N, PK, 8, 8>(A, B, rows, scratch, out, s); return;
-      default: launch_gram_tw<T, N, PK, 16, 4>(A, B, rows, scratch, out, s); return;
+      case 1: launch_gram_tw<T, N, PK, 32, 8>(A, B, rows, scratch, out, done, s); return;
+      case 2: launch_gram_tw<T, N, PK, 16, 8>(A, B, rows, scratch, out, done, s); return;
+      case 3: launch_gram_tw<T, N, PK, 8, 8>(A, B, rows, scratch, out, done, s); return;
+      default: launch_gram_tw<T, N, PK, 16, 4>(A, B, rows, scratch, out, done, s); return;
     }
   }
-  launch_gram_tw<T, N, PK, kGramTileRows, kGramWarps>(A, B, rows, scratch, out, s);
+  launch_gram_tw<T, N, PK, kGramTileRows, kGramWarps>(A, B, rows, scratch, out, done, s);
 }
 
 // packed FMAs for FP32 at n = 16 unless RHMC_TUNE_AXPY_SCALAR = 1
 template <typename T, int N>
-static void launch_gram_any(const C<T> *A, const C<T> *B, long rows, double2 *scratch, double2 *out, cudaStream_t s) {
+static void launch_gram_any(const C<T> *A, const C<T> *B, long rows, double2 *scratch, double2 *out, const int *done,
+                            cudaStream_t s) {
   if constexpr (N == 16 && sizeof(T) == 4) {
     if (tune_get(TUNE_AXPY_SCALAR) != 1) {
-      launch_gram<T, N, true>(A, B, rows, scratch, out, s);
+      launch_gram<T, N, true>(A, B, rows, scratch, out, done, s);
       return;
     }
   }
-  launch_gram<T, N, false>(A, B, rows, scratch, out, s);
+  launch_gram<T, N, false>(A, B, rows, scratch, out, done, s);
 }
 
 // G = A^dagger B into out (n x n, FP64); scratch holds kGramCtas * n * n partials.
 template <typename T>
-rhmc_status_t gram(const C<T> *A, const C<T> *B, long rows, int n, double2 *scratch, double2 *out, cudaStream_t s) {
+rhmc_status_t gram(const C<T> *A, const C<T> *B, long rows, int n, double2 *scratch, double2 *out, cudaStream_t s,
+                   const int *done) {
   prof_begin(sizeof(T) == 4 ? PROF_GRAM32 : PROF_GRAM64, s);
-#define L_GRAM(NN) launch_gram_any<T, NN>(A, B, rows, scratch, out, s)
+#define L_GRAM(NN) launch_gram_any<T, NN>(A, B, rows, scratch, out, done, s)
   RHMC_DISPATCH_N(n, L_GRAM)
 #undef L_GRAM
   prof_end(s, (double)rows * n * sizeof(C<T>) * (A == B ? 1 : 2));
   RHMC_LAUNCH_CHECK();
   return RHMC_OK;
 }
-template rhmc_status_t gram<float>(const float2 *, const float2 *, long, int, double2 *, double2 *, cudaStream_t);
-template rhmc_status_t gram<double>(const double2 *, const double2 *, long, int, double2 *, double2 *, cudaStream_t);
+template rhmc_status_t gram<float>(const float2 *, const float2 *, long, int, double2 *, double2 *, cudaStream_t,
+                                          const int *);
+template rhmc_status_t gram<double>(const double2 *, const double2 *, long, int, double2 *, double2 *, cudaStream_t,
+                                           const int *);
 
 template <typename TA, typename TY>
 rhmc_status_t block_axpy(const C<TA> *A, const C<TY> *Cin, const C<TA> *M, C<TY> *Y, long rows, int n,

@@ -325,7 +325,9 @@ static void launch_hop(const Geom &g, int par, const C<T> *links, const C<T> *in
 template <int N, int R, bool SELF, bool REC>
 __global__ void __launch_bounds__(128) k_hop_pf(Geom g, int par, const float2 *__restrict__ links,
                                                 const float2 *__restrict__ in, float2 *__restrict__ out,
-                                                const float2 *__restrict__ self, float a, int bc_t) {
+                                                const float2 *__restrict__ self, float a, int bc_t,
+                                                const SolverState *__restrict__ st) {
+  const int done = st ? st->done : 0;                        // (tested once the loads below are on their way)
   constexpr int TPS = N / R;                                 // threads per site
   constexpr int TILE = (128 / TPS) < 32 ? (128 / TPS) : 32;  // sites per CTA (static shared memory <= 20 KB)
   constexpr int LR = REC ? 48 : 72;  // complex per site record as stored
@@ -357,7 +359,12 @@ __global__ void __launch_bounds__(128) k_hop_pf(Geom g, int par, const float2 *_
     const int lex = y0 + g.L[0] * (y1 + g.L[1] * (y2 + g.L[2] * y3));
     snb[k] = (lex >> 1) * 3 * N;
   }
+  const double a_st = (SELF && st) ? st->a0 : 0.0;
   __syncthreads();
+  if (done) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    return;
+  }
   const int ls = tid / TPS, j = (tid - (tid / TPS) * TPS) * R;
   const bool live = ls < nsites;
   float2 v[8][3][R];
@@ -406,6 +413,7 @@ __global__ void __launch_bounds__(128) k_hop_pf(Geom g, int par, const float2 *_
       }
   float2 *op = out + (long)(h0 + ls) * 3 * N + j;
   if (SELF) {
+    if (st) a = (float)a_st;
     const float2 *sp = self + (long)(h0 + ls) * 3 * N + j;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -421,25 +429,27 @@ __global__ void __launch_bounds__(128) k_hop_pf(Geom g, int par, const float2 *_
 
 template <int N, int R>
 static void launch_hop_pf_n(const Geom &g, int par, const float2 *links, const float2 *in, float2 *out,
-                            const float2 *self, double a, const float2 *links12, int bc_t, cudaStream_t s) {
+                            const float2 *self, double a, const float2 *links12, int bc_t, const SolverState *st,
+                            cudaStream_t s) {
   constexpr int TPS = N / R;
   constexpr int TILE = (128 / TPS) < 32 ? (128 / TPS) : 32;
   const int threads = ((TILE * TPS + 31) / 32) * 32;
   const unsigned grid = (unsigned)((g.Vh + TILE - 1) / TILE);
   if (links12) {
     if (self)
-      k_hop_pf<N, R, true, true><<<grid, threads, 0, s>>>(g, par, links12, in, out, self, (float)a, bc_t);
+      k_hop_pf<N, R, true, true><<<grid, threads, 0, s>>>(g, par, links12, in, out, self, (float)a, bc_t, st);
     else
-      k_hop_pf<N, R, false, true><<<grid, threads, 0, s>>>(g, par, links12, in, out, self, (float)a, bc_t);
+      k_hop_pf<N, R, false, true><<<grid, threads, 0, s>>>(g, par, links12, in, out, self, (float)a, bc_t, st);
   } else if (self) {
-    k_hop_pf<N, R, true, false><<<grid, threads, 0, s>>>(g, par, links, in, out, self, (float)a, bc_t);
+    k_hop_pf<N, R, true, false><<<grid, threads, 0, s>>>(g, par, links, in, out, self, (float)a, bc_t, st);
   } else {
-    k_hop_pf<N, R, false, false><<<grid, threads, 0, s>>>(g, par, links, in, out, self, (float)a, bc_t);
+    k_hop_pf<N, R, false, false><<<grid, threads, 0, s>>>(g, par, links, in, out, self, (float)a, bc_t, st);
   }
 }
 
 static bool launch_hop_pf(const Geom &g, int par, const float2 *links, const float2 *in, float2 *out,
-                          const float2 *self, double a, int n, const float2 *links12, int bc_t, cudaStream_t s) {
+                          const float2 *self, double a, int n, const float2 *links12, int bc_t,
+                          const SolverState *st, cudaStream_t s) {
   // two right-hand sides per thread (16-byte loads, half the load instructions): built-in
   // for even n >= 12 (measured at 24^4: n = 16 65 us against 71 us; n = 8 no gain)
   const int mode = tune_get(TUNE_HOP_STAGED);
@@ -449,11 +459,11 @@ static bool launch_hop_pf(const Geom &g, int par, const float2 *links, const flo
   case NN:                                                                         \
     if constexpr (NN % 2 == 0) {                                                   \
       if (r2) {                                                                    \
-        launch_hop_pf_n<NN, 2>(g, par, links, in, out, self, a, links12, bc_t, s); \
+        launch_hop_pf_n<NN, 2>(g, par, links, in, out, self, a, links12, bc_t, st, s); \
         return true;                                                               \
       }                                                                            \
     }                                                                              \
-    launch_hop_pf_n<NN, 1>(g, par, links, in, out, self, a, links12, bc_t, s);     \
+    launch_hop_pf_n<NN, 1>(g, par, links, in, out, self, a, links12, bc_t, st, s);     \
     return true;
     L_PF(1) L_PF(2) L_PF(3) L_PF(4) L_PF(5) L_PF(6) L_PF(7) L_PF(8)
     L_PF(9) L_PF(10) L_PF(11) L_PF(12) L_PF(13) L_PF(14) L_PF(15) L_PF(16)
@@ -672,7 +682,8 @@ static bool try_hop_staged(const Geom &g, int par, const C<T> *links, const C<T>
 
 template <typename T>
 rhmc_status_t hop(const Geom &g, int par, const C<T> *links, const C<T> *in, C<T> *out, const C<T> *self, double a,
-                  int n, int nbatch, long bstride, cudaStream_t s, const C<T> *links12, int bc_t) {
+                  int n, int nbatch, long bstride, cudaStream_t s, const C<T> *links12, int bc_t,
+                  const SolverState *st) {
   if (n < 1 || n > RHMC_MAX_NRHS || g.Vh * 3L * n > 0x7fffffffL) return RHMC_ERR_INVALID_ARG;
   prof_begin(sizeof(T) == 4 ? PROF_HOP32 : PROF_HOP64, s);
   int R = tune_get(TUNE_HOP_RHS_PER_THREAD);
@@ -682,7 +693,7 @@ rhmc_status_t hop(const Geom &g, int par, const C<T> *links, const C<T> *in, C<T
   } else if (use_hop_pf<T>(links, in, nbatch)) {
     launch_hop_pf(g, par, reinterpret_cast<const float2 *>(links), reinterpret_cast<const float2 *>(in),
                   reinterpret_cast<float2 *>(out), reinterpret_cast<const float2 *>(self), a, n,
-                  reinterpret_cast<const float2 *>(links12), bc_t, s);
+                  reinterpret_cast<const float2 *>(links12), bc_t, st, s);
   } else if (R == 4)
     launch_hop<T, 4>(g, par, links, in, out, self, a, n, nbatch, bstride, s);
   else if (R == 2)
@@ -1131,9 +1142,9 @@ rhmc_status_t df_split(const double2 *in, float4 *out, long len, cudaStream_t s)
 }
 
 template rhmc_status_t hop<float>(const Geom &, int, const float2 *, const float2 *, float2 *, const float2 *, double,
-                                  int, int, long, cudaStream_t, const float2 *, int);
+                                  int, int, long, cudaStream_t, const float2 *, int, const SolverState *);
 template rhmc_status_t hop<double>(const Geom &, int, const double2 *, const double2 *, double2 *, const double2 *,
-                                   double, int, int, long, cudaStream_t, const double2 *, int);
+                                   double, int, int, long, cudaStream_t, const double2 *, int, const SolverState *);
 
 // 12-real copies of the FP32 records; returns through *ok whether every record
 // is f V with V in SU(3) to FP32 accuracy (then the hop may use the copies).

@@ -32,16 +32,22 @@ struct SolverState {
   int kabs[kSlots];           // absolute iteration number of slot k % kSlots (graph replays reuse k's slot)
   int breakdown;              // nonzero: which coefficient step failed
   int device_timeout;         // a bounded device-side wait expired
+  int done;                   // the base residuals are below stop_tol: later iterations change nothing
+  int nit;                    // iterations run (device count; up to the one that set done)
+  double stop_tol;            // > 0: stop on the device once every base residual is below (single shift, mixed)
+  double a0;                  // 4 m^2 + sigma_0 (the mixed solve's operator reads it here)
 };
 
 // dslash.cu
 rhmc_status_t stage_links(const Geom &g, const double2 *U, int bc_t, double2 *l64[2], float2 *l32[2],
                           cudaStream_t s);
 // links12: optional 12-real copy of `links` (FP32 single-field hops use it), bc_t
-// its boundary condition (signs of the rebuilt third rows)
+// its boundary condition (signs of the rebuilt third rows); st (optional, all-directions
+// kernel): a is read from st->a0 and nothing is done once st->done is set
 template <typename T>
 rhmc_status_t hop(const Geom &g, int par, const C<T> *links, const C<T> *in, C<T> *out, const C<T> *self, double a,
-                  int n, int nbatch, long bstride, cudaStream_t s, const C<T> *links12 = nullptr, int bc_t = -1);
+                  int n, int nbatch, long bstride, cudaStream_t s, const C<T> *links12 = nullptr, int bc_t = -1,
+                  const SolverState *st = nullptr);
 rhmc_status_t stage_links12(const Geom &g, int bc_t, float2 *const l32[2], float2 *l12[2], bool *ok, cudaStream_t s);
 
 // FP64-accurate operator on the integer units (fx.cuh): integer link records (int4 per
@@ -79,7 +85,8 @@ rhmc_status_t df_split(const double2 *in, float4 *out, long len, cudaStream_t s)
 // blas.cu
 constexpr int kGramCtas = 4 * 152;  // CTAs of the Gram kernel (its scratch holds kGramCtas * n * n partials)
 template <typename T>
-rhmc_status_t gram(const C<T> *A, const C<T> *B, long rows, int n, double2 *scratch, double2 *out, cudaStream_t s);
+rhmc_status_t gram(const C<T> *A, const C<T> *B, long rows, int n, double2 *scratch, double2 *out, cudaStream_t s,
+                   const int *done = nullptr);
 template <typename TA, typename TY>
 rhmc_status_t block_axpy(const C<TA> *A, const C<TY> *Cin, const C<TA> *M, C<TY> *Y, long rows, int n,
                          cudaStream_t s);
@@ -96,11 +103,12 @@ rhmc_status_t axpy_cols(const float2 *A, const float2 *C, const float2 *M, float
                         cudaStream_t s);
 // Y = C + A M fused with out = Y^dagger Y (n x n FP64, scratch: kGramCtas * n * n partials)
 rhmc_status_t axpy_gram_cols(const float2 *A, const float2 *C, const float2 *M, float2 *Y, long rows, int n,
-                             double2 *scratch, double2 *out, cudaStream_t s);
+                             double2 *scratch, double2 *out, cudaStream_t s, const int *done = nullptr);
 // The base step after rho_k in one pass: Q = W rho^-1, X^(0) += P^(0) M1, P^(0) = Q + P^(0) M2
-// (coef: rho^-1, M1, M2), and Q into basis block *kdev when basis is given (capacity cap)
+// (coef: rho^-1, M1, M2), and Q into basis block *kdev when basis is given (capacity cap);
+// nothing when *upd is 0
 rhmc_status_t base_step(const float2 *W, float2 *Q, float2 *P, float2 *X, const float2 *coef, float2 *basis, int cap,
-                        const int *kdev, long rows, int n, cudaStream_t s);
+                        const int *kdev, const int *upd, long rows, int n, cudaStream_t s);
 // FP32 shifted updates (Algorithm 1) with column-owner lanes and cp.async-staged row tiles
 rhmc_status_t update_shifts_cols(const float2 *Q, float2 *P, float2 *X, const float2 *coef, const int *upd,
                                  int s_begin, int s_end, long rows, int n, long fstride, cudaStream_t s);

@@ -462,6 +462,8 @@ __global__ void __launch_bounds__(256) k_qr_init(const double2 *partial, int npa
   if (c.t == 0) {
     st->breakdown = 0;
     st->device_timeout = 0;
+    st->done = 0;
+    st->nit = 0;
   }
 }
 

@@ -312,9 +312,12 @@ __global__ void __launch_bounds__(256) k_nxn_alpha_dd(const double2 *G, int n, S
   const int cur = k % kSlots;
   const int t = threadIdx.x, i = t >> 4, j = t & 15;
   const bool in = i < n && j < n;
-  if (t == 0) st->kabs[cur] = st->kabs[(k - 1) % kSlots] + 1;
+  const int done = st->done;  // a later iteration of a chunk whose solve has stopped: no output
   cd h0;
-  if (!ldl16(n, G, A, Li, rd, &flag, h0)) {
+  const bool ok = ldl16(n, G, A, Li, rd, &flag, h0);
+  if (done) return;
+  if (t == 0) st->kabs[cur] = st->kabs[(k - 1) % kSlots] + 1;
+  if (!ok) {
     if (t == 0) st->breakdown = 2;
     return;
   }
@@ -353,13 +356,19 @@ __global__ void __launch_bounds__(256) k_nxn_rho_dd(const double2 *G, int n, Sol
   const int cur = k % kSlots, prev = (k - 1) % kSlots;
   const int t = threadIdx.x, i = t >> 4, j = t & 15, nn = n * n;
   const bool in = i < n && j < n;
+  const int done = st->done;  // a later iteration of a chunk whose solve has stopped: no output
   // alpha_k and delta_{k-1} do not depend on the factorisation (ldl16's barriers publish them)
   if (in) {
     Al[t] = from_z(st->alpha[cur][i * n + j]);
     Dp[t] = from_z(st->delta[prev][i * n + j]);
   }
   cd h0;
-  if (!ldl16(n, G, A, Li, rd, &flag, h0)) {
+  const bool ok = ldl16(n, G, A, Li, rd, &flag, h0);
+  if (done) {
+    if (t == 0) st->upd[0] = 0;
+    return;
+  }
+  if (!ok) {
     if (t == 0) st->breakdown = 3;
     return;
   }
@@ -410,8 +419,20 @@ __global__ void __launch_bounds__(256) k_nxn_rho_dd(const double2 *G, int n, Sol
   __syncthreads();  // A, Li, Al are read above: reuse Li for delta_k
   Li[t] = dk;
   __syncthreads();
-  colnorms_upper_dd(n, Li, kS, st->res[0], st->inv_d0);
-  if (t == 0) st->upd[0] = 1;
+  __shared__ double res[kMaxN];
+  colnorms_upper_dd(n, Li, kS, res, st->inv_d0);
+  __syncthreads();
+  if (t < n) st->res[0][t] = res[t];
+  if (t == 0) {
+    st->upd[0] = 1;
+    st->nit += 1;
+    const double stop = st->stop_tol;
+    if (stop > 0.0) {
+      bool all = true;
+      for (int q = 0; q < n; ++q) all = all && res[q] < stop;
+      if (all) st->done = 1;
+    }
+  }
 }
 
 // shifted coefficients and updates for shift s = blockIdx.x + 1 (the FP64 k_nxn_shifts of small.cu in

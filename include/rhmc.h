@@ -113,7 +113,8 @@ rhmc_status_t rhmc_set_gauge(rhmc_ctx_t *ctx, const void *U_dev, rhmc_stream_t s
  * arguments.  In mixed precision with several shifts this includes the stored
  * block basis (RHMC_TUNE_BASIS_ITERS: built in, up to 384 blocks of
  * V/2 * 3 * n_rhs * 8 bytes within a quarter of the device memory, e.g.
- * 24.5 GB at 24^4, n_rhs = 16); RHMC_TUNE_BASIS_ITERS = 1 sizes without it. */
+ * 24.5 GB at 24^4, n_rhs = 16), in FP64 one of up to 768 blocks of 16 bytes per
+ * entry within the same limit; RHMC_TUNE_BASIS_ITERS = 1 sizes without it. */
 size_t rhmc_workspace_bytes(const rhmc_ctx_t *ctx, int n_rhs, int n_shifts, rhmc_precision_t p);
 
 /* Y = (A + sigma) X for an n_rhs-wide block (multi-RHS operator, each link
@@ -236,9 +237,9 @@ rhmc_status_t rhmc_force_lie(rhmc_ctx_t *ctx, const void *U_dev, const void *G_d
  * the rational sum is needed):
  *   Y = alpha0 Phi + sum_s alpha_s (A + beta_s)^-1 Phi.
  * FP64 throughout.  The solve keeps X^(0) (smallest shift) and one field for
- * sum_{s>=1} alpha_s X^(s), added in the fused shifted update (the per-shift
- * X^(s) are never written), so it needs about n_shifts - 2 fewer fields than
- * rhmc_block_multishift_cg and moves less data per iteration.
+ * sum_{s>=1} alpha_s X^(s), formed at the end from the stored block basis and the
+ * summed coefficients (the per-shift X^(s) are never written; a solve longer
+ * than the basis adds the rest in the fused shifted update).
  *   Phi, Y   complex128 [V/2][3][n_pf] on the device (no aliasing)
  *   alpha, beta  host [n_shifts], beta >= 0 (any sign of alpha: x^(+r) works)
  *   workspace  rhmc_rational_solve_bytes(ctx, n_pf, n_shifts) bytes, or NULL (pool)

@@ -371,6 +371,7 @@ struct SolveBufs {
   double2 *hist = nullptr;
   BasisBufs asmb;
   int cap = 0;
+  double2 *basis64 = nullptr;  // the FP64 solve's stored basis [cap][rows][n]; Q_k is formed in block k
 };
 
 // Stored-basis capacity.  RHMC_TUNE_BASIS_ITERS: 0 = built-in, 1 = off, >= 2 = that
@@ -400,6 +401,20 @@ static int basis_cap(const Geom &g, int n, int ns, bool mixed) {
   const size_t block = (size_t)g.Vh * 3 * n * sizeof(float2);
   const size_t fit = (device_total_memory() / 4) / std::max<size_t>(block, 1);
   const int cap = (int)std::min<size_t>(fit, kBasisCapMax) & ~1;
+  return cap >= kBasisCapMin ? cap : 0;
+}
+
+// Stored-basis capacity of the FP64 solve (same setting): up to kBasisCapMax64 blocks within a
+// quarter of the device's memory.
+constexpr int kBasisCapMax64 = 768;
+static int basis_cap64(const Geom &g, int n, int ns) {
+  if (ns < 2) return 0;
+  const int v = tune_get(TUNE_BASIS_ITERS);
+  if (v == 1) return 0;
+  if (v >= 2) return v;
+  const size_t block = (size_t)g.Vh * 3 * n * sizeof(double2);
+  const size_t fit = (device_total_memory() / 4) / std::max<size_t>(block, 1);
+  const int cap = (int)std::min<size_t>(fit, kBasisCapMax64);
   return cap >= kBasisCapMin ? cap : 0;
 }
 
@@ -440,6 +455,15 @@ static void layout_solve(Arena &a, const Geom &g, int n, int ns, bool mixed, Sol
     b.asmb.bpack = a.take<unsigned char>(basis_pack_bytes(n, ns, cap));
     b.asmb.bscale = a.take<double>((size_t)ns);
     b.asmb.tile_nkt = a.take<int>((size_t)ns);
+  }
+  const int cap64 = mixed ? 0 : basis_cap64(g, n, ns);
+  if (cap64 > 0) {
+    b.cap = cap64;
+    b.basis64 = a.take<double2>((size_t)cap64 * len);
+    b.hist = a.take<double2>((size_t)cap64 * ns * 2 * n * n);
+    b.asmb.hist = b.hist;
+    b.asmb.cap = cap64;
+    b.asmb.cf = a.take<double2>((size_t)ns * (cap64 + 1) * n * n);
   }
 }
 
@@ -568,6 +592,24 @@ static rhmc_status_t sbcgrq_iteration(rhmc_ctx *c, const SolveBufs &b, TX *Xacc,
   RHMC_TRY(gram<T>(P, AP, rows, n, b.gscratch, b.partial, s, done));
   RHMC_TRY(nxn_alpha<T>(b.partial, kGramParts, n, b.st, k, (C<T> *)b.mw, s));
   const bool cols = use_column_update<T>();
+  if constexpr (sizeof(T) == 8) {
+    if (b.basis64) {
+      const int *kdev = &b.st->kabs[k % kSlots];
+      RHMC_TRY(axpy64(AP, b.basis64, kdev, (const double2 *)b.mw, W, rows, n, s));
+      RHMC_TRY(gram<T>(W, W, rows, n, b.gscratch, b.partial, s));
+      RHMC_TRY(nxn_rho<T>(b.partial, kGramParts, n, b.st, k, (C<T> *)b.coef, s));
+      RHMC_TRY(base64(W, b.basis64, kdev, P, (double2 *)Xacc, (const double2 *)b.coef, rows, n, s));
+      if (ns > 1) {
+        if (split) {
+          RHMC_CUDA_TRY(cudaEventRecord(c->ev_base[k % 3], s));
+          RHMC_CUDA_TRY(cudaStreamWaitEvent(ss, c->ev_base[k % 3], 0));
+        }
+        RHMC_TRY(nxn_shifts<T>(n, ns, b.st, k, (C<T> *)b.coef, tol_shift, freeze, b.hist, b.cap, ss));
+        if (split) RHMC_CUDA_TRY(cudaEventRecord(c->ev_side[k % 3], ss));
+      }
+      return RHMC_OK;
+    }
+  }
   if (cols) {
     // W = Q - (AP) alpha and its Gram W^dagger W in one pass
     RHMC_TRY(axpy_gram_cols((const float2 *)AP, (const float2 *)Qprev, (const float2 *)b.mw, (float2 *)W, rows, n,
@@ -651,7 +693,7 @@ static rhmc_status_t run_chunk_graph(rhmc_ctx *c, const SolveBufs &b, double2 *X
   // (mixed: the chunk does not touch X; with device stop it reads sigma_0 and the tolerance
   // from the state, so that one graph serves the corrections of every shift)
   const bool mixed = sizeof(T) == 4;
-  std::vector<double> key = {(double)(uintptr_t)b.P, mixed ? 0.0 : (double)(uintptr_t)X, (double)(uintptr_t)b.basis,
+  std::vector<double> key = {(double)(uintptr_t)b.P, mixed ? 0.0 : (double)(uintptr_t)X, (double)(uintptr_t)b.basis + (double)(uintptr_t)b.basis64,
                              (double)b.accumulate, (double)n,
                              (double)ns, b.device_stop ? 0.0 : sigma0, b.device_stop ? 0.0 : target, (double)freeze,
                              (double)sizeof(T), (double)len, (double)(chunk_start % kCheckEvery),
@@ -738,21 +780,26 @@ static rhmc_status_t solve_phase1(rhmc_ctx *c, const double2 *B, int n, int ns, 
   const double sigma0 = shifts[0];
   // stored-basis mode (mixed, several shifts, not accumulating): b.basis set
   SolveBufs b = b0;
-  if (!mixed || ns < 2 || b.accumulate) b.basis = nullptr, b.hist = nullptr, b.cap = 0;
+  if (mixed && (ns < 2 || b.accumulate)) b.basis = nullptr, b.hist = nullptr, b.cap = 0;
+  const bool has64 = b.basis64 != nullptr;
   // X^(s) = sum_i Q_i C_i (want_p = 0), or P^(s) = sum_{i <= K} Q_i D_i (want_p = 1),
   // for s >= 1 from the stored basis (tcgen05 kernel whose epilogue writes the FP64
   // solutions; RHMC_TUNE_BASIS_CHUNK: FP32 partial sums over that many blocks).  X^(s),
   // s >= 1, is zero until then: the shifted increments are not updated in this mode.
   auto assemble = [&](int K, int want_p) -> rhmc_status_t {
     if (K <= 0 && !want_p) return RHMC_OK;
+    if (has64)
+      return basis64_assemble(b.asmb, b.basis64, n, ns, b.st, rows, K, want_p, b.accumulate,
+                              want_p ? (double2 *)b.P + len : X + len, len, s);
     return basis_assemble(b.asmb, n, ns, b.st, rows, K, want_p, X, (float2 *)b.P, len, tune_get(TUNE_BASIS_CHUNK),
                           tune_get(TUNE_BASIS_GEMM) == 1, tune_get(TUNE_BASIS_ACC_KT), &b.st->device_timeout, s);
   };
   // end of the stored-basis mode at iteration K: the shifted solutions so far into X
   auto finish_basis = [&](int K) -> rhmc_status_t {
-    if (!b.basis) return RHMC_OK;
+    if (!b.basis && !b.basis64) return RHMC_OK;
     RHMC_TRY(assemble(K, 0));
-    b.basis = nullptr, b.hist = nullptr, b.cap = 0;
+    b.basis = nullptr, b.basis64 = nullptr, b.hist = nullptr, b.cap = 0;
+    if (has64) return RHMC_OK;
     StateView vf;
     RHMC_TRY(read_state(c, b.st, vf, s));
     if (vf.device_timeout) {
@@ -791,7 +838,9 @@ static rhmc_status_t solve_phase1(rhmc_ctx *c, const double2 *B, int n, int ns, 
     RHMC_TRY(nxn_qr_init<double>(b.partial, kGramParts, n, ns, b.st, b.rinv64, s));
     RHMC_TRY(block_axpy<double, T>(B, nullptr, b.rinv64, (C<T> *)b.Qb[0], rows, n, s));
   }
-  for (int q = 0; q < ns; ++q)
+  if (has64)
+    RHMC_CUDA_TRY(cudaMemcpyAsync(b.basis64, b.Qb[0], sizeof(double2) * len, cudaMemcpyDeviceToDevice, s));
+  for (int q = 0; q < (has64 ? 1 : ns); ++q)
     RHMC_CUDA_TRY(cudaMemcpyAsync((C<T> *)b.P + q * len, b.Qb[0], sizeof(C<T>) * len, cudaMemcpyDeviceToDevice, s));
   if (mixed) RHMC_CUDA_TRY(cudaMemsetAsync(b.Xinc, 0, sizeof(float2) * len * ns, s));
   if (b.basis) RHMC_TRY(basis_store((const float2 *)b.Qb[0], b.basis, rows, n, b.cap, 0, s));
@@ -824,11 +873,15 @@ static rhmc_status_t solve_phase1(rhmc_ctx *c, const double2 *B, int n, int ns, 
   while (k < kmax) {
     const int chunk = prm.fixed_iters > 0 ? kmax : std::min(check_every, kmax - k);
     const int freeze = prm.fixed_iters > 0 ? 0 : 1;
-    if (b.basis && k + chunk > b.cap - 1) {
+    if ((b.basis || b.basis64) && k + chunk > b.cap - 1) {
       // the basis is full: X^(s) and P^(s) from it, then the shifted updates in HBM
       RHMC_TRY(assemble(k, 0));
       RHMC_TRY(assemble(k, 1));
-      b.basis = nullptr, b.hist = nullptr, b.cap = 0;
+      // (the FP64 basis also held Q_k)
+      if (b.basis64)
+        RHMC_CUDA_TRY(cudaMemcpyAsync(b.Qb[k & 1], b.basis64 + (size_t)k * len, sizeof(double2) * len,
+                                      cudaMemcpyDeviceToDevice, s));
+      b.basis = nullptr, b.basis64 = nullptr, b.hist = nullptr, b.cap = 0;
     }
     // a captured chunk replays for every later chunk with the same start modulo kCheckEvery
     // (the k % 2 buffer and k % 3 state-slot patterns), so its length must divide kCheckEvery

@@ -644,15 +644,21 @@ __global__ void __launch_bounds__(256) k_basis_gemm_simt(const float2 *__restric
 }
 
 // ------------------------------------------------------------ host
+rhmc_status_t basis_coef(const BasisBufs &bb, int n, int nshift, const SolverState *st, int K, int want_p,
+                         cudaStream_t s) {
+  prof_begin(PROF_NXN_SHIFTS, s);
+  k_basis_coef<<<nshift - 1, 256, 0, s>>>(n, nshift, st, bb.hist, K, want_p, bb.cf, bb.cap + 1);
+  prof_end(s, 0.0);
+  RHMC_LAUNCH_CHECK();
+  return RHMC_OK;
+}
+
 rhmc_status_t basis_assemble(const BasisBufs &bb, int n, int nshift, const SolverState *st, long rows, int K,
                              int want_p, double2 *X, float2 *P, long fstride, int chunk_blocks, int simt, int acc_kt,
                              int *err, cudaStream_t s) {
   if (nshift < 2 || (K <= 0 && !want_p)) return RHMC_OK;
   const long cfstride = bb.cap + 1;
-  prof_begin(PROF_NXN_SHIFTS, s);
-  k_basis_coef<<<nshift - 1, 256, 0, s>>>(n, nshift, st, bb.hist, K, want_p, bb.cf, cfstride);
-  prof_end(s, 0.0);
-  RHMC_LAUNCH_CHECK();
+  RHMC_TRY(basis_coef(bb, n, nshift, st, K, want_p, s));
   const int nblk_all = want_p ? K + 1 : K;
   const double out_bytes = (double)rows * n * (nshift - 1) * (want_p ? sizeof(float2) : sizeof(double2));
   if (simt) {

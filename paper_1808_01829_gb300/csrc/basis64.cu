@@ -1,0 +1,265 @@
+// FP64 solve with the stored block Krylov basis.
+//
+// The shifted updates of Algorithm 1 cost two n x n products per row, shift and
+// iteration, at this GPU's FP64 rate the largest part of an FP64 solve (36 us on average
+// per update at 8^4, n = 4, 11 shifts, against 100 us per iteration).  As in the
+// mixed solve (basis.cu), the solve keeps the blocks Q_0, Q_1, ... and the recorded
+// n x n coefficients, and forms the shifted solutions once at the end,
+//   X^(s) = sum_{i < L_s} Q_i C^(s)_i,
+// one product per row, shift and iteration instead of two, off the iteration's path,
+// without P^(s) and X^(s) going through memory.  Where only the rational sum
+// sum_s w_s X^(s) is wanted (heatbath, action), the coefficients are summed first:
+// one product per row and iteration for all shifts together.
+// The blocks are written where they stay ([block][rows][n]): iteration k forms Q_k in block
+// k of the basis (k from the device counter: graph replays).
+#include <algorithm>
+#include <mutex>
+
+#include "common.cuh"
+#include "kernels.h"
+
+namespace rhmc {
+
+#define RHMC_DISPATCH_N(n, MACRO) \
+  switch (n) {                    \
+    case 1: MACRO(1); break;      \
+    case 2: MACRO(2); break;      \
+    case 3: MACRO(3); break;      \
+    case 4: MACRO(4); break;      \
+    case 5: MACRO(5); break;      \
+    case 6: MACRO(6); break;      \
+    case 7: MACRO(7); break;      \
+    case 8: MACRO(8); break;      \
+    case 9: MACRO(9); break;      \
+    case 10: MACRO(10); break;    \
+    case 11: MACRO(11); break;    \
+    case 12: MACRO(12); break;    \
+    case 13: MACRO(13); break;    \
+    case 14: MACRO(14); break;    \
+    case 15: MACRO(15); break;    \
+    case 16: MACRO(16); break;    \
+    default: return RHMC_ERR_INVALID_ARG; \
+  }
+
+namespace {
+// Rows of n columns, one lane per (row, column); the rows of a warp lie side by side and do
+// not straddle it (32 / N rows, the remaining lanes idle).
+template <int N> struct Lanes {
+  static constexpr int RPW = 32 / N;
+  long row;
+  int j;
+  bool in;
+  __device__ Lanes(long base, long rows) {
+    const int lane = threadIdx.x & 31, slot = lane / N;
+    j = lane - slot * N;
+    row = base + (threadIdx.x >> 5) * RPW + slot;
+    in = slot < RPW && row < rows;
+  }
+};
+}  // namespace
+
+// W = Q_{k-1} + A M: the block QR step, Q_{k-1} in block *kdev - 1 of the basis.  One lane per
+// output, so that small lattices spread over the FP64 units of the whole GPU (each FP64
+// instruction of a warp takes 64 clocks however few there are).
+template <int N>
+__global__ void __launch_bounds__(128) k_axpy64(const double2 *__restrict__ A, const double2 *__restrict__ basis,
+                                                const int *__restrict__ kdev, const double2 *__restrict__ M,
+                                                double2 *__restrict__ Y, long rows) {
+  __shared__ double2 sm[N * N];
+  for (int k = threadIdx.x; k < N * N; k += blockDim.x) sm[k] = M[k];
+  const double2 *Q = basis + (size_t)(*kdev - 1) * rows * N;
+  __syncthreads();
+  const long per = 4 * Lanes<N>::RPW;
+  for (long base = (long)blockIdx.x * per; base < rows; base += (long)gridDim.x * per) {
+    const Lanes<N> l(base, rows);
+    if (!l.in) continue;
+    double2 acc = czero<double>();
+#pragma unroll
+    for (int k = 0; k < N; ++k) cmac<double>(acc, __ldg(A + l.row * N + k), sm[k * N + l.j]);
+    const double2 q = Q[l.row * N + l.j];
+    Y[l.row * N + l.j] = make_double2(q.x + acc.x, q.y + acc.y);
+  }
+}
+
+// The base updates of Algorithm 1 after rho_k: Q_k = W rho^-1 into block *kdev of the basis,
+// X^(0) += P M1, P = Q_k + P M2.  rho^-1 is upper and M2 = rho^dagger lower triangular, so
+// column j of Q takes terms k <= j and column j of P M2 terms k >= j: n + 1 products
+// together, formed in one running sum whose value after the first j + 1 is Q.
+template <int N>
+__global__ void __launch_bounds__(128) k_base64(const double2 *__restrict__ W, double2 *__restrict__ basis,
+                                                const int *__restrict__ kdev, double2 *P, double2 *X,
+                                                const double2 *__restrict__ coef, long rows) {
+  __shared__ double2 sm[3 * N * N];
+  for (int k = threadIdx.x; k < 3 * N * N; k += blockDim.x) sm[k] = coef[k];
+  double2 *Q = basis + (size_t)*kdev * rows * N;
+  __syncthreads();
+  const long per = 4 * Lanes<N>::RPW;
+  for (long base = (long)blockIdx.x * per; base < rows; base += (long)gridDim.x * per) {
+    const Lanes<N> l(base, rows);
+    double2 p[N];
+    const long o = l.row * N;
+    if (l.in) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) p[k] = P[o + k];
+    }
+    __syncwarp();  // the row is read by all its lanes before any of them writes its column
+    if (l.in) {
+      double2 x = X[o + l.j], a = czero<double>(), q = czero<double>(), acc = czero<double>();
+#pragma unroll
+      for (int t = 0; t <= N; ++t) {
+        if (t == l.j + 1) q = acc;
+        const bool first = t <= l.j;
+        const double2 u = first ? __ldg(W + o + (t < N ? t : N - 1)) : p[t > 0 ? t - 1 : 0];
+        const double2 c = first ? sm[(t < N ? t : N - 1) * N + l.j] : sm[2 * N * N + (t > 0 ? t - 1 : 0) * N + l.j];
+        cmac<double>(acc, u, c);
+      }
+#pragma unroll
+      for (int k = 0; k < N; ++k) cmac<double>(a, p[k], sm[N * N + k * N + l.j]);
+      Q[o + l.j] = q;
+      P[o + l.j] = acc;
+      X[o + l.j] = make_double2(x.x + a.x, x.y + a.y);
+    }
+    __syncwarp();
+  }
+}
+
+// Weighted sum of the shifts' expansion coefficients (basis_coef's cf): block i of the sum
+// takes w_s C^(s)_i of every shift s >= 1 with more than i blocks.
+__global__ void __launch_bounds__(256) k_basis64_combine(int n, int nshift, const SolverState *__restrict__ st, int K,
+                                                         const double2 *__restrict__ cf, long cfstride,
+                                                         double2 *__restrict__ out) {
+  const int i = blockIdx.x, t = threadIdx.x, nn = n * n;
+  if (t >= nn) return;
+  double2 sum = make_double2(0.0, 0.0);
+  for (int s = 1; s < nshift; ++s) {
+    if (i >= min(st->last_k[s], K)) continue;
+    const double w = st->w1[s];
+    const double2 c = cf[((size_t)(s - 1) * cfstride + i) * nn + t];
+    sum.x = fma(w, c.x, sum.x);
+    sum.y = fma(w, c.y, sum.y);
+  }
+  out[(size_t)i * nn + t] = sum;
+}
+
+// out_s = sum_i Q_i C^(s)_i for the shifts s0 + SG blockIdx.y ... (want = 0: X^(s), last_s
+// blocks; 1: P^(s), K + 1 blocks, active shifts; 2: one combined set, all K blocks).  One lane
+// per (row, column), SG shifts each, so that a row of Q is read once for SG shifts;
+// coefficients staged IC blocks at a time.  Bound by the FP64 pipe.
+template <int N, int SG>
+__global__ void __launch_bounds__(128) k_basis64_apply(const double2 *__restrict__ basis, long rows,
+                                                       const SolverState *__restrict__ st, int K, int want, int nshift,
+                                                       const double2 *__restrict__ cf, long cfstride, int IC,
+                                                       double2 *__restrict__ out, long fstride) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2 *sc = reinterpret_cast<double2 *>(smem_raw);  // [SG][IC][N * N]
+  constexpr int NN = N * N;
+  const int s0 = 1 + SG * blockIdx.y;
+  int nblk[SG], most = 0;
+#pragma unroll
+  for (int g = 0; g < SG; ++g) {
+    const int s = s0 + g;
+    nblk[g] = s >= nshift ? 0 : want == 2 ? K : want == 1 ? (st->active[s] ? K + 1 : 0) : max(0, min(st->last_k[s], K));
+    most = max(most, nblk[g]);
+  }
+  const Lanes<N> l((long)blockIdx.x * 4 * Lanes<N>::RPW, rows);
+  double2 acc[SG];
+#pragma unroll
+  for (int g = 0; g < SG; ++g) acc[g] = czero<double>();
+  for (int b = 0; b < most; b += IC) {
+    const int nb = min(IC, most - b);
+    __syncthreads();
+    for (int k = threadIdx.x; k < SG * nb * NN; k += blockDim.x) {
+      const int g = k / (nb * NN), r = k - g * (nb * NN);
+      const int i = b + r / NN;
+      sc[g * IC * NN + r] = i < (g < SG ? nblk[g] : 0) ? cf[((size_t)(s0 - 1 + g) * cfstride + b) * NN + r]
+                                                       : make_double2(0.0, 0.0);
+    }
+    __syncthreads();
+    if (!l.in) continue;
+    for (int i = 0; i < nb; ++i) {
+      const double2 *q = basis + ((size_t)(b + i) * rows + l.row) * N;
+      const double2 *c = sc + i * NN + l.j;
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        const double2 u = __ldg(q + k);
+#pragma unroll
+        for (int g = 0; g < SG; ++g)
+          if (b + i < nblk[g]) cmac<double>(acc[g], u, c[g * IC * NN + k * N]);
+      }
+    }
+  }
+  if (!l.in) return;
+#pragma unroll
+  for (int g = 0; g < SG; ++g)
+    if (s0 + g < nshift && (want != 1 || nblk[g])) out[(size_t)(s0 - 1 + g) * fstride + l.row * N + l.j] = acc[g];
+}
+
+rhmc_status_t axpy64(const double2 *A, const double2 *basis, const int *kdev, const double2 *M, double2 *Y, long rows,
+                     int n, cudaStream_t s) {
+  prof_begin(PROF_AXPY, s);
+#define L_(NN)                                                                                          \
+  {                                                                                                     \
+    const long grid = std::min<long>((rows + 4 * Lanes<NN>::RPW - 1) / (4 * Lanes<NN>::RPW), 16 * 152); \
+    k_axpy64<NN><<<(unsigned)grid, 128, 0, s>>>(A, basis, kdev, M, Y, rows);                            \
+  }
+  RHMC_DISPATCH_N(n, L_)
+#undef L_
+  prof_end(s, (double)rows * n * sizeof(double2) * 3);
+  RHMC_LAUNCH_CHECK();
+  return RHMC_OK;
+}
+
+rhmc_status_t base64(const double2 *W, double2 *basis, const int *kdev, double2 *P, double2 *X, const double2 *coef,
+                     long rows, int n, cudaStream_t s) {
+  prof_begin(PROF_UPDATE64, s);
+#define L_(NN)                                                                                          \
+  {                                                                                                     \
+    const long grid = std::min<long>((rows + 4 * Lanes<NN>::RPW - 1) / (4 * Lanes<NN>::RPW), 16 * 152); \
+    k_base64<NN><<<(unsigned)grid, 128, 0, s>>>(W, basis, kdev, P, X, coef, rows);                      \
+  }
+  RHMC_DISPATCH_N(n, L_)
+#undef L_
+  prof_end(s, (double)rows * n * sizeof(double2) * 6);
+  RHMC_LAUNCH_CHECK();
+  return RHMC_OK;
+}
+
+template <int N, int SG>
+static void launch_apply(const BasisBufs &bb, const double2 *basis, const double2 *cf, int nshift,
+                         const SolverState *st, long rows, int K, int want, double2 *out, long fstride,
+                         cudaStream_t s) {
+  constexpr int NN = N * N;
+  const int IC = std::max(1, std::min(16, 40 * 1024 / (int)(SG * NN * sizeof(double2))));
+  const dim3 grid((unsigned)((rows + 4 * Lanes<N>::RPW - 1) / (4 * Lanes<N>::RPW)), (unsigned)((nshift - 2 + SG) / SG));
+  k_basis64_apply<N, SG><<<grid, 128, (size_t)SG * IC * NN * sizeof(double2), s>>>(
+      basis, rows, st, K, want, nshift, cf, bb.cap + 1, IC, out, fstride);
+}
+
+rhmc_status_t basis64_assemble(const BasisBufs &bb, const double2 *basis, int n, int nshift, const SolverState *st,
+                               long rows, int K, int want_p, int combine, double2 *out, long fstride, cudaStream_t s) {
+  if (nshift < 2 || (K <= 0 && !want_p)) return RHMC_OK;
+  RHMC_TRY(basis_coef(bb, n, nshift, st, K, want_p, s));
+  const double2 *cf = bb.cf;
+  int ns = nshift, want = want_p;
+  if (combine && !want_p) {
+    double2 *sum = bb.cf + (size_t)(nshift - 1) * (bb.cap + 1) * n * n;
+    k_basis64_combine<<<K, 256, 0, s>>>(n, nshift, st, K, bb.cf, bb.cap + 1, sum);
+    RHMC_LAUNCH_CHECK();
+    cf = sum;
+    ns = 2;
+    want = 2;
+  }
+  prof_begin(PROF_UPDATE64, s);
+#define L_(NN)                                                                                   \
+  if (ns > 2)                                                                                    \
+    launch_apply<NN, 4>(bb, basis, cf, ns, st, rows, K, want, out, fstride, s);                  \
+  else                                                                                           \
+    launch_apply<NN, 1>(bb, basis, cf, ns, st, rows, K, want, out, fstride, s)
+  RHMC_DISPATCH_N(n, L_)
+#undef L_
+  prof_end(s, (double)rows * n * sizeof(double2) * (K + ns - 1.0));
+  RHMC_LAUNCH_CHECK();
+  return RHMC_OK;
+}
+
+}  // namespace rhmc

@@ -589,15 +589,17 @@ static rhmc_status_t sbcgrq_iteration(rhmc_ctx *c, const SolveBufs &b, TX *Xacc,
   // rest of its chunk)
   const int *done = b.device_stop ? &b.st->done : nullptr;
   RHMC_TRY(apply_A<T>(c, P, AP, Todd, b.ex, n, sigma0, s, b.device_stop ? b.st : nullptr));
-  RHMC_TRY(gram<T>(P, AP, rows, n, b.gscratch, b.partial, s, done));
-  RHMC_TRY(nxn_alpha<T>(b.partial, kGramParts, n, b.st, k, (C<T> *)b.mw, s));
+  int np = 1;  // partials left for the n x n kernel (in gscratch), or 1: the summed matrix
+  auto gsum = [&]() { return np > 1 ? b.gscratch : b.partial; };
+  RHMC_TRY(gram<T>(P, AP, rows, n, b.gscratch, b.partial, s, done, &np));
+  RHMC_TRY(nxn_alpha<T>(gsum(), np, n, b.st, k, (C<T> *)b.mw, s));
   const bool cols = use_column_update<T>();
   if constexpr (sizeof(T) == 8) {
     if (b.basis64) {
       const int *kdev = &b.st->kabs[k % kSlots];
       RHMC_TRY(axpy64(AP, b.basis64, kdev, (const double2 *)b.mw, W, rows, n, s));
-      RHMC_TRY(gram<T>(W, W, rows, n, b.gscratch, b.partial, s));
-      RHMC_TRY(nxn_rho<T>(b.partial, kGramParts, n, b.st, k, (C<T> *)b.coef, s));
+      RHMC_TRY(gram<T>(W, W, rows, n, b.gscratch, b.partial, s, nullptr, &np));
+      RHMC_TRY(nxn_rho<T>(gsum(), np, n, b.st, k, (C<T> *)b.coef, s));
       RHMC_TRY(base64(W, b.basis64, kdev, P, (double2 *)Xacc, (const double2 *)b.coef, rows, n, s));
       if (ns > 1) {
         if (split) {
@@ -613,12 +615,12 @@ static rhmc_status_t sbcgrq_iteration(rhmc_ctx *c, const SolveBufs &b, TX *Xacc,
   if (cols) {
     // W = Q - (AP) alpha and its Gram W^dagger W in one pass
     RHMC_TRY(axpy_gram_cols((const float2 *)AP, (const float2 *)Qprev, (const float2 *)b.mw, (float2 *)W, rows, n,
-                            b.gscratch, b.partial, s, done));
+                            b.gscratch, b.partial, s, done, &np));
   } else {
     RHMC_TRY(block_axpy<T, T>(AP, Qprev, (const C<T> *)b.mw, W, rows, n, s));
-    RHMC_TRY(gram<T>(W, W, rows, n, b.gscratch, b.partial, s));
+    RHMC_TRY(gram<T>(W, W, rows, n, b.gscratch, b.partial, s, nullptr, &np));
   }
-  RHMC_TRY(nxn_rho<T>(b.partial, kGramParts, n, b.st, k, (C<T> *)b.coef, s));
+  RHMC_TRY(nxn_rho<T>(gsum(), np, n, b.st, k, (C<T> *)b.coef, s));
   // base: Q_k = W rho_k^-1, X^(0), P^(0)
   if (cols && tune_get(TUNE_AXPY_SCALAR) != 1) {
     // one pass: Q_k = W rho^-1, X^(0), P^(0), and block k of the stored basis (k from the

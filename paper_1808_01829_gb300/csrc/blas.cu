@@ -17,6 +17,7 @@
 #include <tuple>
 
 #include "common.cuh"
+#include "gramsum.cuh"
 #include "kernels.h"
 
 namespace rhmc {
@@ -101,6 +102,7 @@ __global__ void __launch_bounds__(WG * 32) k_gram(const C<T> *__restrict__ A, co
   if (done && *done) return;
   constexpr int TE = TR * N;  // complex per tile and operand
   constexpr int E = (N * N + 31) / 32;   // entries per lane
+  constexpr int SL = N * N <= 16 ? 32 / (N * N) : 1;  // small n: row slices, N * N lanes each
   constexpr bool STRUCT = (N == 16);
   constexpr bool PACKED = PK && STRUCT && sizeof(T) == 4;
   constexpr int NQ = 5;  // circulant entries per lane (packed form)
@@ -176,13 +178,21 @@ __global__ void __launch_bounds__(WG * 32) k_gram(const C<T> *__restrict__ A, co
         for (int q = 0; q < 8; ++q) cmac_cj<T>(acc[q], a, b[q]);
       }
     } else {
+      if constexpr (SL > 1) {
+        const int sl = lane / (N * N), e = lane - sl * (N * N);
+        if (sl < SL) {
 #pragma unroll 4
-      for (int r = 0; r < TR; ++r)
-#pragma unroll
-        for (int q = 0; q < E; ++q) {
-          const int e = lane + 32 * q;
-          if (e < N * N) cmac_cj<T>(acc[q], ta[r * N + e / N], tb[r * N + e % N]);
+          for (int r = sl; r < TR; r += SL) cmac_cj<T>(acc[0], ta[r * N + e / N], tb[r * N + e % N]);
         }
+      } else {
+#pragma unroll 4
+        for (int r = 0; r < TR; ++r)
+#pragma unroll
+          for (int q = 0; q < E; ++q) {
+            const int e = lane + 32 * q;
+            if (e < N * N) cmac_cj<T>(acc[q], ta[r * N + e / N], tb[r * N + e % N]);
+          }
+      }
     }
     __syncwarp();
     st ^= 1;
@@ -204,6 +214,14 @@ __global__ void __launch_bounds__(WG * 32) k_gram(const C<T> *__restrict__ A, co
       if (o > 0 && 2 * o != N) red[warp * N * N + j * N + i] = make_double2(gx, -gy);
     }
   } else {
+    if constexpr (SL > 1) {  // the slices' sums to the first one's lanes
+      const C<T> own = acc[0];
+#pragma unroll 1
+      for (int q = 1; q < SL; ++q) {
+        acc[0].x += __shfl_sync(0xffffffffu, own.x, (lane + q * N * N) & 31);
+        acc[0].y += __shfl_sync(0xffffffffu, own.y, (lane + q * N * N) & 31);
+      }
+    }
 #pragma unroll
     for (int q = 0; q < E; ++q) {
       const int e = STRUCT ? (lane >> 1) * N + (lane & 1) * 8 + q : lane + 32 * q;
@@ -243,6 +261,20 @@ __global__ void __launch_bounds__(128) k_gram_sum(const double2 *__restrict__ pa
     __syncthreads();
   }
   if (threadIdx.x == 0) out[e] = red[0];
+}
+
+// After a Gram kernel of nparts CTAs: with `left` and few partials they are left for the n x n
+// kernel (*left = nparts), else summed into out (*left = 1).
+template <int N>
+static void sum_or_leave(const double2 *scratch, int nparts, double2 *out, const int *done, int *left,
+                         cudaStream_t s) {
+  if (left) *left = 1;
+  if (left && nparts > 1 && nparts <= gram_sum_most(N * N)) {
+    *left = nparts;
+    return;
+  }
+  k_gram_sum<<<N * N, 128, 0, s>>>(scratch, nparts, out, done);
+  count_launch();  // the second kernel of its launcher (the caller counts the first)
 }
 
 // Whole-row loads: 16-byte vector loads when the row is 16-byte aligned.
@@ -756,7 +788,9 @@ static rhmc_status_t launch_update_cols_variant(const float2 *Q, float2 *P, floa
 // rho^-1, M1, M2 (n x n each).  Each warp stages a tile of R rows of W, P^(0)
 // and X^(0) by cp.async; pass 1: lane j < n forms column j of Q (stored to Q
 // and the basis) while lane n + j forms column j of X; pass 2: lane n + j
-// (with lane j) forms column j of P, each lane of the pair half of the sum.  It
+// (with lane j) forms column j of P, each lane of the pair half of the sum.  For
+// n <= 8 the warp holds 32 / 2n such groups of lanes, on different rows (16^3 x 32,
+// n = 8: 31 -> 21 us; 12^4, n = 4: 6.3 -> 3.9 us).  It
 // replaces three passes (Q = W rho^-1, the basis copy, the base update):
 // W, P, X read once, Q, P, X (and the basis block) written once.  The tiles
 // are double-buffered: a warp's next row tile is in flight while the current
@@ -778,8 +812,12 @@ __global__ void __launch_bounds__(WW * 32, 1) k_base_step(const float2 *__restri
   const int kb = (basis && kdev) ? *kdev : -1;
   const bool store_basis = kb >= 0 && kb < cap;
   __syncthreads();
-  const bool lo = lane < N, hi = lane >= N && lane < 2 * N;
-  const int j = lo ? lane : (hi ? lane - N : 0);
+  // 32 / 2N groups of 2N lanes, each on every NG-th row of the tile
+  constexpr int NG = N <= 16 ? 32 / (2 * N) : 1;
+  constexpr int RL = (R + NG - 1) / NG;  // rows per lane
+  const int grp = lane / (2 * N), l2 = lane - grp * (2 * N);
+  const bool lo = grp < NG && l2 < N, hi = grp < NG && l2 >= N;
+  const int j = lo ? l2 : (hi ? l2 - N : 0);
   const long ntiles = (rows + R - 1) / R;
   const long t0 = (long)blockIdx.x * WW + warp, dt = (long)gridDim.x * WW;
   auto issue = [&](long tile, int b) {
@@ -817,10 +855,11 @@ __global__ void __launch_bounds__(WW * 32, 1) k_base_step(const float2 *__restri
     cpa_wait<1>();
     __syncwarp();
     // pass 1: row r of W (lanes < N) or of P (lanes N .. 2N-1) times the lane's column
-    float2 qv[R];
+    float2 qv[RL];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      qv[r] = make_float2(0.f, 0.f);
+    for (int i = 0; i < RL; ++i) {
+      const int r = i * NG + grp;
+      qv[i] = make_float2(0.f, 0.f);
       if (r < nr && (lo || hi)) {
         const float2 *u = (lo ? wt : pt) + r * N;
         unsigned long long a = 0ull, b = 0ull;
@@ -834,7 +873,7 @@ __global__ void __launch_bounds__(WW * 32, 1) k_base_step(const float2 *__restri
         const float2 prod = make_float2(A.x - B.y, A.y + B.x);
         const long row = r0 + r;
         if (lo) {
-          qv[r] = prod;
+          qv[i] = prod;
           Q[row * N + j] = prod;
           if (store_basis) basis[row * (long)cap * N + (long)kb * N + j] = prod;
         } else {
@@ -858,7 +897,8 @@ __global__ void __launch_bounds__(WW * 32, 1) k_base_step(const float2 *__restri
       }
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
+    for (int i = 0; i < RL; ++i) {
+      const int r = i * NG + grp;
       float2 part = make_float2(0.f, 0.f);
       if (r < nr && (lo || hi)) {
         const float2 *u = pt + r * N + k0;
@@ -874,7 +914,7 @@ __global__ void __launch_bounds__(WW * 32, 1) k_base_step(const float2 *__restri
       }
       const float ox = __shfl_down_sync(0xffffffffu, part.x, N);
       const float oy = __shfl_down_sync(0xffffffffu, part.y, N);
-      if (r < nr && lo) P[(r0 + r) * N + j] = make_float2(qv[r].x + part.x + ox, qv[r].y + part.y + oy);
+      if (r < nr && lo) P[(r0 + r) * N + j] = make_float2(qv[i].x + part.x + ox, qv[i].y + part.y + oy);
     }
     __syncwarp();  // buffer buf is refilled for the tile after next
   }
@@ -1105,10 +1145,14 @@ __global__ void __launch_bounds__(W * 32, PK ? 1 : 2) k_axpy_cols(const float2 *
 }
 
 // Y = C + A M fused with the Gram G = Y^dagger Y (the thin-QR Gram of the block QR step):
-// after a row pair of Y is formed, it is written to the warp's row buffer and
-// lane (h, j) adds conj(Y[r][i]) Y[r][j] for all i to its FP32 column of G;
-// the columns are combined across the row parities, the warps (FP64, shared
-// memory) and the CTAs (partials summed in fixed order by k_gram_sum).
+// the warp works on 32 / n rows at once, lane (h, j) on column j of the h-th; after these rows
+// of Y are formed, they are written to the warp's row buffer and lane (h, j) adds
+// conj(Y[r][i]) Y[r][j] for all i to its FP32 column of G; the columns are combined
+// across the lanes, the warps (FP64, shared memory) and the CTAs (partials summed in
+// fixed order by k_gram_sum or the coefficient kernel).  Two rows per warp at every n took
+// 18.6 us at 16^3 x 32, n = 8, 32 / n take 13.7.
+// float2 of shared memory per warp: two buffers of A and C tiles, and the rows in flight
+template <int N, int R> constexpr int axpy_gram_warp_floats() { return 4 * R * N + ((32 / N) * N + 1) / 2 * 2; }
 template <int N, int R, int W, bool PK>
 __global__ void __launch_bounds__(W * 32, 1) k_axpy_gram_cols(const float2 *__restrict__ A,
                                                            const float2 *__restrict__ Cin,
@@ -1119,10 +1163,11 @@ __global__ void __launch_bounds__(W * 32, 1) k_axpy_gram_cols(const float2 *__re
   constexpr int TILE = R * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float2 *wb = reinterpret_cast<float2 *>(smem_raw) + (size_t)warp * (4 * TILE + 2 * N);  // [2][A, C], row pair
+  constexpr int H = 32 / N;  // rows in flight per warp
+  float2 *wb = reinterpret_cast<float2 *>(smem_raw) + (size_t)warp * axpy_gram_warp_floats<N, R>();  // [2][A, C], rows
   float2 *wrow = wb + 4 * TILE;
   const int h = lane / N, j = lane - (lane / N) * N;
-  const bool act = lane < 2 * N;
+  const bool act = h < H;
   // W^dagger W is Hermitian: lane j accumulates the circulant half G[(j + o) mod N][j],
   // o = 0 .. N/2; the reduction writes the other entries as conjugates
   constexpr int NO = N / 2 + 1;
@@ -1158,9 +1203,10 @@ __global__ void __launch_bounds__(W * 32, 1) k_axpy_gram_cols(const float2 *__re
     const int nr = (int)min((long)R, rows - r0);
     const float2 *at = wb + (2 * b) * TILE, *ct = wb + (2 * b + 1) * TILE;
 #pragma unroll 1
-    for (int r = 0; r < nr; r += 2) {
+    for (int r = 0; r < nr; r += H) {
       float2 y = make_float2(0.f, 0.f);
-      if (act) {
+      const bool on = act && r + h < nr;
+      if (on) {
         const float2 *ar = at + (r + h) * N;
         float2 p;
         if constexpr (PK)
@@ -1173,7 +1219,7 @@ __global__ void __launch_bounds__(W * 32, 1) k_axpy_gram_cols(const float2 *__re
         wrow[h * N + j] = y;
       }
       __syncwarp();
-      if (act) {
+      if (on) {
         const float2 *wr = wrow + h * N;
 #pragma unroll
         for (int o = 0; o < NO; ++o) {  // g[o] += conj(Y[r][i]) Y[r][j], i = (j + o) mod N
@@ -1187,11 +1233,18 @@ __global__ void __launch_bounds__(W * 32, 1) k_axpy_gram_cols(const float2 *__re
     __syncwarp();  // buffer b is refilled for the tile after next
   }
   cpa_wait<0>();
-  // row parities: lane j += lane N + j
+  // lane j += the lanes of its column on the other rows
+  {
+    float2 t[NO];
 #pragma unroll
-  for (int o = 0; o < NO; ++o) {
-    g[o].x += __shfl_down_sync(0xffffffffu, g[o].x, N);
-    g[o].y += __shfl_down_sync(0xffffffffu, g[o].y, N);
+    for (int o = 0; o < NO; ++o) t[o] = g[o];
+#pragma unroll 1
+    for (int q = 1; q < H; ++q)
+#pragma unroll
+      for (int o = 0; o < NO; ++o) {
+        g[o].x += __shfl_sync(0xffffffffu, t[o].x, (lane + q * N) & 31);
+        g[o].y += __shfl_sync(0xffffffffu, t[o].y, (lane + q * N) & 31);
+      }
   }
   __syncthreads();
   double2 *red = reinterpret_cast<double2 *>(smem_raw);  // [W][N * N], reuses the tile buffers
@@ -1239,42 +1292,42 @@ static void launch_axpy_cols(const float2 *A, const float2 *C, const float2 *M, 
 
 template <int N, bool PK>
 static void launch_axpy_gram_cols(const float2 *A, const float2 *C, const float2 *M, float2 *Y, long rows,
-                                  double2 *scratch, double2 *out, const int *done, cudaStream_t s) {
+                                  double2 *scratch, double2 *out, const int *done, int *nparts, cudaStream_t s) {
   constexpr int W = axpy_gram_warps<PK>();
   // rows per warp tile: 8, or 16 at n = 16 with RHMC_TUNE_AXPY_ROWS = 1
-  constexpr int R = (PK && N == 16) ? 16 : kAxpyRows;
+  constexpr int R0 = N == 1 ? 32 : N <= 3 ? 16 : kAxpyRows;  // (at least the 32 / n rows in flight)
+  constexpr int R = (PK && N == 16) ? 16 : R0;
   const bool big = (PK && N == 16) && tune_get(TUNE_AXPY_ROWS) == 1;
   static std::once_flag attr;
   std::call_once(attr, [] {
     cudaFuncSetAttribute(k_axpy_gram_cols<N, R, W, PK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-    cudaFuncSetAttribute(k_axpy_gram_cols<N, kAxpyRows, W, PK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         220 * 1024);
+    cudaFuncSetAttribute(k_axpy_gram_cols<N, R0, W, PK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
   });
-  auto run = [&](auto kern, int rr) {
+  auto run = [&](auto kern, int rr, int wf) {
     const int threads = W * 32;
-    const size_t smem = std::max((size_t)W * (4 * rr * N + 2 * N) * sizeof(float2), (size_t)W * N * N * sizeof(double2));
+    const size_t smem = std::max((size_t)W * wf * sizeof(float2), (size_t)W * N * N * sizeof(double2));
     const long ntiles = (rows + rr - 1) / rr;
     long grid = (ntiles + W - 1) / W;
     grid = std::min(grid, (long)std::min(kGramCtas, resident_ctas(kern, threads, smem)));
     kern<<<(unsigned)grid, threads, smem, s>>>(A, C, M, Y, rows, scratch, done);
     return grid;
   };
-  const long grid = big ? run(k_axpy_gram_cols<N, R, W, PK>, R) : run(k_axpy_gram_cols<N, kAxpyRows, W, PK>, kAxpyRows);
-  k_gram_sum<<<N * N, 128, 0, s>>>(scratch, (int)grid, out, done);
-  count_launch();  // the second kernel of this launcher (the caller counts the first)
+  const long grid = big ? run(k_axpy_gram_cols<N, R, W, PK>, R, axpy_gram_warp_floats<N, R>())
+                        : run(k_axpy_gram_cols<N, R0, W, PK>, R0, axpy_gram_warp_floats<N, R0>());
+  sum_or_leave<N>(scratch, (int)grid, out, done, nparts, s);
 }
 
 // Y = C + A M and out = Y^dagger Y (FP64 sums of FP32 products) in one pass over
 // the rows; scratch holds kGramCtas * n * n partials.
 rhmc_status_t axpy_gram_cols(const float2 *A, const float2 *C, const float2 *M, float2 *Y, long rows, int n,
-                             double2 *scratch, double2 *out, cudaStream_t s, const int *done) {
+                             double2 *scratch, double2 *out, cudaStream_t s, const int *done, int *nparts) {
   if (rows % 8 || !C) return RHMC_ERR_INVALID_ARG;
   prof_begin(PROF_AXPY, s);
 #define L_AG(NN)                                                        \
   if (axpy_packed())                                                    \
-    launch_axpy_gram_cols<NN, true>(A, C, M, Y, rows, scratch, out, done, s); \
+    launch_axpy_gram_cols<NN, true>(A, C, M, Y, rows, scratch, out, done, nparts, s); \
   else                                                                  \
-    launch_axpy_gram_cols<NN, false>(A, C, M, Y, rows, scratch, out, done, s)
+    launch_axpy_gram_cols<NN, false>(A, C, M, Y, rows, scratch, out, done, nparts, s)
   RHMC_DISPATCH_N(n, L_AG)
 #undef L_AG
   prof_end(s, (double)rows * n * sizeof(float2) * 3);
@@ -1378,7 +1431,7 @@ __global__ void __launch_bounds__(256) k_redot(const double2 *__restrict__ A, co
 
 template <typename T, int N, bool PK, int TR, int WG>
 static void launch_gram_tw(const C<T> *A, const C<T> *B, long rows, double2 *scratch, double2 *out, const int *done,
-                           cudaStream_t s) {
+                           int *nparts, cudaStream_t s) {
   const bool same = (A == B);
   const size_t smem = (size_t)WG * 2 * (same ? 1 : 2) * TR * N * sizeof(C<T>);
   const size_t smem_red = (size_t)WG * N * N * sizeof(double2);
@@ -1393,49 +1446,50 @@ static void launch_gram_tw(const C<T> *A, const C<T> *B, long rows, double2 *scr
   const int threads = WG * 32;
   const int resident = same ? resident_ctas(k_gram<T, N, true, PK, TR, WG>, threads, bytes)
                             : resident_ctas(k_gram<T, N, false, PK, TR, WG>, threads, bytes);
-  const int grid = (int)std::min<long>((ntiles + WG - 1) / WG, std::min(kGramCtas, resident));
+  int grid = (int)std::min<long>((ntiles + WG - 1) / WG, std::min(kGramCtas, resident));
+  // a little over what the n x n kernel sums itself: fewer CTAs with more tiles each
+  if (nparts && N <= 4 && grid > gram_sum_most(N * N) && grid <= 2 * gram_sum_most(N * N)) grid = gram_sum_most(N * N);
   if (same)
     k_gram<T, N, true, PK, TR, WG><<<grid, threads, bytes, s>>>(A, B, rows, scratch, done);
   else
     k_gram<T, N, false, PK, TR, WG><<<grid, threads, bytes, s>>>(A, B, rows, scratch, done);
-  k_gram_sum<<<N * N, 128, 0, s>>>(scratch, grid, out, done);
-  count_launch();  // the second kernel of this launcher (the caller counts the first)
+  sum_or_leave<N>(scratch, grid, out, done, nparts, s);
 }
 template <typename T, int N, bool PK>
 static void launch_gram(const C<T> *A, const C<T> *B, long rows, double2 *scratch, double2 *out, const int *done,
-                        cudaStream_t s) {
+                        int *nparts, cudaStream_t s) {
   // packed n = 16: tile rows x warps from RHMC_TUNE_GRAM_TILE (0: 16 x 4, measured at 24^4:
   // 37.6 us against 41.8 for 16 x 8, 38.2 for 32 x 8, 41.5 for 8 x 8)
   if constexpr (PK && N == 16) {
     switch (tune_get(TUNE_GRAM_TILE)) {
-      case 1: launch_gram_tw<T, N, PK, 32, 8>(A, B, rows, scratch, out, done, s); return;
-      case 2: launch_gram_tw<T, N, PK, 16, 8>(A, B, rows, scratch, out, done, s); return;
-      case 3: launch_gram_tw<T, N, PK, 8, 8>(A, B, rows, scratch, out, done, s); return;
-      default: launch_gram_tw<T, N, PK, 16, 4>(A, B, rows, scratch, out, done, s); return;
+      case 1: launch_gram_tw<T, N, PK, 32, 8>(A, B, rows, scratch, out, done, nparts, s); return;
+      case 2: launch_gram_tw<T, N, PK, 16, 8>(A, B, rows, scratch, out, done, nparts, s); return;
+      case 3: launch_gram_tw<T, N, PK, 8, 8>(A, B, rows, scratch, out, done, nparts, s); return;
+      default: launch_gram_tw<T, N, PK, 16, 4>(A, B, rows, scratch, out, done, nparts, s); return;
     }
   }
-  launch_gram_tw<T, N, PK, kGramTileRows, kGramWarps>(A, B, rows, scratch, out, done, s);
+  launch_gram_tw<T, N, PK, kGramTileRows, kGramWarps>(A, B, rows, scratch, out, done, nparts, s);
 }
 
 // packed FMAs for FP32 at n = 16 unless RHMC_TUNE_AXPY_SCALAR = 1
 template <typename T, int N>
 static void launch_gram_any(const C<T> *A, const C<T> *B, long rows, double2 *scratch, double2 *out, const int *done,
-                            cudaStream_t s) {
+                            int *nparts, cudaStream_t s) {
   if constexpr (N == 16 && sizeof(T) == 4) {
     if (tune_get(TUNE_AXPY_SCALAR) != 1) {
-      launch_gram<T, N, true>(A, B, rows, scratch, out, done, s);
+      launch_gram<T, N, true>(A, B, rows, scratch, out, done, nparts, s);
       return;
     }
   }
-  launch_gram<T, N, false>(A, B, rows, scratch, out, done, s);
+  launch_gram<T, N, false>(A, B, rows, scratch, out, done, nparts, s);
 }
 
 // G = A^dagger B into out (n x n, FP64); scratch holds kGramCtas * n * n partials.
 template <typename T>
 rhmc_status_t gram(const C<T> *A, const C<T> *B, long rows, int n, double2 *scratch, double2 *out, cudaStream_t s,
-                   const int *done) {
+                   const int *done, int *nparts) {
   prof_begin(sizeof(T) == 4 ? PROF_GRAM32 : PROF_GRAM64, s);
-#define L_GRAM(NN) launch_gram_any<T, NN>(A, B, rows, scratch, out, done, s)
+#define L_GRAM(NN) launch_gram_any<T, NN>(A, B, rows, scratch, out, done, nparts, s)
   RHMC_DISPATCH_N(n, L_GRAM)
 #undef L_GRAM
   prof_end(s, (double)rows * n * sizeof(C<T>) * (A == B ? 1 : 2));
@@ -1443,9 +1497,9 @@ rhmc_status_t gram(const C<T> *A, const C<T> *B, long rows, int n, double2 *scra
   return RHMC_OK;
 }
 template rhmc_status_t gram<float>(const float2 *, const float2 *, long, int, double2 *, double2 *, cudaStream_t,
-                                          const int *);
+                                          const int *, int *);
 template rhmc_status_t gram<double>(const double2 *, const double2 *, long, int, double2 *, double2 *, cudaStream_t,
-                                           const int *);
+                                           const int *, int *);
 
 template <typename TA, typename TY>
 rhmc_status_t block_axpy(const C<TA> *A, const C<TY> *Cin, const C<TA> *M, C<TY> *Y, long rows, int n,

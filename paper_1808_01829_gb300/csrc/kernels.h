@@ -84,9 +84,11 @@ rhmc_status_t df_split(const double2 *in, float4 *out, long len, cudaStream_t s)
 
 // blas.cu
 constexpr int kGramCtas = 4 * 152;  // CTAs of the Gram kernel (its scratch holds kGramCtas * n * n partials)
+// G = A^dagger B into out; with nparts and few CTAs their partials stay in scratch
+// ([entry][part]) for the n x n kernel to sum: *nparts > 1, else 1
 template <typename T>
 rhmc_status_t gram(const C<T> *A, const C<T> *B, long rows, int n, double2 *scratch, double2 *out, cudaStream_t s,
-                   const int *done = nullptr);
+                   const int *done = nullptr, int *nparts = nullptr);
 template <typename TA, typename TY>
 rhmc_status_t block_axpy(const C<TA> *A, const C<TY> *Cin, const C<TA> *M, C<TY> *Y, long rows, int n,
                          cudaStream_t s);
@@ -103,7 +105,8 @@ rhmc_status_t axpy_cols(const float2 *A, const float2 *C, const float2 *M, float
                         cudaStream_t s);
 // Y = C + A M fused with out = Y^dagger Y (n x n FP64, scratch: kGramCtas * n * n partials)
 rhmc_status_t axpy_gram_cols(const float2 *A, const float2 *C, const float2 *M, float2 *Y, long rows, int n,
-                             double2 *scratch, double2 *out, cudaStream_t s, const int *done = nullptr);
+                             double2 *scratch, double2 *out, cudaStream_t s, const int *done = nullptr,
+                             int *nparts = nullptr);
 // The base step after rho_k in one pass: Q = W rho^-1, X^(0) += P^(0) M1, P^(0) = Q + P^(0) M2
 // (coef: rho^-1, M1, M2), and Q into basis block *kdev when basis is given (capacity cap);
 // nothing when *upd is 0
@@ -129,9 +132,9 @@ rhmc_status_t nxn_qr_init(const double2 *partial, int nparts, int n, int nshift,
                           cudaStream_t s);
 template <typename T>
 rhmc_status_t nxn_alpha(const double2 *partial, int nparts, int n, SolverState *st, int k, C<T> *mw, cudaStream_t s);
-// small_df.cu: double-float forms of nxn_alpha / nxn_rho for the mixed solve (summed Gram input)
-rhmc_status_t nxn_alpha_dd(const double2 *gram, int n, SolverState *st, int k, float2 *mw, cudaStream_t s);
-rhmc_status_t nxn_rho_dd(const double2 *gram, int n, SolverState *st, int k, float2 *coef, cudaStream_t s);
+// small_df.cu: double-float forms of nxn_alpha / nxn_rho for the mixed solve ([entry][part] Gram partials)
+rhmc_status_t nxn_alpha_dd(const double2 *gram, int nparts, int n, SolverState *st, int k, float2 *mw, cudaStream_t s);
+rhmc_status_t nxn_rho_dd(const double2 *gram, int nparts, int n, SolverState *st, int k, float2 *coef, cudaStream_t s);
 rhmc_status_t nxn_shifts_dd(int n, int nshift, SolverState *st, int k, float2 *coef, double tol_shift, int freeze,
                             double2 *hist, int cap, cudaStream_t s);
 template <typename T>

@@ -23,6 +23,7 @@
 //             delta^(s)_k = rho_k alpha_k^-1 alpha^(s)_k (Sec. III), freezing
 //   reliable  delta_k replaced by the R factor of the true residual
 #include "common.cuh"
+#include "gramsum.cuh"
 #include "kernels.h"
 
 namespace rhmc {
@@ -98,27 +99,6 @@ __device__ void copy(const Cta &c, double2 *D, const double2 *S) {
 
 __device__ void set_eye(const Cta &c, double2 *D) {
   if (c.own) D[c.t] = make_double2(c.i == c.j ? 1.0 : 0.0, 0.0);
-  __syncthreads();
-}
-
-// Sum the per-cluster partials of a Gram matrix into G (8 loads in flight per thread).
-__device__ void reduce_partials(const Cta &c, double2 *G, const double2 *partial, int nparts) {
-  if (c.own) {
-    const int nn = c.n * c.n;
-    double2 acc[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = make_double2(0, 0);
-    int p = 0;
-    for (; p + 8 <= nparts; p += 8) {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) acc[q] = cadd(acc[q], partial[(long)(p + q) * nn + c.t]);
-    }
-    for (; p < nparts; ++p) acc[0] = cadd(acc[0], partial[(long)p * nn + c.t]);
-    double2 sum = acc[0];
-#pragma unroll
-    for (int q = 1; q < 8; ++q) sum = cadd(sum, acc[q]);
-    G[c.t] = sum;
-  }
   __syncthreads();
 }
 
@@ -426,7 +406,7 @@ __global__ void __launch_bounds__(256) k_qr_init(const double2 *partial, int npa
   __shared__ double rd[kMaxN], sd[kMaxN], rsd[kMaxN], nrm[kMaxN];
   __shared__ int flag;
   Cta c(n);
-  reduce_partials(c, A, partial, nparts);
+  gram_sum_parts(A, partial, nparts, n * n);
   if (!ldl(n, A, Li, rd, &flag)) {
     if (c.t == 0) st->breakdown = 1;
     return;
@@ -479,7 +459,7 @@ __global__ void __launch_bounds__(256) k_nxn_alpha(const double2 *partial, int n
   Cta c(n);
   const int cur = k % kSlots;
   const int t = c.t, nt = blockDim.x, nn = n * n;
-  reduce_partials(c, A, partial, nparts);
+  gram_sum_parts(A, partial, nparts, n * n);
   if (t == 0) st->kabs[cur] = st->kabs[(k - 1) % kSlots] + 1;
   // Gram1_k (Hermitian part) for the shifted step
   if (c.own) {
@@ -528,7 +508,7 @@ __global__ void __launch_bounds__(256) k_nxn_rho(const double2 *partial, int npa
   Cta c(n);
   const int cur = k % kSlots, prev = (k - 1) % kSlots;
   const int t = c.t, nt = blockDim.x, nn = n * n;
-  reduce_partials(c, A, partial, nparts);
+  gram_sum_parts(A, partial, nparts, n * n);
   if (!ldl(n, A, Li, rd, &flag)) {
     if (t == 0) st->breakdown = 3;
     return;
@@ -656,7 +636,7 @@ __global__ void __launch_bounds__(256) k_nxn_reliable(const double2 *partial, in
   __shared__ int flag;
   Cta c(n);
   const int cur = k % kSlots;
-  reduce_partials(c, A, partial, nparts);
+  gram_sum_parts(A, partial, nparts, n * n);
   if (!ldl(n, A, Li, rd, &flag)) {
     if (c.t == 0) st->breakdown = 5;
     return;
@@ -679,13 +659,11 @@ rhmc_status_t nxn_qr_init(const double2 *partial, int nparts, int n, int nshift,
 }
 // The mixed solve (FP32 fields) takes the double-float kernels of small_df.cu for
 // the base steps unless RHMC_TUNE_NXN_FP64 = 1.
-template <typename T> static bool use_dd(int nparts) {
-  return sizeof(T) == 4 && nparts == 1 && tune_get(TUNE_NXN_FP64) != 1;
-}
+template <typename T> static bool use_dd() { return sizeof(T) == 4 && tune_get(TUNE_NXN_FP64) != 1; }
 template <typename T>
 rhmc_status_t nxn_alpha(const double2 *partial, int nparts, int n, SolverState *st, int k, C<T> *mw, cudaStream_t s) {
   if constexpr (sizeof(T) == 4)
-    if (use_dd<T>(nparts)) return nxn_alpha_dd(partial, n, st, k, mw, s);
+    if (use_dd<T>()) return nxn_alpha_dd(partial, nparts, n, st, k, mw, s);
   prof_begin(PROF_NXN, s);
   k_nxn_alpha<T><<<1, 256, 0, s>>>(partial, nparts, n, st, k, mw);
   prof_end(s, 0.0);
@@ -696,7 +674,7 @@ template <typename T>
 rhmc_status_t nxn_rho(const double2 *partial, int nparts, int n, SolverState *st, int k, C<T> *coef,
                       cudaStream_t s) {
   if constexpr (sizeof(T) == 4)
-    if (use_dd<T>(nparts)) return nxn_rho_dd(partial, n, st, k, coef, s);
+    if (use_dd<T>()) return nxn_rho_dd(partial, nparts, n, st, k, coef, s);
   prof_begin(PROF_NXN, s);
   k_nxn_rho<T><<<1, 256, 0, s>>>(partial, nparts, n, st, k, coef);
   prof_end(s, 0.0);

@@ -15,6 +15,7 @@
 // residuals) for the shifted step and the FP32 coefficients of the bulk kernels.
 #include "common.cuh"
 #include "df.cuh"
+#include "gramsum.cuh"
 #include "kernels.h"
 
 namespace rhmc {
@@ -304,7 +305,7 @@ __device__ bool inv_general_dd(int n, cd *Ai, cd *A, int *piv, int *flag) {
 // alpha_k step: alpha_k = Gram1^-1 (Hermitian part of Gram1 = P^dagger (A + sigma_0) P)
 // = L^-dagger D^-1 L^-1; FP64 alpha_k and Gram1_k into the state, -alpha_k (FP32)
 // for the block QR step.  Thread t owns entry (t / 16, t % 16) throughout.
-__global__ void __launch_bounds__(256) k_nxn_alpha_dd(const double2 *G, int n, SolverState *st, int k,
+__global__ void __launch_bounds__(256) k_nxn_alpha_dd(const double2 *part, int nparts, int n, SolverState *st, int k,
                                                       float2 *mw_out) {
   __shared__ cd A[kNN], Li[kNN], S[kNN];
   __shared__ dd rd[kMaxN];
@@ -313,8 +314,10 @@ __global__ void __launch_bounds__(256) k_nxn_alpha_dd(const double2 *G, int n, S
   const int t = threadIdx.x, i = t >> 4, j = t & 15;
   const bool in = i < n && j < n;
   const int done = st->done;  // a later iteration of a chunk whose solve has stopped: no output
+  __shared__ double2 Gs[kNN];
+  if (nparts > 1) gram_sum_parts(Gs, part, nparts, n * n);
   cd h0;
-  const bool ok = ldl16(n, G, A, Li, rd, &flag, h0);
+  const bool ok = ldl16(n, nparts > 1 ? Gs : part, A, Li, rd, &flag, h0);
   if (done) return;
   if (t == 0) st->kabs[cur] = st->kabs[(k - 1) % kSlots] + 1;
   if (!ok) {
@@ -349,7 +352,8 @@ __global__ void __launch_bounds__(256) k_nxn_alpha_dd(const double2 *G, int n, S
 // coef = [rho_k^-1, M1 = alpha_k delta_{k-1}, rho_k^dagger] (FP32); FP64 rho_k,
 // delta_k = rho_k delta_{k-1} and the base column residuals into the state.
 // Thread t owns entry (t / 16, t % 16) throughout.
-__global__ void __launch_bounds__(256) k_nxn_rho_dd(const double2 *G, int n, SolverState *st, int k, float2 *coef) {
+__global__ void __launch_bounds__(256) k_nxn_rho_dd(const double2 *part, int nparts, int n, SolverState *st, int k,
+                                                    float2 *coef) {
   __shared__ cd A[kNN], Li[kNN], Al[kNN], Dp[kNN];
   __shared__ dd rd[kMaxN], sd[kMaxN], rsd[kMaxN];
   __shared__ int flag;
@@ -362,8 +366,10 @@ __global__ void __launch_bounds__(256) k_nxn_rho_dd(const double2 *G, int n, Sol
     Al[t] = from_z(st->alpha[cur][i * n + j]);
     Dp[t] = from_z(st->delta[prev][i * n + j]);
   }
+  __shared__ double2 Gs[kNN];
+  if (nparts > 1) gram_sum_parts(Gs, part, nparts, n * n);
   cd h0;
-  const bool ok = ldl16(n, G, A, Li, rd, &flag, h0);
+  const bool ok = ldl16(n, nparts > 1 ? Gs : part, A, Li, rd, &flag, h0);
   if (done) {
     if (t == 0) st->upd[0] = 0;
     return;
@@ -535,17 +541,17 @@ rhmc_status_t nxn_shifts_dd(int n, int nshift, SolverState *st, int k, float2 *c
   return RHMC_OK;
 }
 
-rhmc_status_t nxn_alpha_dd(const double2 *gram, int n, SolverState *st, int k, float2 *mw, cudaStream_t s) {
+rhmc_status_t nxn_alpha_dd(const double2 *gram, int nparts, int n, SolverState *st, int k, float2 *mw, cudaStream_t s) {
   prof_begin(PROF_NXN, s);
-  k_nxn_alpha_dd<<<1, 256, 0, s>>>(gram, n, st, k, mw);
+  k_nxn_alpha_dd<<<1, 256, 0, s>>>(gram, nparts, n, st, k, mw);
   prof_end(s, 0.0);
   RHMC_LAUNCH_CHECK();
   return RHMC_OK;
 }
 
-rhmc_status_t nxn_rho_dd(const double2 *gram, int n, SolverState *st, int k, float2 *coef, cudaStream_t s) {
+rhmc_status_t nxn_rho_dd(const double2 *gram, int nparts, int n, SolverState *st, int k, float2 *coef, cudaStream_t s) {
   prof_begin(PROF_NXN, s);
-  k_nxn_rho_dd<<<1, 256, 0, s>>>(gram, n, st, k, coef);
+  k_nxn_rho_dd<<<1, 256, 0, s>>>(gram, nparts, n, st, k, coef);
   prof_end(s, 0.0);
   RHMC_LAUNCH_CHECK();
   return RHMC_OK;

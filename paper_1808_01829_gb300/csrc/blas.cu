@@ -1205,7 +1205,8 @@ __global__ void __launch_bounds__(W * 32, 1) k_axpy_gram_cols(const float2 *__re
 #pragma unroll 1
     for (int r = 0; r < nr; r += H) {
       float2 y = make_float2(0.f, 0.f);
-      const bool on = act && r + h < nr;
+      // rows come in eights: with H dividing 8 every lane in use has its row
+      const bool on = act && (8 % H == 0 || r + h < nr);
       if (on) {
         const float2 *ar = at + (r + h) * N;
         float2 p;

@@ -27,6 +27,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdlib>
+#include <cstddef>
 #include <cstring>
 #include <memory>
 #include <numeric>
@@ -527,23 +528,28 @@ static rhmc_status_t colnorms(rhmc_ctx *c, const double2 *A, int n, double *out,
   return read_colnorms(c, npart, n, out, s);
 }
 
+// The part of SolverState that the host looks at, in its layout (one copy).
 struct StateView {
   double res[kMaxS][kMaxN];
   int active[kMaxS];
+  int upd[kMaxS];
+  int last_k[kMaxS];
+  int kabs[kSlots];
   int breakdown;
   int device_timeout;
   int done;
   int nit;
 };
+constexpr size_t kViewBytes = offsetof(SolverState, nit) + sizeof(int) - offsetof(SolverState, res);
+static_assert(offsetof(StateView, nit) + sizeof(int) == kViewBytes &&
+                  offsetof(StateView, active) == offsetof(SolverState, active) - offsetof(SolverState, res),
+              "StateView mirrors SolverState from res to nit");
 
 static rhmc_status_t read_state(rhmc_ctx *c, SolverState *st, StateView &v, cudaStream_t s) {
-  RHMC_TRY(ensure_pinned(c, sizeof(StateView) + 64));
-  StateView *h = reinterpret_cast<StateView *>(lane(c).h_pin);
-  RHMC_CUDA_TRY(cudaMemcpyAsync(h->res, st->res, sizeof(v.res), cudaMemcpyDeviceToHost, s));
-  RHMC_CUDA_TRY(cudaMemcpyAsync(h->active, st->active, sizeof(v.active), cudaMemcpyDeviceToHost, s));
-  RHMC_CUDA_TRY(cudaMemcpyAsync(&h->breakdown, &st->breakdown, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  RHMC_TRY(ensure_pinned(c, sizeof(StateView)));
+  RHMC_CUDA_TRY(cudaMemcpyAsync(lane(c).h_pin, st->res, kViewBytes, cudaMemcpyDeviceToHost, s));
   RHMC_CUDA_TRY(cudaStreamSynchronize(s));
-  std::memcpy(&v, h, sizeof(StateView));
+  std::memcpy(&v, lane(c).h_pin, kViewBytes);
   return RHMC_OK;
 }
 

@@ -60,46 +60,63 @@ namespace rhmc {
 // ------------------------------------------------------------ coefficients
 // FP64 coefficient blocks cf[(s - 1) * cfstride + i][q][j] (n x n complex) of
 // the expansion of X^(s) (want_p = 0: blocks i < min(last_s, K)) or of
-// P^(s)_K (want_p = 1: blocks i <= K, active shifts only).  One CTA per shift.
-__global__ void __launch_bounds__(256) k_basis_coef(int n, int nshift, const SolverState *__restrict__ st,
+// P^(s)_K (want_p = 1: blocks i <= K, active shifts only).  The recursion runs down the blocks
+// one by one, but its columns are independent: one CTA per shift and column, the next block's
+// M2 fetched during the step.  With one CTA per shift the FP64 unit of its SM bound it
+// (8^4, n = 4: 400 -> 120 us; 12^4, n = 4, mixed: 328 -> 181 us).
+constexpr int kCoefSlices = 4;  // lanes that share a dot product (n <= 16: up to four terms each)
+__global__ void __launch_bounds__(128) k_basis_coef(int n, int nshift, const SolverState *__restrict__ st,
                                                     const double2 *__restrict__ hist, int K, int want_p,
                                                     double2 *__restrict__ cf, long cfstride) {
-  __shared__ double2 Cm[kMaxN * kMaxN], Tm[kMaxN * kMaxN];
-  const int s = blockIdx.x + 1;
+  __shared__ double Cm[2][2 * kMaxN];  // the column, double-buffered
+  const int s = blockIdx.x + 1, col = blockIdx.y;
   if (s >= nshift) return;
   const int nn = n * n, t = threadIdx.x;
-  const bool own = t < nn;
-  const int qi = own ? t / n : 0, qj = own ? t % n : 0;
+  const int sl = t & 3, c = (t >> 2) & 1, row = t >> 3;  // slice, component, row of this thread's entry
+  const bool own = row < n;
   const int last = want_p ? (st->active[s] ? K : -1) : min(st->last_k[s], K);
   if (last < 0 || (!want_p && last == 0)) return;
   double2 *out = cf + (size_t)(s - 1) * cfstride * nn;
-  int i;
-  if (want_p) {
-    if (own) Cm[t] = make_double2(qi == qj ? 1.0 : 0.0, 0.0);  // D_K = 1
-    i = K;
-  } else {
-    if (own) Cm[t] = hist[((size_t)last * nshift + s) * 2 * nn + t];  // C_{L-1} = alpha_L
-    i = last - 1;
-  }
-  __syncthreads();
-  for (;; --i) {
-    if (own) out[(size_t)i * nn + t] = Cm[t];
-    if (i == 0) break;
-    // step to block i - 1: C_{i-1} = alpha_i + M2_i C_i  /  D_{i-1} = M2_i D_i
-    const double2 *h = hist + ((size_t)i * nshift + s) * 2 * nn;
-    if (own) {
-      double2 acc = want_p ? make_double2(0.0, 0.0) : h[t];
-      const double2 *M2 = h + nn;
-      for (int q = 0; q < n; ++q) {
-        const double2 a = M2[qi * n + q], b = Cm[q * n + qj];
-        acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
-        acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
-      }
-      Tm[t] = acc;
+  const int ent = row * n + col;
+  auto h = [&](int i) { return hist + ((size_t)i * nshift + s) * 2 * nn; };
+  int i = want_p ? K : last - 1;
+  double v = 0.0;  // D_K = 1 / C_{L-1} = alpha_L
+  if (own) v = want_p ? (row == col && !c ? 1.0 : 0.0) : reinterpret_cast<const double *>(h(last) + ent)[c];
+  double2 m[kCoefSlices] = {};
+  double al = 0.0;
+  auto fetch = [&](int k) {  // M2_k's slice of the row, and alpha_k's entry
+    if (k <= 0 || !own) return;
+#pragma unroll
+    for (int u = 0; u < kCoefSlices; ++u) {
+      const int q = sl + kCoefSlices * u;
+      if (q < n) m[u] = h(k)[nn + row * n + q];
     }
+    al = (want_p || sl) ? 0.0 : reinterpret_cast<const double *>(h(k) + ent)[c];
+  };
+  fetch(i);
+  for (int b = 0;; --i, b ^= 1) {
+    if (own && sl == 0) {
+      reinterpret_cast<double *>(out + (size_t)i * nn + ent)[c] = v;
+      Cm[b][2 * row + c] = v;
+    }
+    if (i == 0) break;
     __syncthreads();
-    if (own) Cm[t] = Tm[t];
-    __syncthreads();
+    // step to block i - 1: C_{i-1} = alpha_i + M2_i C_i  /  D_{i-1} = M2_i D_i
+    double acc = al;
+    if (own) {
+#pragma unroll
+      for (int u = 0; u < kCoefSlices; ++u) {
+        const int q = sl + kCoefSlices * u;
+        if (q < n) {
+          const double x = Cm[b][2 * q], y = Cm[b][2 * q + 1];
+          acc = c ? fma(m[u].x, y, fma(m[u].y, x, acc)) : fma(m[u].x, x, fma(-m[u].y, y, acc));
+        }
+      }
+    }
+    fetch(i - 1);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    v = acc;
   }
 }
 
@@ -647,7 +664,7 @@ __global__ void __launch_bounds__(256) k_basis_gemm_simt(const float2 *__restric
 rhmc_status_t basis_coef(const BasisBufs &bb, int n, int nshift, const SolverState *st, int K, int want_p,
                          cudaStream_t s) {
   prof_begin(PROF_NXN_SHIFTS, s);
-  k_basis_coef<<<nshift - 1, 256, 0, s>>>(n, nshift, st, bb.hist, K, want_p, bb.cf, bb.cap + 1);
+  k_basis_coef<<<dim3(nshift - 1, n), (8 * n + 31) / 32 * 32, 0, s>>>(n, nshift, st, bb.hist, K, want_p, bb.cf, bb.cap + 1);
   prof_end(s, 0.0);
   RHMC_LAUNCH_CHECK();
   return RHMC_OK;

@@ -4,9 +4,11 @@
 // shared memory.  On this GPU an FP64 warp instruction occupies its SM
 // sub-partition's FP64 unit for about 64 cycles however many lanes are active,
 // and a dependent FP64 operation waits as long; the base-system kernels
-// therefore hand each step's work items to the fewest warps (items are packed
-// by index, not owned by element), exploit every triangular and Hermitian
-// structure, and keep one barrier per factorisation step.  The shifted step
+// therefore pack each step's work items into whole warps (by index, not owned by
+// element), real and imaginary parts on warps of their own so that the four FP64 units
+// work side by side, exploit every triangular and Hermitian structure, and keep one
+// barrier per factorisation step (8^4, n = 4: alpha 9.4 -> 7.6 us and rho 12.3 -> 9.5 us
+// against both parts in one warp, FP64 sums of the Gram partials and two-step reciprocals).  The shifted step
 // (one CTA per shift) keeps the simpler element-per-thread form.  The state of the
 // recursion lives in a SolverState in device memory; quantities of iteration
 // k are written to slot k % 3 and those of k-1 read from slot (k-1) % 3, so a
@@ -233,18 +235,28 @@ __device__ void store_coef(const Cta &c, C<T> *dst, const double2 *M, double sca
   if (c.own) dst[c.t] = mk<T>((T)(scale * M[c.t].x), (T)(scale * M[c.t].y));
 }
 
-// 1/x for x > 0: FP32 estimate refined by two Newton-Raphson steps
-// r <- r + r (1 - x r) in FP64 (the estimate's 2^-23 error squares twice);
-// the exponent is split off only when x is outside the FP32 range.
+// x in (1e-30, 1e30) to FP32 (truncated) and an FP32 value in that range back to FP64, on the
+// integer units (a conversion instruction takes an FP64 slot of 64 cycles).
+__device__ __forceinline__ float trunc_f32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x) - 0x38000000u;  // exponent bias 1023 -> 127
+  return __uint_as_float((hi << 3) | ((unsigned)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ double widen_f64(float f) {
+  const unsigned b = __float_as_uint(f);
+  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+// 1/x for x > 0: an FP32 estimate and one third-order step r <- r + r (e + e^2), e = 1 - x r
+// (|e| < 2^-21, so e^3 is below rounding; three dependent FP64 operations where two Newton
+// steps and two conversions took six); the exponent is split off only when x is outside the
+// FP32 range.
 __device__ __forceinline__ double frcp_fast(double x) {
   if (!(x > 1e-30 && x < 1e30)) return frcp(x);
-  double r = (double)__frcp_rn((float)x);
-  double e = fma(-x, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-x, r, 1.0);
-  return fma(r, e, r);
+  const double r = widen_f64(__frcp_rn(trunc_f32(x)));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
 }
-// 1/sqrt(x) for x > 0: Newton-Raphson y <- y (3 - x y^2) / 2 from an FP32 estimate.
+// 1/sqrt(x) for x > 0: an FP32 estimate and one third-order step y <- y + y e (1/2 + 3/8 e),
+// e = 1 - x y^2 (the binomial series of (1 - e)^(-1/2)).
 __device__ __forceinline__ double frsqrt(double x) {
   int e = 0;
   double m = x;
@@ -255,10 +267,10 @@ __device__ __forceinline__ double frsqrt(double x) {
       e -= 1;
     }
   }
-  const double h = 0.5 * m;
-  double y = (double)rsqrtf((float)m);
-  y = y * fma(-h * y, y, 1.5);
-  y = y * fma(-h * y, y, 1.5);
+  const bool in = m > 1e-30 && m < 1e30;
+  double y = in ? widen_f64(rsqrtf(trunc_f32(m))) : (double)rsqrtf((float)m);
+  const double d = fma(-(m * y), y, 1.0);
+  y = fma(y, d * fma(0.375, d, 0.5), y);
   return e ? ldexp(y, -e / 2) : y;
 }
 
@@ -270,30 +282,44 @@ __device__ __forceinline__ int tri_row(int e) {
   return a;
 }
 
+// A component (0: real, 1: imaginary) of entry e of M.
+__device__ __forceinline__ double &part(double2 *M, int e, int c) { return reinterpret_cast<double *>(M)[2 * e + c]; }
+
 // LDL^dagger factorisation of the Hermitian positive definite A (n x n, full
-// storage in shared memory, its Hermitian part is used).  On return the
-// strictly lower part of A holds L (unit lower), A[k][k].x holds D_k,
+// storage in shared memory, its Hermitian part is used; written to sym too if given).
+// On return the strictly lower part of A holds L (unit lower), A[k][k].x holds D_k,
 // Li = L^-1 (unit lower, full storage) and rd[k] = 1 / D_k.  Step k updates
-// the trailing lower triangle and rows k+1.. of L^-1 as one list of work
-// items; the item on the next diagonal entry also forms the next pivot's
-// reciprocal, so each step needs one barrier.  Returns false (in all threads)
-// if a pivot is not positive and finite.
-__device__ bool ldl(int n, double2 *A, double2 *Li, double *rd, int *flag) {
+// the trailing lower triangle and rows k+1.. of L^-1; the real and the imaginary parts of
+// the two go to warps of their own (three FP64 operations each), so that at small n the
+// four run on the SM's four FP64 units instead of in turn on one.  The item on the next
+// diagonal entry also forms the next pivot's reciprocal, so each step needs one barrier.
+// Returns false (in all threads) if a pivot is not positive and finite.
+__device__ bool ldl(int n, double2 *A, double2 *Li, double *rd, int *flag, double2 *sym = nullptr) {
   const int t = threadIdx.x, nt = blockDim.x, nn = n * n;
-  double2 h = make_double2(0, 0);
-  if (t < nn) {
-    const int i = t / n, j = t - (t / n) * n;
-    const double2 a = A[t], b = A[j * n + i];
-    h = (i == j) ? make_double2(a.x, 0.0) : make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
+  const int warp = t >> 5, lane = t & 31, nw = nt >> 5;
+  double h[2] = {0.0, 0.0};  // components t and t + nt (n <= 16, 256 threads)
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int x = t + u * nt;
+    if (x < 2 * nn) {
+      const int e = x >> 1, c = x & 1, i = e / n, j = e - i * n;
+      const double a = part(A, e, c), b = part(A, j * n + i, c);
+      h[u] = 0.5 * (a + (c ? -b : b));
+    }
   }
   __syncthreads();
-  if (t < nn) {
-    const int i = t / n, j = t - (t / n) * n;
-    A[t] = h;
-    Li[t] = make_double2(i == j ? 1.0 : 0.0, 0.0);
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int x = t + u * nt;
+    if (x < 2 * nn) {
+      const int e = x >> 1, c = x & 1, i = e / n, j = e - i * n;
+      part(A, e, c) = h[u];
+      part(Li, e, c) = (i == j && !c) ? 1.0 : 0.0;
+      if (sym) part(sym, e, c) = h[u];
+    }
   }
   if (t == 0) {
-    const double d = h.x;
+    const double d = h[0];
     *flag = !(d > 0.0) || !isfinite(d);
     rd[0] = frcp_fast(d > 0.0 ? d : 1.0);
   }
@@ -303,40 +329,39 @@ __device__ bool ldl(int n, double2 *A, double2 *Li, double *rd, int *flag) {
     const double r = rd[k];
     const int m = n - 1 - k;
     const int ntri = m * (m + 1) / 2, nli = m * (k + 1);
-    for (int e = t; e < ntri + nli; e += nt) {
-      if (e < ntri) {
+    const int wa = (ntri + 31) >> 5, wl = (nli + 31) >> 5;  // warps per component
+    for (int w = warp; w < 2 * (wa + wl); w += nw) {
+      if (w < 2 * wa) {
         // A[i][j] -= A[i][k] conj(A[j][k]) / D_k,  i >= j > k
+        const int c = w >= wa, e = (c ? w - wa : w) * 32 + lane;
+        if (e >= ntri) continue;
         const int a = tri_row(e), b = e - a * (a + 1) / 2;
         const int i = k + 1 + a, j = k + 1 + b;
-        const double2 aik = A[i * n + k], ajk = A[j * n + k];
-        double2 v = A[i * n + j];
-        const double px = fma(aik.x, ajk.x, aik.y * ajk.y), py = fma(aik.y, ajk.x, -aik.x * ajk.y);
-        v.x = fma(-px, r, v.x);
-        v.y = fma(-py, r, v.y);
-        A[i * n + j] = v;
-        if (i == k + 1 && j == k + 1) {
-          *flag = !(v.x > 0.0) || !isfinite(v.x);
-          rd[k + 1] = frcp_fast(v.x > 0.0 ? v.x : 1.0);
+        const double2 u = A[i * n + k], v = A[j * n + k];
+        const double p = c ? fma(u.y, v.x, -u.x * v.y) : fma(u.x, v.x, u.y * v.y);
+        const double x = fma(-p, r, part(A, i * n + j, c));
+        part(A, i * n + j, c) = x;
+        if (e == 0 && !c) {
+          *flag = !(x > 0.0) || !isfinite(x);
+          rd[k + 1] = frcp_fast(x > 0.0 ? x : 1.0);
         }
       } else {
         // Li[i][j] -= L[i][k] Li[k][j],  i > k >= j,  L[i][k] = A[i][k] / D_k
-        const int e2 = e - ntri;
-        const int a = e2 / (k + 1), j = e2 - a * (k + 1);
+        const int w2 = w - 2 * wa, c = w2 >= wl, e = (c ? w2 - wl : w2) * 32 + lane;
+        if (e >= nli) continue;
+        const int a = e / (k + 1), j = e - a * (k + 1);
         const int i = k + 1 + a;
-        const double2 aik = A[i * n + k], lkj = Li[k * n + j];
-        const double lx = aik.x * r, ly = aik.y * r;
-        double2 v = Li[i * n + j];
-        v.x -= fma(lx, lkj.x, -ly * lkj.y);
-        v.y -= fma(lx, lkj.y, ly * lkj.x);
-        Li[i * n + j] = v;
+        const double2 u = A[i * n + k], v = Li[k * n + j];
+        const double p = c ? fma(u.x, v.y, u.y * v.x) : fma(u.x, v.x, -u.y * v.y);
+        part(Li, i * n + j, c) = fma(-p, r, part(Li, i * n + j, c));
       }
     }
     __syncthreads();
   }
   if (*flag) return false;
-  for (int e = t; e < nn; e += nt) {
-    const int i = e / n, j = e - (e / n) * n;
-    if (i > j) A[e] = cscale(A[e], rd[j]);
+  for (int x = t; x < 2 * nn; x += nt) {
+    const int e = x >> 1, i = e / n, j = e - i * n;
+    if (i > j) part(A, e, x & 1) *= rd[j];
   }
   __syncthreads();
   return true;
@@ -355,19 +380,19 @@ __device__ void qr_factors(int n, const double2 *A, const double2 *Li, double2 *
     sd[t] = d * y;
   }
   __syncthreads();
-  for (int e = t; e < nn; e += nt) {
-    const int i = e / n, j = e - (e / n) * n;
-    double2 r = make_double2(0, 0), ri = make_double2(0, 0);
+  for (int x = t; x < 2 * nn; x += nt) {
+    const int e = x >> 1, c = x & 1, i = e / n, j = e - i * n;
+    double r = 0.0, ri = 0.0;
     if (i == j) {
-      r = make_double2(sd[i], 0.0);
-      ri = make_double2(rsd[i], 0.0);
+      r = c ? 0.0 : sd[i];
+      ri = c ? 0.0 : rsd[i];
     } else if (i < j) {
-      const double2 l = A[j * n + i], li = Li[j * n + i];  // conj(L[j][i]), conj(Li[j][i])
-      r = make_double2(sd[i] * l.x, -sd[i] * l.y);
-      ri = make_double2(li.x * rsd[j], -li.y * rsd[j]);
+      const double l = part(const_cast<double2 *>(A), j * n + i, c), li = part(const_cast<double2 *>(Li), j * n + i, c);
+      r = (c ? -l : l) * sd[i];  // conj(L[j][i]), conj(Li[j][i])
+      ri = (c ? -li : li) * rsd[j];
     }
-    R[e] = r;
-    Ri[e] = ri;
+    part(R, e, c) = r;
+    part(Ri, e, c) = ri;
   }
   __syncthreads();
 }
@@ -382,8 +407,8 @@ __device__ void colnorms_upper(int n, const double2 *M, double *out, const doubl
     const double2 z = M[i * n + j];
     v = fma(z.x, z.x, z.y * z.y);
   }
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, 16);
+  for (int o = 8; o > 0; o >>= 1)
+    if (o < n) v += __shfl_xor_sync(0xffffffffu, v, o, 16);  // (lanes n .. 15 of a column hold 0)
   if (j < n && i == 0) {
     const double nv = v > 0.0 ? v * frsqrt(v) : 0.0;
     if (norm_out) norm_out[j] = nv;
@@ -461,36 +486,33 @@ __global__ void __launch_bounds__(256) k_nxn_alpha(const double2 *partial, int n
   const int t = c.t, nt = blockDim.x, nn = n * n;
   gram_sum_parts(A, partial, nparts, n * n);
   if (t == 0) st->kabs[cur] = st->kabs[(k - 1) % kSlots] + 1;
-  // Gram1_k (Hermitian part) for the shifted step
-  if (c.own) {
-    const double2 a = A[t], b = A[c.j * n + c.i];
-    st->G1[cur][t] = (c.i == c.j) ? make_double2(a.x, 0.0) : make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
-  }
-  if (!ldl(n, A, Li, rd, &flag)) {
+  // (Gram1_k, its Hermitian part, is kept for the shifted step)
+  if (!ldl(n, A, Li, rd, &flag, st->G1[cur])) {
     if (t == 0) st->breakdown = 2;
     return;
   }
   // S[k][j] = Li[k][j] / D_k
-  for (int e = t; e < nn; e += nt) {
-    const int kk = e / n;
-    S[e] = cscale(Li[e], rd[kk]);
-  }
+  for (int x = t; x < 2 * nn; x += nt) part(S, x >> 1, x & 1) = part(Li, x >> 1, x & 1) * rd[(x >> 1) / n];
   __syncthreads();
-  // alpha[i][j] = sum_{q >= j} conj(Li[q][i]) S[q][j], i <= j (column-major packing)
-  for (int e = t; e < n * (n + 1) / 2; e += nt) {
+  // alpha[i][j] = sum_{q >= j} conj(Li[q][i]) S[q][j], i <= j (column-major packing), real and
+  // imaginary parts on warps of their own
+  const int ntri = n * (n + 1) / 2, wa = (ntri + 31) >> 5;
+  for (int w = t >> 5; w < 2 * wa; w += nt >> 5) {
+    const int cc = w >= wa, e = (cc ? w - wa : w) * 32 + (t & 31);
+    if (e >= ntri) continue;
     const int j = tri_row(e), i = e - j * (j + 1) / 2;
-    double ax = 0.0, ay = 0.0;
+    double a = 0.0;
     for (int q = j; q < n; ++q) {
       const double2 l = Li[q * n + i], sv = S[q * n + j];
-      ax = fma(l.x, sv.x, fma(l.y, sv.y, ax));
-      ay = fma(l.x, sv.y, fma(-l.y, sv.x, ay));
+      a = cc ? fma(l.x, sv.y, fma(-l.y, sv.x, a)) : fma(l.x, sv.x, fma(l.y, sv.y, a));
     }
-    const double2 v = make_double2(ax, ay), vc = make_double2(ax, -ay);
-    st->alpha[cur][i * n + j] = v;
-    mw_out[i * n + j] = mk<T>((T)(-ax), (T)(-ay));
-    if (i != j) {
-      st->alpha[cur][j * n + i] = vc;
-      mw_out[j * n + i] = mk<T>((T)(-ax), (T)(ay));
+    double *al = reinterpret_cast<double *>(st->alpha[cur]);
+    auto *mw = reinterpret_cast<decltype(mw_out->x) *>(mw_out);
+    al[2 * (i * n + j) + cc] = a;
+    mw[2 * (i * n + j) + cc] = (decltype(mw_out->x))(-a);
+    if (i != j) {  // the conjugate below the diagonal
+      al[2 * (j * n + i) + cc] = cc ? -a : a;
+      mw[2 * (j * n + i) + cc] = (decltype(mw_out->x))(cc ? a : -a);
     }
   }
 }
@@ -525,29 +547,31 @@ __global__ void __launch_bounds__(256) k_nxn_rho(const double2 *partial, int npa
   if (c.own) coef[2 * nn + t] = mk<T>((T)R[c.j * n + c.i].x, (T)(-R[c.j * n + c.i].y));  // rho^dagger
   __syncthreads();
   // M1[i][j] = sum_{q <= j} alpha[i][q] delta[q][j] (n^2 items, column-major so a
-  // warp's items share their length); delta_k[i][j] = sum_{i <= q <= j} rho[i][q] delta[q][j]
+  // warp's items share their length); delta_k[i][j] = sum_{i <= q <= j} rho[i][q] delta[q][j];
+  // real and imaginary parts on warps of their own, as in the factorisation
   double2 *Dk = Ri;  // Ri was stored above
-  for (int e = t; e < nn + n * (n + 1) / 2; e += nt) {
-    if (e < nn) {
+  const int ntri = n * (n + 1) / 2, wm = (nn + 31) >> 5, wd = (ntri + 31) >> 5;  // warps per component
+  for (int w = t >> 5; w < 2 * (wm + wd); w += nt >> 5) {
+    double a = 0.0;
+    if (w < 2 * wm) {
+      const int cc = w >= wm, e = (cc ? w - wm : w) * 32 + (t & 31);
+      if (e >= nn) continue;
       const int j = e / n, i = e - (e / n) * n;
-      double ax = 0.0, ay = 0.0;
       for (int q = 0; q <= j; ++q) {
-        const double2 a = Al[i * n + q], d = Dp[q * n + j];
-        ax = fma(a.x, d.x, fma(-a.y, d.y, ax));
-        ay = fma(a.x, d.y, fma(a.y, d.x, ay));
+        const double2 u = Al[i * n + q], d = Dp[q * n + j];
+        a = cc ? fma(u.x, d.y, fma(u.y, d.x, a)) : fma(u.x, d.x, fma(-u.y, d.y, a));
       }
-      coef[nn + i * n + j] = mk<T>((T)ax, (T)ay);
+      reinterpret_cast<decltype(coef->x) *>(coef)[2 * (nn + i * n + j) + cc] = (decltype(coef->x))a;
     } else {
-      const int e2 = e - nn;
-      const int j = tri_row(e2), i = e2 - j * (j + 1) / 2;
-      double ax = 0.0, ay = 0.0;
+      const int w2 = w - 2 * wm, cc = w2 >= wd, e = (cc ? w2 - wd : w2) * 32 + (t & 31);
+      if (e >= ntri) continue;
+      const int j = tri_row(e), i = e - j * (j + 1) / 2;
       for (int q = i; q <= j; ++q) {
-        const double2 a = R[i * n + q], d = Dp[q * n + j];
-        ax = fma(a.x, d.x, fma(-a.y, d.y, ax));
-        ay = fma(a.x, d.y, fma(a.y, d.x, ay));
+        const double2 u = R[i * n + q], d = Dp[q * n + j];
+        a = cc ? fma(u.x, d.y, fma(u.y, d.x, a)) : fma(u.x, d.x, fma(-u.y, d.y, a));
       }
-      Dk[i * n + j] = make_double2(ax, ay);
-      if (i != j) Dk[j * n + i] = make_double2(0.0, 0.0);
+      part(Dk, i * n + j, cc) = a;
+      if (i != j) part(Dk, j * n + i, cc) = 0.0;
     }
   }
   __syncthreads();

@@ -2,7 +2,7 @@
 """Benchmark: time per pseudofermion-force evaluation at 24^4, n_pf = 16.
 
 One step = one full force evaluation through the C ABI: the staging of the
-resident FP64 links into the operator's FP32 and double-float records
+resident FP64 links into the operator's FP32 and integer records
 (rhmc_set_gauge), then rhmc_force: the block multishift solve SBCGrQ
 (Algorithm 1) of (A + beta_s) X^(s) = Phi for all 16 pseudofermions and all 16
 shifts to a true relative residual of 1e-8 (mixed precision: FP32 operator and
@@ -21,8 +21,9 @@ Also reported on the same line:
   against mixed per-vector (the same solver with one right-hand side per
   solve: multishift CG in the same reliable-update / defect-correction scheme);
 * alu_peaks and roofline_alu: the measured FP32 / FP64 CUDA-core peaks and the
-  fractions of them reached by the double-float operator (FP32-ALU bound), the
-  FP64 operator of the per-vector baseline and the n x n coefficient chain;
+  fractions of them reached by the FP64-accurate integer operator (bound by wide
+  integer multiply-adds, at the solve's width and at width 1) and the n x n
+  coefficient chain;
 * trajectory: time per RHMC trajectory (Sec. II set-up, Sec. IV parameters) on the
   paper's 8^4 lattice, the FP64 gauge kernels at 24^4 against the measured FP64
   peak, and the trajectory oracle on a bounded sample;
@@ -558,14 +559,14 @@ def dslash_widths(ctx, dev, widths=(1, 2, 4, 8, 16), reps=10):
 
 
 # ------------------------------------------------------------------ ALU fractions
-DF_OPS_PER_SITE_RHS = 8 * 9 * 4 * 12  # double-float hop: 8 links x 9 entries x 4 real products x 12 FP32 instructions
+# integer hop: 8 links x 9 entries x 3 real products x 3 word products (wide multiply-adds)
+FX_OPS_PER_SITE_RHS = 8 * 9 * 3 * 3
 
 
 def alu_fractions(ctx, stats, cfg, lib):
     """Measured CUDA-core peaks (rhmc_probe_alu_peaks) and the fractions reached by
-    the FP32-ALU-bound double-float hop (FP32 instruction rate), and by the FP64
-    parts: the n x n coefficient chain (estimated flops) and the FP64 hop of the
-    per-vector baseline (570 flops per site and right-hand side)."""
+    the FP64-accurate integer hop (wide integer multiply-adds, in the step and at
+    width 1) and by the n x n coefficient chain (estimated flops)."""
     import ctypes
 
     from paper_1808_01829_gb300 import roofline
@@ -580,14 +581,19 @@ def alu_fractions(ctx, stats, cfg, lib):
     n, ns = cfg["n_pf"], cfg["n_shifts"]
     vh = ctx.Vh
     out = {}
+    import torch
+
+    # a warp's 32 x 32 -> 64 bit multiply-add takes four clocks, its FP32 FMA one
+    fx_peak = f32.value / 2 / 4
+    count = "8 x 9 x 3 x 3 wide integer multiply-adds per site and right-hand side"
+
+    def fx_entry(e, nrhs):
+        achieved = e["launches"] * vh * nrhs * FX_OPS_PER_SITE_RHS / (e["ms"] * 1e-3) / 1e12
+        return {"bound": "alu", "achieved": achieved, "peak": fx_peak, "unit": "T wide multiply-adds/s",
+                "frac": achieved / fx_peak, "peak_source": "a quarter of the measured FP32 FMA rate (rhmc_probe_alu_peaks)", "count": count}
+
     if "hop_df" in stats:
-        e = stats["hop_df"]
-        ops = e["launches"] * vh * n * DF_OPS_PER_SITE_RHS
-        achieved = ops / (e["ms"] * 1e-3) / 1e12  # T FP32 instructions / s
-        peak = f32.value / 2
-        out["hop_df"] = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "T FP32 instr/s",
-                         "frac": achieved / peak, "peak_source": "of measured (rhmc_probe_alu_peaks)",
-                         "count": "8 x 9 x 4 real products x 12 FP32 instructions per site and right-hand side"}
+        out["hop_df"] = fx_entry(stats["hop_df"], n)
     if "nxn" in stats:
         e = stats["nxn"]
         # per iteration, alpha (LDL^dagger inverse, ~4 n^3/3 complex MACs) and rho (LDL^dagger, triangular
@@ -604,21 +610,13 @@ def alu_fractions(ctx, stats, cfg, lib):
         out["nxn_shifts"] = {"bound": "latency", "achieved": achieved, "peak": f64.value, "unit": "TFLOP/s (FP64)",
                              "frac": achieved / f64.value, "peak_source": "of measured (rhmc_probe_alu_peaks)",
                              "count": "estimated: 10 n^3 complex MACs per shift and iteration"}
-    try:  # the FP64 hop of the per-vector baseline (width 1)
-        import torch
-
+    try:  # the FP64-accurate hop at width 1
         X = torch.randn(ctx.Vh, 3, 1, dtype=torch.complex128, device=ctx.device)
         ctx.hop(X, 1, precision="fp64")
         st = roofline.profile(lambda: [ctx.hop(X, r & 1, precision="fp64") for r in range(10)])
         e = st["hop_fp64"]
-        flops = e["launches"] * vh * 570
-        achieved = flops / (e["ms"] * 1e-3) / 1e12
         gbs = e["bytes"] / (e["ms"] * 1e-3) / 1e9
-        out["hop_fp64_width1"] = {"bound": "fp64", "achieved": achieved, "peak": f64.value,
-                                  "unit": "TFLOP/s (FP64)", "frac": achieved / f64.value,
-                                  "hbm_GB/s": gbs, "hbm_frac": gbs / roofline.peaks()["hbm_gbs"],
-                                  "peak_source": "of measured (rhmc_probe_alu_peaks)",
-                                  "count": "570 flops per site per right-hand side"}
+        out["hop_fp64_width1"] = fx_entry(e, 1) | {"hbm_GB/s": gbs, "hbm_frac": gbs / roofline.peaks()["hbm_gbs"]}
     except Exception as ex:  # a measurement beside the bench line: it never fails the line
         out["hop_fp64_width1"] = {"error": f"{type(ex).__name__}: {ex}"[:200]}
     return {"peaks": peaks, "fractions": out}
@@ -659,7 +657,7 @@ def run_gpu(args):
     stream = torch.cuda.current_stream(dev)
 
     def step():
-        # one force evaluation: FP32 (and double-float) link staging from the resident FP64
+        # one force evaluation: FP32 (and integer) link staging from the resident FP64
         # links, the solve, the force
         ctx.set_gauge(Ud)
         return ctx.force(Pd, ra.alpha0, ra.alpha, ra.beta, cfg["tol"], precision=cfg["precision"], out=G,

@@ -415,8 +415,9 @@ rhmc_status_t rhmc_profile_enable(int on);
  *   RHMC_TUNE_RELIABLE_DELTA_MILLI  mixed precision: reliable update when the
  *                                 base residual fell by value/1000 (0: 0.1)
  *   RHMC_TUNE_CHECK_EVERY         iterations between host convergence checks (0: 6)
- *   RHMC_TUNE_NATIVE_FP64_RESIDUALS  mixed precision: compute the reliable-update and
- *                                 true residuals with native FP64 instead of RHMC_DF64
+ *   RHMC_TUNE_NATIVE_FP64_RESIDUALS  apply the FP64-accurate operator (reliable-update and
+ *                                 true residuals, FP64 solves) with native FP64 operations
+ *                                 instead of exact integer sums
  *   RHMC_TUNE_UPDATE_TENSOR       mixed precision, shifted updates: on the tensor cores
  *                                 (tcgen05, three-piece TF32 split, n_rhs = 16 only) = 1; CUDA-core kernel with
  *                                 lane-owned row slices = 2; CUDA-core kernel with column-owner
@@ -446,14 +447,14 @@ rhmc_status_t rhmc_profile_enable(int on);
  *   RHMC_TUNE_NO_DEFECT_CORRECTION  1: no defect corrections after the multishift phase; the
  *                                 FP64 true residuals it left are reported (info) and shifts
  *                                 above tol give NOT_CONVERGED (for convergence studies)
- *   RHMC_TUNE_BASIS_ITERS         mixed precision, several shifts: the block basis Q_k is kept for
+ *   RHMC_TUNE_BASIS_ITERS         several shifts: the block basis Q_k is kept for
  *                                 up to this many iterations (V/2 * 3 * n_rhs * 8 bytes each,
  *                                 counted by rhmc_workspace_bytes) and the shifted solutions are
  *                                 assembled from it at the end of the multishift phase instead of
  *                                 updating P^(s), X^(s) every iteration; a solve that runs longer
  *                                 switches to the updates at that point.  0 = built-in (up to 384
- *                                 iterations within a quarter of the device memory, off below
- *                                 24), 1 = off, >= 2 = that capacity
+ *                                 iterations, in FP64 768 of 16 bytes per entry, within a quarter
+ *                                 of the device memory, off below 24), 1 = off, >= 2 = that capacity
  *   RHMC_TUNE_BASIS_GEMM          the assembly's contraction: 0 = tcgen05 tensor-core kernel (FP16
  *                                 pieces of the scaled FP32 operands, three products, FP32
  *                                 accumulation moved to a correctly rounded running sum every 48
@@ -521,7 +522,7 @@ rhmc_status_t rhmc_selftest_bounded_wait(int device, double seconds, rhmc_stream
  * best of five launches of independent FMA chains filling every SM (2 flops
  * per FMA lane), timed with CUDA events on stream s after one warm-up launch;
  * about 50 ms in all.  They are the denominators of the FP32 and FP64 roofline
- * fractions (double-float operator, n x n coefficient chain, FP64 baseline).
+ * fractions (FP64-accurate operator, n x n coefficient chain).
  * The call synchronises s.  INVALID_ARG for a null output pointer. */
 rhmc_status_t rhmc_probe_alu_peaks(int device, double *fp32_tflops, double *fp32x2_tflops, double *fp64_tflops,
                                    rhmc_stream_t s);

@@ -63,7 +63,7 @@ namespace rhmc {
 // P^(s)_K (want_p = 1: blocks i <= K, active shifts only).  The recursion runs down the blocks
 // one by one, but its columns are independent: one CTA per shift and column, the next block's
 // M2 fetched during the step.  With one CTA per shift the FP64 unit of its SM bound it
-// (8^4, n = 4: 400 -> 120 us; 12^4, n = 4, mixed: 328 -> 181 us).
+// (8^4, n = 4: 211 -> 120 us; 12^4, n = 4, mixed: 328 -> 181 us).
 constexpr int kCoefSlices = 4;  // lanes that share a dot product (n <= 16: up to four terms each)
 __global__ void __launch_bounds__(128) k_basis_coef(int n, int nshift, const SolverState *__restrict__ st,
                                                     const double2 *__restrict__ hist, int K, int want_p,

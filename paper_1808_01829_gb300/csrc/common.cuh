@@ -113,7 +113,7 @@ enum TuneKey {
   TUNE_FLUSH_EVERY,          // mixed: also flush FP32 increments every k iterations (0: at reliable updates only)
   TUNE_RELIABLE_DELTA_MILLI, // mixed: reliable update when the base residual fell by this / 1000 (0: 100)
   TUNE_CHECK_EVERY,          // iterations between host convergence checks (0: 8)
-  TUNE_NATIVE_FP64_RESIDUALS, // mixed: native FP64 instead of double-float for residuals (0: double-float)
+  TUNE_NATIVE_FP64_RESIDUALS, // FP64-accurate operator in native FP64 (1) instead of exact integer sums (0)
   TUNE_UPDATE_TENSOR,         // mixed, n = 16: shifted updates on tcgen05 (1) or CUDA cores (2); 0: built-in
   TUNE_GRAPHS,                // solver chunks as captured CUDA graphs (0/1) or eager launches (2)
   TUNE_HOP_STAGED,            // FP32 hop with cp.async-staged tiles: built-in (0), always (1), never (2)

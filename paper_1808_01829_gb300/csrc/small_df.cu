@@ -572,7 +572,7 @@ __global__ void k_df_helpers(const double *__restrict__ x, const double *__restr
   out[4 * c + k] = to_d(dmul(da, db));
   out[5 * c + k] = to_d(drcp(da));
   out[6 * c + k] = a > 0.0 ? to_d(drsqrt(da)) : 0.0;
-  df::DF acc{0.f, 0.f};  // running sum of products, as the double-float hop and force form them
+  df::DF acc{0.f, 0.f};  // running sum of products, as the force forms them
   df::df_add_prod(acc, da.h, da.l, db.h, db.l);
   df::df_add_prod(acc, db.h, db.l, db.h, db.l);
   const df::DF an = df::df_norm(acc);

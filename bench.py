@@ -25,8 +25,8 @@ Also reported on the same line:
   integer multiply-adds, at the solve's width and at width 1) and the n x n
   coefficient chain;
 * trajectory: time per RHMC trajectory (Sec. II set-up, Sec. IV parameters) on the
-  paper's 8^4 lattice, the FP64 gauge kernels at 24^4 against the measured FP64
-  peak, and the trajectory oracle on a bounded sample;
+  paper's 8^4 lattice, the gauge kernels at 24^4 against the measured integer
+  and FP64 rates, and the trajectory oracle on a bounded sample;
 * cpu_baseline: the FP64 CPU oracle on the host cores, on a bounded sample.
 
 --impl reference times the oracle (the only reference available: the paper
@@ -436,15 +436,15 @@ TRAJ = {
     "dims": (8, 8, 8, 8), "mass": 0.025, "n_pf": 4, "beta": 5.12, "tau": 1.0, "n_steps": 10, "n_gauge": 3,
     "lam": 1.0 / 6, "tol_md": 1e-7, "tol_action": 1e-14,
 }
-# real flops per link of the FP64 trajectory kernels (3 x 3 complex product = 27 complex MACs
-# = 216 flops): gauge kick 13 products (six staples of two products each, then U V); link
-# update 17 (degree-16 Taylor polynomial in Horner form, then E U; no squaring at these steps)
-TRAJ_FLOPS = {"gauge_kick": 13 * 216, "link_update": 17 * 216}
+# operations per link of the trajectory kernels: gauge kick 13 products of 3 x 3 complex matrices
+# (six staples of two each, then U V), 27 complex products each of nine wide integer multiply-adds;
+# link update about 500 FP64 instructions (its exponential on three complex numbers, D U)
+TRAJ_OPS = {"gauge_kick": 13 * 27 * 9, "link_update": 500}
 
 
-def run_trajectory(dev, fp64_peak, with_oracle, reps=3):
-    """Time per RHMC trajectory (rhmc_hmc_trajectory) on the 8^4 workload above, the FP64
-    gauge kernels at 24^4 against the measured FP64 peak, and the oracle on a bounded
+def run_trajectory(dev, fp32_peak, fp64_peak, with_oracle, reps=3):
+    """Time per RHMC trajectory (rhmc_hmc_trajectory) on the 8^4 workload above, the gauge
+    kernels at 24^4 against the measured integer and FP64 rates, and the oracle on a bounded
     sample (one outer OMF2 step with its gauge drifts, plus the heatbath and the two
     actions, scaled to n_steps outer steps)."""
     import torch
@@ -502,10 +502,13 @@ def run_trajectory(dev, fp64_peak, with_oracle, reps=3):
         b.record(stream)
         torch.cuda.synchronize()
         us = a.elapsed_time(b) * 100.0
-        tf = TRAJ_FLOPS[name] * links / (us * 1e-6) / 1e12
-        kern[name] = {"us_per_launch": us, "bound": "fp64", "achieved": tf, "peak": fp64_peak,
-                      "unit": "TFLOP/s (FP64)", "frac": tf / fp64_peak if fp64_peak else None,
-                      "count": f"{TRAJ_FLOPS[name]} flops per link, {links} links (24^4)"}
+        t = TRAJ_OPS[name] * links / (us * 1e-6) / 1e12
+        kick = name == "gauge_kick"
+        peak = (fp32_peak / 8 if kick else fp64_peak / 2) if fp64_peak else None  # (FMA = 2 flops; wide: 1/4 of FP32's)
+        kern[name] = {"us_per_launch": us, "bound": "int" if kick else "fp64", "achieved": t, "peak": peak,
+                      "unit": "T wide multiply-adds/s" if kick else "T FP64 instr/s",
+                      "frac": t / peak if peak else None,
+                      "count": f"{TRAJ_OPS[name]} per link, {links} links (24^4)"}
     c24.close()
     out["kernels_24x24x24x24"] = kern
 
@@ -795,7 +798,8 @@ def run_gpu(args):
     traj = None
     if not args.no_traj and not args.small and rank == 0:
         try:
-            traj = run_trajectory(dev, alu["peaks"]["fp64_tflops"] if alu else None,
+            traj = run_trajectory(dev, alu["peaks"]["fp32_tflops"] if alu else None,
+                                  alu["peaks"]["fp64_tflops"] if alu else None,
                                   with_oracle=not args.no_cpu and world == 1)
         except Exception as e:  # a measurement beside the bench line: it never fails the line
             traj = {"error": f"{type(e).__name__}: {e}"[:300]}

@@ -1,6 +1,6 @@
 // Arithmetic peaks of the CUDA cores, measured (the denominators of the FP32
-// and FP64 roofline fractions of the double-float hop, the n x n coefficient
-// chain and the FP64 per-vector baseline).
+// and FP64 roofline fractions of the integer hop, the n x n coefficient
+// chain and the gauge kernels).
 //
 // Every thread runs kChains independent fused multiply-add chains for `iters`
 // rounds, so that the pipes see independent instructions back to back; the

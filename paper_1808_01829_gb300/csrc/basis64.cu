@@ -16,6 +16,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "fx.cuh"
 #include "kernels.h"
 
 namespace rhmc {
@@ -143,16 +144,23 @@ __global__ void __launch_bounds__(256) k_basis64_combine(int n, int nshift, cons
 
 // out_s = sum_i Q_i C^(s)_i for the shifts s0 + SG blockIdx.y ... (want = 0: X^(s), last_s
 // blocks; 1: P^(s), K + 1 blocks, active shifts; 2: one combined set, all K blocks).  One lane
-// per (row, column), SG shifts each, so that a row of Q is read once for SG shifts;
-// coefficients staged IC blocks at a time.  Bound by the FP64 pipe.
+// per (row, column), SG shifts each, so that a row of Q is read once for SG shifts.
+// The products are exact integer sums (fx.cuh) over T blocks at a time, up to 24 terms: the
+// row's entries in these blocks are brought to one exponent, as are the T n coefficients of
+// each (shift, column), and a sum is added to the FP64 result as one value.  A term costs 9
+// multiply-adds of four clocks where FP64 takes 4 of 64; converting and the FP64 value per
+// sum take about as long again.  8^4, n = 4, 12 shifts: 342 us, 1250 us with FP64 FMAs.
+// A block with an infinity or NaN gives NaN.
 template <int N, int SG>
-__global__ void __launch_bounds__(128) k_basis64_apply(const double2 *__restrict__ basis, long rows,
-                                                       const SolverState *__restrict__ st, int K, int want, int nshift,
-                                                       const double2 *__restrict__ cf, long cfstride, int IC,
-                                                       double2 *__restrict__ out, long fstride) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  double2 *sc = reinterpret_cast<double2 *>(smem_raw);  // [SG][IC][N * N]
-  constexpr int NN = N * N;
+__global__ void __launch_bounds__(128, 4)
+    k_basis64_apply(const double2 *__restrict__ basis, long rows, const SolverState *__restrict__ st, int K, int want,
+                    int nshift, const double2 *__restrict__ cf, long cfstride, double2 *__restrict__ out,
+                    long fstride) {
+  constexpr int NN = N * N, RPW = Lanes<N>::RPW;
+  constexpr int T = 24 / N > 8 ? 8 : 24 / N < 1 ? 1 : 24 / N;  // blocks per sum
+  __shared__ int4 sq[4][RPW * T * N];                         // rows: [slot][block][column]
+  __shared__ int4 sc[SG * T * NN];                             // coefficients: [shift][block][row][column]
+  __shared__ int ce[SG * N];                                   // largest exponent field of (shift, column)
   const int s0 = 1 + SG * blockIdx.y;
   int nblk[SG], most = 0;
 #pragma unroll
@@ -161,30 +169,82 @@ __global__ void __launch_bounds__(128) k_basis64_apply(const double2 *__restrict
     nblk[g] = s >= nshift ? 0 : want == 2 ? K : want == 1 ? (st->active[s] ? K + 1 : 0) : max(0, min(st->last_k[s], K));
     most = max(most, nblk[g]);
   }
-  const Lanes<N> l((long)blockIdx.x * 4 * Lanes<N>::RPW, rows);
+  const Lanes<N> l((long)blockIdx.x * 4 * RPW, rows);
+  const int lane = threadIdx.x & 31, slot = lane / N;
+  int4 *wq = sq[threadIdx.x >> 5];
   double2 acc[SG];
 #pragma unroll
   for (int g = 0; g < SG; ++g) acc[g] = czero<double>();
-  for (int b = 0; b < most; b += IC) {
-    const int nb = min(IC, most - b);
+  for (int b = 0; b < most; b += T) {
+    const int nb = min(T, most - b);
+    // this lane's column of the row in the nb blocks, and the row's largest exponent field
+    double2 v[T];
+    int ef = 0;
+#pragma unroll
+    for (int i = 0; i < T; ++i) {
+      v[i] = (l.in && i < nb) ? basis[((size_t)(b + i) * rows + l.row) * N + l.j] : make_double2(0.0, 0.0);
+      ef = max(ef, max(fx::expo(v[i].x), fx::expo(v[i].y)));
+    }
+    {
+      const int own = ef;
+#pragma unroll
+      for (int q = 1; q < N; ++q) ef = max(ef, __shfl_sync(0xffffffffu, own, (slot * N + (l.j + q) % N) & 31));
+    }
+    __syncthreads();  // the previous sums have been formed
+    for (int k = threadIdx.x; k < SG * N; k += blockDim.x) ce[k] = 0;
+    if (slot < RPW) {
+#pragma unroll
+      for (int i = 0; i < T; ++i) {
+        const int2 re = fx::split(v[i].x, ef), im = fx::split(v[i].y, ef);
+        wq[(slot * T + i) * N + l.j] = make_int4(re.x, re.y, im.x, im.y);
+      }
+    }
+    __syncthreads();
+    double2 *raw = reinterpret_cast<double2 *>(sc);
+    for (int k = threadIdx.x; k < SG * nb * NN; k += blockDim.x) {
+      const int g = k / (nb * NN), r = k - g * (nb * NN), i = b + r / NN;
+      int most_g = 0;
+#pragma unroll
+      for (int q = 0; q < SG; ++q) most_g = q == g ? nblk[q] : most_g;
+      const double2 c = i < most_g ? cf[((size_t)(s0 - 1 + g) * cfstride + b) * NN + r] : make_double2(0.0, 0.0);
+      raw[g * T * NN + r] = c;
+      atomicMax(&ce[g * N + r % N], max(fx::expo(c.x), fx::expo(c.y)));
+    }
     __syncthreads();
     for (int k = threadIdx.x; k < SG * nb * NN; k += blockDim.x) {
       const int g = k / (nb * NN), r = k - g * (nb * NN);
-      const int i = b + r / NN;
-      sc[g * IC * NN + r] = i < (g < SG ? nblk[g] : 0) ? cf[((size_t)(s0 - 1 + g) * cfstride + b) * NN + r]
-                                                       : make_double2(0.0, 0.0);
+      const double2 c = raw[g * T * NN + r];
+      const int e = ce[g * N + r % N];
+      const int2 re = fx::split(c.x, e), im = fx::split(c.y, e);
+      sc[g * T * NN + r] = make_int4(re.x, re.y, im.x, im.y);
     }
     __syncthreads();
     if (!l.in) continue;
-    for (int i = 0; i < nb; ++i) {
-      const double2 *q = basis + ((size_t)(b + i) * rows + l.row) * N;
-      const double2 *c = sc + i * NN + l.j;
+    long long pA[SG], pB[SG], mA[SG], mB[SG], iA[SG], iB[SG];  // sums of a c, b d, (a + b)(c + d)
 #pragma unroll
-      for (int k = 0; k < N; ++k) {
-        const double2 u = __ldg(q + k);
+    for (int g = 0; g < SG; ++g) pA[g] = pB[g] = mA[g] = mB[g] = iA[g] = iB[g] = 0;
+    const int4 *q = wq + slot * T * N, *c = sc + l.j;
+#pragma unroll 1
+    for (int t = 0; t < nb * N; ++t) {
+      const int4 w = q[t];
+      const int sx = w.x + w.z, sy = w.y + w.w;
 #pragma unroll
-        for (int g = 0; g < SG; ++g)
-          if (b + i < nblk[g]) cmac<double>(acc[g], u, c[g * IC * NN + k * N]);
+      for (int g = 0; g < SG; ++g) {
+        const int4 u = c[g * T * NN + t * N];
+        fx::mac2(pA[g], pB[g], u.x, u.y, w.x, w.y);
+        fx::mac2(mA[g], mB[g], u.z, u.w, w.z, w.w);
+        fx::mac2(iA[g], iB[g], u.x + u.z, u.y + u.w, sx, sy);
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < SG; ++g) {
+      if (b >= nblk[g]) continue;
+      const int e = ce[g * N + l.j], k = (ef - 1022) + (e - 1022) - 56;
+      if (ef == 0x7ff || e == 0x7ff) {
+        acc[g].x = acc[g].y = __longlong_as_double(0x7ff8000000000000LL);
+      } else {
+        acc[g].x += fx::value(fx::join(pA[g] - mA[g], pB[g] - mB[g]), k);
+        acc[g].y += fx::value(fx::join(iA[g] - pA[g] - mA[g], iB[g] - pB[g] - mB[g]), k);
       }
     }
   }
@@ -228,11 +288,8 @@ template <int N, int SG>
 static void launch_apply(const BasisBufs &bb, const double2 *basis, const double2 *cf, int nshift,
                          const SolverState *st, long rows, int K, int want, double2 *out, long fstride,
                          cudaStream_t s) {
-  constexpr int NN = N * N;
-  const int IC = std::max(1, std::min(16, 40 * 1024 / (int)(SG * NN * sizeof(double2))));
   const dim3 grid((unsigned)((rows + 4 * Lanes<N>::RPW - 1) / (4 * Lanes<N>::RPW)), (unsigned)((nshift - 2 + SG) / SG));
-  k_basis64_apply<N, SG><<<grid, 128, (size_t)SG * IC * NN * sizeof(double2), s>>>(
-      basis, rows, st, K, want, nshift, cf, bb.cap + 1, IC, out, fstride);
+  k_basis64_apply<N, SG><<<grid, 128, 0, s>>>(basis, rows, st, K, want, nshift, cf, bb.cap + 1, out, fstride);
 }
 
 rhmc_status_t basis64_assemble(const BasisBufs &bb, const double2 *basis, int n, int nshift, const SolverState *st,

@@ -1821,6 +1821,9 @@ rhmc_status_t rhmc_rational_solve(rhmc_ctx_t *c, const void *Phi, int n, double 
 
 size_t rhmc_rational_solve_bytes(const rhmc_ctx_t *c, int n, int ns) {
   if (!c || n < 1 || n > RHMC_MAX_NRHS || ns < 1 || ns > RHMC_MAX_SHIFTS) return 0;
+  // sized under the context's own settings and device, as the solve lays it out
+  DeviceGuard dg(c->device);
+  TuneScope tscope(c);
   Arena a(nullptr);
   a.take<double2>((size_t)2 * c->g.Vh * 3 * n);
   SolveBufs b;

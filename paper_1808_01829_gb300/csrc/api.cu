@@ -184,6 +184,14 @@ struct SolverLane {
   }
 };
 
+// A buffer of a context that calls on any of its streams may use: a call's kernels wait for the
+// last ones that used it.
+struct Scratch {
+  void *p = nullptr;
+  size_t bytes = 0;
+  cudaEvent_t used = nullptr;
+};
+
 struct rhmc_ctx {
   int device = 0;
   Geom g{};
@@ -211,6 +219,7 @@ struct rhmc_ctx {
   int4 *ulfx = nullptr;            // links of a gauge-force kick in integer form, with their exponents
   int *ulex = nullptr;
   cudaEvent_t ulfx_used = nullptr; // the last kernel that reads them
+  Scratch hopfx;                   // the converted input of a lone FP64 hop
 };
 
 namespace rhmc {
@@ -251,6 +260,44 @@ static rhmc_status_t ensure_pool(rhmc_ctx *c, size_t bytes) {
   return RHMC_OK;
 }
 
+// `bytes` for kernels on s, which wait for the buffer's last users; nullptr where there is no
+// memory for it, or while s is being captured (the graph would keep an address that a later
+// call may free, and run at any time).  The callers have forms that need no buffer.
+static void *scratch_begin(Scratch &b, size_t bytes, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return nullptr;
+  if (!b.used && cudaEventCreateWithFlags(&b.used, cudaEventDisableTiming) != cudaSuccess) {
+    b.used = nullptr;
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (b.bytes < bytes) {
+    if (b.p) {  // (its users may still run)
+      if (cudaEventSynchronize(b.used) != cudaSuccess) return nullptr;
+      cudaFree(b.p);
+    }
+    b.p = nullptr;
+    b.bytes = 0;
+    if (cudaMalloc(&b.p, bytes) != cudaSuccess) {
+      b.p = nullptr;
+      cudaGetLastError();
+      return nullptr;
+    }
+    b.bytes = bytes;
+  }
+  if (cudaStreamWaitEvent(s, b.used, 0) != cudaSuccess) return nullptr;
+  return b.p;
+}
+static rhmc_status_t scratch_end(Scratch &b, cudaStream_t s) {
+  RHMC_CUDA_TRY(cudaEventRecord(b.used, s));
+  return RHMC_OK;
+}
+static void scratch_free(Scratch &b) {
+  if (b.p) cudaFree(b.p);
+  if (b.used) cudaEventDestroy(b.used);
+  b = Scratch{};
+}
+
 // The lane the calling host thread works on (the main lane unless a
 // defect-correction worker set its own).
 static thread_local SolverLane *t_lane = nullptr;
@@ -287,14 +334,17 @@ struct FxExp {
   int *in = nullptr, *mid = nullptr;
 };
 
-// out = D in for FP64 fields, or out = a self - D in: on the integer units (FP64-accurate;
-// conv: an FP64-sized buffer for the converted input, not aliasing out), or in native FP64 with
-// RHMC_TUNE_NATIVE_FP64_RESIDUALS.
-static rhmc_status_t hop64(const rhmc_ctx *c, int par, const double2 *in, double2 *out, double2 *conv, int *ex, int n,
-                           cudaStream_t s) {
+// out = D in for FP64 fields: on the integer units (FP64-accurate), or in native FP64 with
+// RHMC_TUNE_NATIVE_FP64_RESIDUALS.  Hops of one context may be enqueued on several streams and
+// captured before any other call.
+static rhmc_status_t hop64(rhmc_ctx *c, int par, const double2 *in, double2 *out, int n, cudaStream_t s) {
   if (tune_get(TUNE_NATIVE_FP64_RESIDUALS))
     return hop<double>(c->g, par, c->l64[par], in, out, nullptr, 0.0, n, 1, 0, s);
-  return hop_fx_to64(c->g, par, fx_links(c, par), in, {(int4 *)conv, ex}, out, n, s);
+  const size_t bytes = hop_fx_conv_bytes(c->g, n);
+  int4 *v = bytes ? (int4 *)scratch_begin(c->hopfx, bytes, s) : nullptr;
+  const FxField conv{v, v ? (int *)(v + c->g.Vh * 3 * n) : nullptr};
+  RHMC_TRY(hop_fx_to64(c->g, par, fx_links(c, par), in, conv, out, n, s));
+  return v ? scratch_end(c->hopfx, s) : RHMC_OK;
 }
 
 // Y = (A + sigma) X in FP64, tmp: odd-parity field of the same width.  Y may hold the
@@ -1389,6 +1439,7 @@ rhmc_status_t rhmc_destroy(rhmc_ctx_t *c) {
   if (c->ulfx) cudaFree(c->ulfx);
   if (c->ulex) cudaFree(c->ulex);
   if (c->ulfx_used) cudaEventDestroy(c->ulfx_used);
+  scratch_free(c->hopfx);
   for (int q = 0; q < 3; ++q) {
     if (c->ev_base[q]) cudaEventDestroy(c->ev_base[q]);
     if (c->ev_side[q]) cudaEventDestroy(c->ev_side[q]);
@@ -1483,12 +1534,7 @@ rhmc_status_t rhmc_hop(rhmc_ctx_t *c, const void *X, void *Y, int n, int out_par
   TuneScope tscope(c);
   cudaStream_t s = (cudaStream_t)sv;
   const long len = c->g.Vh * 3 * n;
-  if (p == RHMC_FP64 || p == RHMC_DF64) {
-    RHMC_TRY(ensure_pool(c, sizeof(double2) * len + sizeof(int) * c->g.Vh * n + 1024));
-    Arena a(c->pool);
-    double2 *conv = a.take<double2>(len);
-    return hop64(c, out_par, (const double2 *)X, (double2 *)Y, conv, a.take<int>(c->g.Vh * n), n, s);
-  }
+  if (p == RHMC_FP64 || p == RHMC_DF64) return hop64(c, out_par, (const double2 *)X, (double2 *)Y, n, s);
   RHMC_TRY(ensure_pool(c, 2 * (sizeof(float2) * len + 256)));
   Arena a(c->pool);
   float2 *x32 = a.take<float2>(len), *y32 = a.take<float2>(len);

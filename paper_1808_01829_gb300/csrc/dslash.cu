@@ -1045,29 +1045,34 @@ __global__ void __launch_bounds__(256) k_fold_parts(const double *__restrict__ p
 // each of 152 SMs), else one.  Sites per CTA: up to 128 threads, but at least a warp's
 // worth while that gives the SMs more than two CTAs each, and at most 32 link records.
 static int fx_split(const Geom &g, int n) { return g.Vh * n <= 2L * 4 * 152 * 32 ? 4 : 1; }
-static int fx_tile(const Geom &g, int n) {
-  const int items = 128 / fx_split(g, n);
+static int fx_tile(const Geom &g, int n, int split) {
+  const int items = 128 / split;
   const int least = std::max(1, items / 4 / n);
   int tile = std::max(std::min(items / n, 32), least);
   while (tile > least && (g.Vh + tile - 1) / tile < 2 * 152) tile = std::max(least, tile / 2);
   return tile;
 }
 
+size_t hop_fx_conv_bytes(const Geom &g, int n) {
+  return fx_split(g, n) == 4 ? 0 : (size_t)g.Vh * n * (3 * sizeof(int4) + sizeof(int));
+}
+
 long hop_fx_parts(const Geom &g, int n) {
-  const int tile = fx_tile(g, n);
+  const int tile = fx_tile(g, n, fx_split(g, n));
   return (g.Vh + tile - 1) / tile;
 }
 
-// in64 (optional): the input in FP64; the small-lattice kernel converts it itself, else it is
-// converted into `in` first.
+// in64 (optional): the input in FP64; the four-lane kernel converts it itself, else it is
+// converted into `in` first.  A lone FP64 hop (MODE 0) without a buffer for that takes the
+// four-lane kernel on every lattice (24^4, n = 16: 913 us; with the conversion 393 us).
 template <int MODE>
 static rhmc_status_t launch_hop_fx(const Geom &g, int par, const FxLinks &L, const double2 *in64, FxField in,
                                    void *out, int *oex, const double2 *self, double a, int n, const double2 *B,
                                    float2 *outf, double *part, int cat, cudaStream_t s) {
   if (n < 1 || n > RHMC_MAX_NRHS || g.Vh * 3L * n > 0x7fffffffL) return RHMC_ERR_INVALID_ARG;
-  const int split = fx_split(g, n), iw = 32 / split;
+  const int split = MODE == 0 && !in.v ? 4 : fx_split(g, n), iw = 32 / split;
   if (in64 && split == 1) RHMC_TRY(fx_convert(g, in64, in, n, s));
-  const int tile = fx_tile(g, n);
+  const int tile = fx_tile(g, n, split);
   const int threads = (tile * n + iw - 1) / iw * 32;
   const size_t smem = (size_t)tile * (73 * sizeof(int4) + 8 * sizeof(int));
   const unsigned grid = (unsigned)((g.Vh + tile - 1) / tile);

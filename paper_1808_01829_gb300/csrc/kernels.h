@@ -67,7 +67,9 @@ rhmc_status_t stage_links_fx(const Geom &g, const double2 *l64, int4 *lfx, int *
 // FP64-sized buffer and exponents for the converted input
 rhmc_status_t hop_fx(const Geom &g, int par, const FxLinks &L, const double2 *in, FxField conv, FxField out, int n,
                      int cat, cudaStream_t s);
-// the same with FP64 output, and as double-float pairs
+// the same with FP64 output (conv may be empty; the values and then the exponents take
+// hop_fx_conv_bytes, 0 where it would not be used), and as double-float pairs
+size_t hop_fx_conv_bytes(const Geom &g, int n);
 rhmc_status_t hop_fx_to64(const Geom &g, int par, const FxLinks &L, const double2 *in, FxField conv, double2 *out,
                           int n, cudaStream_t s);
 rhmc_status_t hop_fx_to_df(const Geom &g, int par, const FxLinks &L, const double2 *in, FxField conv, float4 *out,

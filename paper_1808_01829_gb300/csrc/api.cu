@@ -216,9 +216,7 @@ struct rhmc_ctx {
   double *d_parts = nullptr;       // partial sums of rhmc_force_lie's norm (kParts)
   void *md_buf = nullptr;          // molecular-dynamics fields (momenta, force, trial links)
   size_t md_bytes = 0;
-  int4 *ulfx = nullptr;            // links of a gauge-force kick in integer form, with their exponents
-  int *ulex = nullptr;
-  cudaEvent_t ulfx_used = nullptr; // the last kernel that reads them
+  Scratch ulfx;                    // links of a gauge-force kick in integer form, and whether each fits
   Scratch hopfx;                   // the converted input of a lone FP64 hop
 };
 
@@ -1225,30 +1223,11 @@ rhmc_status_t ctx_partials(rhmc_ctx_t *c, double **parts, int *nparts) {
   return RHMC_OK;
 }
 
-rhmc_status_t ctx_links_fx_begin(rhmc_ctx_t *c, int4 **v, int **ex, cudaStream_t s) {
-  if (!c->ulfx) {
-    RHMC_CUDA_TRY(cudaMalloc(&c->ulfx, sizeof(int4) * 36 * c->g.V));
-    if (cudaMalloc(&c->ulex, sizeof(int) * 4 * c->g.V) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ulfx_used, cudaEventDisableTiming) != cudaSuccess) {
-      cudaFree(c->ulfx);
-      if (c->ulex) cudaFree(c->ulex);
-      c->ulfx = nullptr;
-      c->ulex = nullptr;
-      set_error("out of device memory for the integer links");
-      return RHMC_ERR_CUDA;
-    }
-  } else {
-    RHMC_CUDA_TRY(cudaStreamWaitEvent(s, c->ulfx_used, 0));
-  }
-  *v = c->ulfx;
-  *ex = c->ulex;
-  return RHMC_OK;
+int4 *ctx_links_fx_begin(rhmc_ctx_t *c, cudaStream_t s) {
+  return (int4 *)scratch_begin(c->ulfx, (sizeof(int4) * 36 + sizeof(int) * 4) * c->g.V, s);
 }
 
-rhmc_status_t ctx_links_fx_end(rhmc_ctx_t *c, cudaStream_t s) {
-  RHMC_CUDA_TRY(cudaEventRecord(c->ulfx_used, s));
-  return RHMC_OK;
-}
+rhmc_status_t ctx_links_fx_end(rhmc_ctx_t *c, cudaStream_t s) { return scratch_end(c->ulfx, s); }
 
 rhmc_status_t ctx_md_buffer(rhmc_ctx_t *c, size_t bytes, void **buf) {
   if (c->md_bytes < bytes) {
@@ -1436,9 +1415,7 @@ rhmc_status_t rhmc_destroy(rhmc_ctx_t *c) {
   if (c->pool) cudaFree(c->pool);
   if (c->d_parts) cudaFree(c->d_parts);
   if (c->md_buf) cudaFree(c->md_buf);
-  if (c->ulfx) cudaFree(c->ulfx);
-  if (c->ulex) cudaFree(c->ulex);
-  if (c->ulfx_used) cudaEventDestroy(c->ulfx_used);
+  scratch_free(c->ulfx);
   scratch_free(c->hopfx);
   for (int q = 0; q < 3; ++q) {
     if (c->ev_base[q]) cudaEventDestroy(c->ev_base[q]);

@@ -584,14 +584,10 @@ rhmc_status_t gauge_momentum(rhmc_ctx_t *c, const Geom &g, const double2 *U, dou
   const long nl = g.V * 4;
   const unsigned grid = (unsigned)((g.V + 31) / 32);  // 128 threads: four directions of 32 sites
   // The integer form needs the links in integer form, in a buffer of the context.  A stream
-  // that is being captured takes the FP64 kernel: its graph may run at any later time,
-  // next to other users of the buffer.
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  RHMC_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
-  int4 *v = nullptr;
-  int *ex = nullptr;
-  if (cap == cudaStreamCaptureStatusNone) {
-    RHMC_TRY(ctx_links_fx_begin(c, &v, &ex, s));
+  // that is being captured, and one for which there is no memory, takes the FP64 kernel.
+  int4 *v = ctx_links_fx_begin(c, s);
+  int *ex = v ? (int *)(v + 36 * g.V) : nullptr;
+  if (v) {
     prof_begin(PROF_OTHER, s);
     k_links_to_fx<<<grid, 128, 0, s>>>(U, v, ex, g.V);
     prof_end(s, (double)nl * 2 * kLinkBytes);

@@ -231,10 +231,10 @@ rhmc_status_t ctx_partials(rhmc_ctx_t *ctx, double **parts, int *nparts);
 // across calls, reallocated when too small)
 rhmc_status_t ctx_md_buffer(rhmc_ctx_t *ctx, size_t bytes, void **buf);
 
-// api.cu: the context's buffer for one set of links in integer form (4 V x 9 int4 and 4 V
-// exponents, allocated on first use).  begin makes stream s wait for the buffer's last
-// user, end marks s's use of it; not for streams under capture.
-rhmc_status_t ctx_links_fx_begin(rhmc_ctx_t *c, int4 **v, int **ex, cudaStream_t s);
+// api.cu: the context's buffer for one set of links in integer form (4 V x 9 int4, then 4 V
+// flags; allocated on first use).  begin makes stream s wait for the buffer's last user and
+// gives nullptr where there is no memory or s is being captured; end marks s's use of it.
+int4 *ctx_links_fx_begin(rhmc_ctx_t *c, cudaStream_t s);
 rhmc_status_t ctx_links_fx_end(rhmc_ctx_t *c, cudaStream_t s);
 
 // scg.cu (per-vector FP64 multishift CG baseline)

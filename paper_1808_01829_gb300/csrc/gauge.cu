@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(128) k_gauge_momentum(Geom g, const double2 *_
 // entries of SU(3) links, their products and the sum of six staples have known sizes, so
 // everything is held in units of 2^-54 (two words, hi 2^27 + lo) and a product needs no
 // shift: 2^-54 2^-54 (h1 h2 2^54 + (h1 l2 + l1 h2) 2^27 + l1 l2), the last term dropped.
-// Links whose largest entry is not in [1/2, 2), products above 2 and staple sums above 8
+// Links whose largest entry is not in [1/2, 2), products of 2 and staple sums of 8 or more
 // (never for SU(3)) send the link's kick to the FP64 form.
 // The links are converted once, to v[(mu * 9 + entry) * V + site], so that the warps of the
 // kick, 32 consecutive sites of one direction each, read whole lines; ok[mu * V + site] says
@@ -306,10 +306,13 @@ __device__ __forceinline__ void row_times(const int4 *a, const int4 *b, long lon
 __device__ __forceinline__ int4 conj_if(int4 z, int m) {  // m = -1: the conjugate, 0: z
   return make_int4(z.x, z.y, (z.z ^ m) - m, (z.w ^ m) - m);
 }
-// |r| < 2^bits
-__device__ __forceinline__ bool below(long long r, int bits) {
-  return (int)(r >> bits) == 0 || (int)(r >> bits) == -1;
+// |r| <= most
+__device__ __forceinline__ bool within(long long r, long long most) {
+  return (unsigned long long)(r + most) <= 2ull * most;
 }
+// largest product and staple sum: sums of the two high words of a complex stay within 2^29 and
+// 2^31 - 2 (a value rounds up to the next high word within 2^26 of it)
+constexpr long long kMostProduct = (1ll << 55) - (1ll << 26) - 1, kMostStaples = (1ll << 57) - (1ll << 26) - 1;
 }  // namespace
 
 // The kick of k_gauge_momentum with integer products.  A staple is op(X) Y^dagger op'(Z)
@@ -374,7 +377,7 @@ __global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4
       row_times(a, y, r);
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        fits = fits && below(r[2 * k], 55) && below(r[2 * k + 1], 55);
+        fits = fits && within(r[2 * k], kMostProduct) && within(r[2 * k + 1], kMostProduct);
         const int2 re = fx::words(r[2 * k]), im = fx::words(r[2 * k + 1]);
         a[k] = make_int4(re.x, re.y, im.x, im.y);
       }
@@ -387,7 +390,7 @@ __global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4
 #pragma unroll
   for (int c = 0; c < 9; ++c) {
     const long long re = sV[2 * c][tid], im = sV[2 * c + 1][tid];
-    fits = fits && below(re, 57) && below(im, 57);
+    fits = fits && within(re, kMostStaples) && within(im, kMostStaples);
     const int2 wr = fx::words(re), wi = fx::words(im);
     b[c] = make_int4(wr.x, wr.y, wi.x, wi.y);
   }

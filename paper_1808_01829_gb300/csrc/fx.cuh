@@ -55,12 +55,12 @@ __device__ __forceinline__ int2 split(double x, int ef) {
   return words((long long)(mag ^ (unsigned long long)sg) - sg);
 }
 
-// x 2^54 rounded, for |x| < 2
-__device__ __forceinline__ long long fixed54(double x) {
+// x 2^55 rounded, for |x| < 2
+__device__ __forceinline__ long long fixed55(double x) {
   const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
   const int e = (int)(hw >> 20) & 0x7ff;
   const unsigned long long m = ((unsigned long long)((hw & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lw;
-  const int s = 1023 + 52 - 54 - e;  // x = m 2^(e - 1075), 2^54 x = m 2^(e - 1021)
+  const int s = 1023 + 52 - 55 - e;  // x = m 2^(e - 1075), 2^55 x = m 2^(e - 1020)
   const unsigned long long mag = s <= 0 ? m << -s : ((m >> min(63, s - 1)) + 1) >> 1;
   const long long sg = (long long)((int)hw >> 31);
   return (long long)(mag ^ (unsigned long long)sg) - sg;

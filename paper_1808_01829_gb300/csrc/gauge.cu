@@ -257,36 +257,59 @@ __global__ void __launch_bounds__(128) k_gauge_momentum(Geom g, const double2 *_
 }
 
 // ------------------------------------------------------------ the kick on the integer units
+namespace {
+// |r| <= most
+__device__ __forceinline__ bool within(long long r, long long most) {
+  return (unsigned long long)(r + most) <= 2ull * most;
+}
+// Largest entry of a link and of a product (one, to rounding) and largest staple sum (eight): sums
+// of the two high words of a complex stay within 2^29 + 2^14, 2^30 + 2^15 and 2^31 - 2 (a value
+// rounds up to the next high word within 2^26 of it), and sums of three products below 2^62.
+constexpr long long kMostLink = (1ll << 55) + (1ll << 40), kMostProduct = (1ll << 56) + (1ll << 41),
+                    kMostStaples = (1ll << 57) - (1ll << 26) - 1;
+}  // namespace
+
 // The 13 products of 3 x 3 matrices of a link's kick (1404 FP64 FMAs, 64 clocks each for a
 // warp) as exact integer sums (fx.cuh): 243 multiply-adds of four clocks per product.  The
 // entries of SU(3) links, their products and the sum of six staples have known sizes, so
-// everything is held in units of 2^-54 (two words, hi 2^27 + lo) and a product needs no
-// shift: 2^-54 2^-54 (h1 h2 2^54 + (h1 l2 + l1 h2) 2^27 + l1 l2), the last term dropped.
-// Links whose largest entry is not in [1/2, 2), products of 2 and staple sums of 8 or more
-// (never for SU(3)) send the link's kick to the FP64 form.
+// links are held in units of 2^-55, products of two in 2^-56, staples in 2^-57 and their sum in
+// 2^-54 (two words, hi 2^27 + lo), and a product needs no shift: 2^-54 of it is
+// h1 h2 + (h1 l2 + l1 h2) 2^-27 + l1 l2 2^-54, the last term dropped.
+// Links whose largest entry is not in [1/4, 1] (to rounding), products above that and staple
+// sums of 8 or more (never for SU(3)) send the link's kick to the FP64 form.
+// So does a kick whose FP64 form would be more accurate than these units: its rounding is
+// relative to the sizes of the products that form an entry, sum_k |U_ik| |V_kj|, which is small
+// next to one for links near the unit matrix (weak fields) or near a block form.
 // The links are converted once, to v[(mu * 9 + entry) * V + site], so that the warps of the
 // kick, 32 consecutive sites of one direction each, read whole lines; ok[mu * V + site] says
-// whether the link fits.
+// whether the link fits (kFits) and whether it is near a real diagonal matrix (kWeak).
+constexpr int kFits = 1, kWeak = 2;
 __global__ void __launch_bounds__(128) k_links_to_fx(const double2 *__restrict__ U, int4 *__restrict__ v,
                                                      int *__restrict__ ok, long V) {
   const int mu = threadIdx.x >> 5;
   const long site = (long)blockIdx.x * 32 + (threadIdx.x & 31);
   if (site >= V) return;
   const M3 u = ld3(U + (site * 4 + mu) * 9);
-  int ef = 0;
-#pragma unroll
-  for (int c = 0; c < 9; ++c) ef = max(ef, max(fx::expo(u.e[c].x), fx::expo(u.e[c].y)));
-  const bool fits = ef == 1022 || ef == 1023;
+  int ef = 0, small = 0;  // largest exponent field, and that of all but the real diagonal
 #pragma unroll
   for (int c = 0; c < 9; ++c) {
-    const int2 re = fx::words(fits ? fx::fixed54(u.e[c].x) : 0), im = fx::words(fits ? fx::fixed54(u.e[c].y) : 0);
+    const int re = fx::expo(u.e[c].x), im = fx::expo(u.e[c].y);
+    ef = max(ef, max(re, im));
+    small = max(small, max(c % 4 ? re : 0, im));
+  }
+  bool fits = ef >= 1021 && ef <= 1023;
+#pragma unroll
+  for (int c = 0; c < 9; ++c) {
+    const long long qr = fits ? fx::fixed55(u.e[c].x) : 0, qi = fits ? fx::fixed55(u.e[c].y) : 0;
+    fits = fits && within(qr, kMostLink) && within(qi, kMostLink);
+    const int2 re = fx::words(qr), im = fx::words(qi);
     v[(mu * 9 + c) * V + site] = make_int4(re.x, re.y, im.x, im.y);
   }
-  ok[mu * V + site] = fits;
+  ok[mu * V + site] = (fits ? kFits : 0) | (small < 1023 - 6 ? kWeak : 0);
 }
 
 namespace {
-// three sums r_j = sum_k a_k b[k][j] in units of 2^-54, rounded (reals: re, im)
+// three sums r_j = sum_k a_k b[k][j] in a_k's and b's units multiplied by 2^54, rounded (re, im)
 __device__ __forceinline__ void row_times(const int4 *a, const int4 *b, long long *r) {
   constexpr long long half = 1ll << (fx::kLow - 1);
 #pragma unroll
@@ -303,16 +326,11 @@ __device__ __forceinline__ void row_times(const int4 *a, const int4 *b, long lon
     r[2 * j + 1] = fx::join(iA - pA - mA, iB - pB - mB);
   }
 }
+// Sizes (in units of 2^-20) below which the FP64 form is the more accurate one; see k_gauge_momentum_fx
+constexpr int kOffSize = (int)(0.8 * (1 << 20)), kDiagSize = (int)(0.4 * (1 << 20));
 __device__ __forceinline__ int4 conj_if(int4 z, int m) {  // m = -1: the conjugate, 0: z
   return make_int4(z.x, z.y, (z.z ^ m) - m, (z.w ^ m) - m);
 }
-// |r| <= most
-__device__ __forceinline__ bool within(long long r, long long most) {
-  return (unsigned long long)(r + most) <= 2ull * most;
-}
-// largest product and staple sum: sums of the two high words of a complex stay within 2^29 and
-// 2^31 - 2 (a value rounds up to the next high word within 2^26 of it)
-constexpr long long kMostProduct = (1ll << 55) - (1ll << 26) - 1, kMostStaples = (1ll << 57) - (1ll << 26) - 1;
 }  // namespace
 
 // The kick of k_gauge_momentum with integer products.  A staple is op(X) Y^dagger op'(Z)
@@ -321,8 +339,14 @@ constexpr long long kMostProduct = (1ll << 55) - (1ll << 26) - 1, kMostStaples =
 // The loops over staples and rows are not unrolled, and the sum lives in shared memory:
 // unrolled, the warps waited for instructions.  Bound by the integer multiplier, 13 x 243
 // multiply-adds of four clocks per link (175 us at 16^3 x 32), and by the adds and shifts around
-// them at two warps per scheduler.  Measured at 16^3 x 32: 518 us, and 27 us for the conversion,
-// 1791 us in FP64; error of P after a kick of eps = 0.5 7.6e-17 (FP64 form 1.0e-16).
+// them at two warps per scheduler.  Measured at 16^3 x 32, with the conversion: 562 us, 1795 us in
+// FP64.  Error of the force (largest entry, relative to the largest of the lattice): links
+// exp(i eps H) with eps = 0.5 8.1e-17, FP64 form 2.3e-16.
+// The error in these units is the same for every link, that of the FP64 form is relative to
+// S_ij = sum_k |U_ik| |V_kj| + |U_jk| |V_ki| off the diagonal and to the largest of
+// sum_k |Re U_ik| |Im V_ki| + |Im U_ik| |Re V_ki| on it.  They meet where these are 0.8 and 0.4
+// (both forms up to 1.6e-16 S and 4.4e-16 S); a link below either takes the FP64 form.  At
+// eps = 0.5 no link does, at 0.3 one in 2000 (659 us), from 0.1 down nearly all (1.8 ms).
 __global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4 *__restrict__ v,
                                                               const int *__restrict__ ok,
                                                               const double2 *__restrict__ U, double2 *__restrict__ P,
@@ -345,7 +369,8 @@ __global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4
   }
   step(g, x, mu, 1, xp);
   const int sp = (int)lex_of(g, xp);
-  bool fits = ok[mu * nsite + site];
+  const int flags = ok[mu * nsite + site];
+  bool fits = flags & kFits;
 #pragma unroll 1
   for (int q = 0; q < 6; ++q) {
     const int nu = (q >> 1) < mu ? (q >> 1) : (q >> 1) + 1;
@@ -355,7 +380,13 @@ __global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4
     step(g, xn, mu, 1, xq);
     const int sn = (int)lex_of(g, xn);
     const int sx = fwd ? sp : (int)lex_of(g, xq), sz = fwd ? site : sn;
-    fits = fits && ok[nu * nsite + sx] && ok[mu * nsite + sn] && ok[nu * nsite + sz];
+    const int near = flags & ok[nu * nsite + sx] & ok[mu * nsite + sn] & ok[nu * nsite + sz];
+    fits = fits && (near & kFits);
+    // one such plaquette in a warp: the FP64 form will be needed at the end, so at once
+    if (q == 0 && __any_sync(__activemask(), near & kWeak)) {
+      kick_fp64(g, U, P, coef, (long)site * 4 + mu);
+      return;
+    }
     const int4 *px = v + (long)nu * 9 * nsite + sx, *py = v + (long)mu * 9 * nsite + sn,
                *pz = v + (long)nu * 9 * nsite + sz;
     const int cz = fwd ? -1 : 0;
@@ -387,38 +418,51 @@ __global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4
     }
   }
   int4 b[9];
+  int vr[9], vi[9];  // sizes of the parts of V in units of 2^-10
 #pragma unroll
   for (int c = 0; c < 9; ++c) {
-    const long long re = sV[2 * c][tid], im = sV[2 * c + 1][tid];
+    const long long re = (sV[2 * c][tid] + 4) >> 3, im = (sV[2 * c + 1][tid] + 4) >> 3;
     fits = fits && within(re, kMostStaples) && within(im, kMostStaples);
     const int2 wr = fx::words(re), wi = fx::words(im);
     b[c] = make_int4(wr.x, wr.y, wi.x, wi.y);
-  }
-  if (!fits) {
-    kick_fp64(g, U, P, coef, (long)site * 4 + mu);
-    return;
+    vr[c] = abs(wr.x) >> 17;
+    vi[c] = abs(wi.x) >> 17;
   }
   long long w[18];
+  int od[3] = {0, 0, 0}, di = 0;  // sum_k |U_ik| |V_kj| + |U_jk| |V_ki|, and that of the diagonal's imaginary part
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     int4 a[3];
+    int d = 0;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) a[c] = __ldg(v + (long)(mu * 9 + i * 3 + c) * nsite + site);
+    for (int c = 0; c < 3; ++c) {
+      a[c] = __ldg(v + (long)(mu * 9 + i * 3 + c) * nsite + site);
+      const int ur = abs(a[c].x) >> 18, ui = abs(a[c].z) >> 18;  // (units of 2^-10)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (j != i) od[i + j - 1] += (ur + ui) * (vr[c * 3 + j] + vi[c * 3 + j]);
+      d += ur * vi[c * 3 + i] + ui * vr[c * 3 + i];
+    }
+    di = max(di, d);
     row_times(a, b, w + 6 * i);
+  }
+  if (!fits || min(od[0], min(od[1], od[2])) < kOffSize || di < kDiagSize) {
+    kick_fp64(g, U, P, coef, (long)site * 4 + mu);
+    return;
   }
   // TA(w) = (w - w^dagger)/2 - tr(w - w^dagger)/6; its upper triangle, twice as large
   double2 *p = P + ((long)site * 4 + mu) * 9;
   const long long tr = (w[1] + w[9] + w[17]) / 3;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    const double d = fx::value(w[2 * (i * 4) + 1] - tr, -53);
+    const double d = fx::value(w[2 * (i * 4) + 1] - tr, -54);
     double2 z = p[i * 4];
     z.y = fma(0.5 * coef, d, z.y);
     p[i * 4] = z;
 #pragma unroll
     for (int j = i + 1; j < 3; ++j) {
       const int a = 2 * (i * 3 + j), c = 2 * (j * 3 + i);
-      const double re = fx::value(w[a] - w[c], -54), im = fx::value(w[a + 1] + w[c + 1], -54);
+      const double re = fx::value(w[a] - w[c], -55), im = fx::value(w[a + 1] + w[c + 1], -55);
       double2 z1 = p[i * 3 + j], z2 = p[j * 3 + i];
       z1.x = fma(0.5 * coef, re, z1.x);
       z1.y = fma(0.5 * coef, im, z1.y);

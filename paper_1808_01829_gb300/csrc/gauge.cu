@@ -504,13 +504,24 @@ __global__ void __launch_bounds__(128) k_link_update(double2 *__restrict__ U, co
                                                      double eps) {
   const long l = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= nlinks) return;
-  const M3 p = ld3(P + l * 9);
-  double n2 = 0.0;
+  M3 p = ld3(P + l * 9);
+  auto norm2 = [&]() {
+    double n = 0.0;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) n2 = fma(p.e[k].x, p.e[k].x, fma(p.e[k].y, p.e[k].y, n2));
-  n2 *= eps * eps;
+    for (int k = 0; k < 9; ++k) n = fma(p.e[k].x, p.e[k].x, fma(p.e[k].y, p.e[k].y, n));
+    return n;
+  };
+  double n2 = norm2();
   int sq = 0;
   double sc = eps;
+  if (n2 > 1e-100 && n2 < 1e100) {
+    n2 *= eps * eps;
+  } else {  // det P could leave the range of FP64 where Y = eps P does not
+#pragma unroll
+    for (int k = 0; k < 9; ++k) p.e[k] = zscale(p.e[k], eps);
+    sc = 1.0;
+    n2 = norm2();
+  }
   while (n2 > 0.25 && sq < 64) {  // bounded: a non-finite norm stops at 64
     n2 *= 0.25;
     sc *= 0.5;

@@ -572,15 +572,17 @@ __global__ void __launch_bounds__(128) k_link_update(double2 *__restrict__ U, co
     cmac<double>(a, f1, p.e[q]);
     D.e[q] = a;
   }
-  for (int i = 0; i < sq; ++i) {  // (1 + D)^2 - 1 = 2 D + D^2
-    const M3 D2 = mul(D, D);
-#pragma unroll
-    for (int q = 0; q < 9; ++q) D.e[q] = make_double2(fma(2.0, D.e[q].x, D2.e[q].x), fma(2.0, D.e[q].y, D2.e[q].y));
+  if (sq) {  // |Y| > 1/2: 1 + D itself, squared (an exponential of small entries keeps their relative accuracy)
+    D.e[0].x += 1.0;
+    D.e[4].x += 1.0;
+    D.e[8].x += 1.0;
+    for (int i = 0; i < sq; ++i) D = mul(D, D);
   }
   const M3 u = ld3(U + l * 9);
   const M3 w = mul(D, u);
 #pragma unroll
-  for (int k = 0; k < 9; ++k) U[l * 9 + k] = make_double2(u.e[k].x + w.e[k].x, u.e[k].y + w.e[k].y);
+  for (int k = 0; k < 9; ++k)
+    U[l * 9 + k] = sq ? w.e[k] : make_double2(u.e[k].x + w.e[k].x, u.e[k].y + w.e[k].y);
 }
 
 // ------------------------------------------------------------ launch wrappers

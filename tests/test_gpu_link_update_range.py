@@ -1,5 +1,5 @@
 """The link update exp(eps P) U where P alone is near the ends of the FP64 range (eps P is not),
-against a plain sum.
+and for P whose exponential is small (negative real parts), against a plain sum.
 
 Tolerance: 1e-12 of the largest entry of each link's result: exp(Y) takes up to eight squarings of
 a sum of unit size, 2^8 roundings of a three-term complex product (2^-53 x 2^8 x 8 = 2.3e-13), in
@@ -43,3 +43,9 @@ def test_momenta_near_the_ends_of_the_range(power):
     need_gpu()
     H = _random()
     _check(H * 10.0 ** power, 0.1 / 10.0 ** power, 0.1 * H)
+
+@pytest.mark.parametrize("decay", [0.1, 3.0, 30.0])
+def test_small_exponentials(decay):
+    need_gpu()
+    H = 0.2 * _random()
+    _check(10 * (H - decay * np.eye(3)), 0.1, H, decay)

@@ -716,28 +716,38 @@ using namespace df;
 // converting inside the hop took 465 us per hop at 24^4, n = 16.
 //
 // Integer link records, one int4 per complex of the FP64 records, and the exponent of each
-// site's largest entry (kSpecial where the site takes FP64 arithmetic).  Eight lanes
-// per site, one per direction.
+// site's largest entry (kSpecial where the site takes FP64 arithmetic: non-finite or zero
+// links, or a row of one of them more than 2^3 below it, which never happens for SU(3)).
+// Eight lanes per site, one per direction.
 __global__ void __launch_bounds__(256) k_stage_links_fx(const double2 *__restrict__ l64, int4 *__restrict__ lfx,
                                                         int *__restrict__ lexp, long nrec) {
   const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;  // (site, direction)
   const bool in = k < nrec;
   double2 v[9];
-  int ef = 0;
+  int ef = 0, row = 0x7ff;  // largest exponent field; that of the smallest row
 #pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    v[e] = in ? l64[k * 9 + e] : make_double2(0.0, 0.0);
-    ef = max(ef, max(fx::expo(v[e].x), fx::expo(v[e].y)));
+  for (int a = 0; a < 3; ++a) {
+    int er = 0;
+#pragma unroll
+    for (int e = 3 * a; e < 3 * a + 3; ++e) {
+      v[e] = in ? l64[k * 9 + e] : make_double2(0.0, 0.0);
+      er = max(er, max(fx::expo(v[e].x), fx::expo(v[e].y)));
+    }
+    ef = max(ef, er);
+    row = min(row, er);
   }
 #pragma unroll
-  for (int off = 4; off > 0; off >>= 1) ef = max(ef, __shfl_xor_sync(0xffffffffu, ef, off, 8));
+  for (int off = 4; off > 0; off >>= 1) {
+    ef = max(ef, __shfl_xor_sync(0xffffffffu, ef, off, 8));
+    row = min(row, __shfl_xor_sync(0xffffffffu, row, off, 8));
+  }
   if (!in) return;
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
     const int2 re = fx::split(v[e].x, ef), im = fx::split(v[e].y, ef);
     lfx[k * 9 + e] = make_int4(re.x, re.y, im.x, im.y);
   }
-  if ((k & 7) == 0) lexp[k >> 3] = (ef == 0 || ef == 0x7ff) ? fx::kSpecial : ef - 1022;
+  if ((k & 7) == 0) lexp[k >> 3] = (ef == 0 || ef == 0x7ff || row < ef - 3) ? fx::kSpecial : ef - 1022;
 }
 
 rhmc_status_t stage_links_fx(const Geom &g, const double2 *l64, int4 *lfx, int *lexp, cudaStream_t s) {
@@ -790,19 +800,21 @@ static rhmc_status_t fx_convert(const Geom &g, const double2 *in, FxField out, i
 // the first hop) against 1246 us with FP64 FMAs; an operator application at 8^4,
 // n = 4 16 against 37 us.  Against a long-double sum its error is 1.0e-16 relative for
 // Gaussian fields, that of FP64 FMAs 2.9e-16.
-// Lanes with a special block among their inputs, or neighbours more than 2^26
-// apart in size, take FP64 arithmetic.
+// Lanes with a special block among their inputs, neighbours more than 2^26 apart in
+// size, or no neighbour with its colours of like size (fx.cuh) take FP64 arithmetic, on
+// in64 where the input was given in FP64; its result is kept in FP64 (MODE 4).
 //
 // MODE 0: out = D in.  1: out = a self - D in.  2: out = B - (a self - D in), with
 // the optional FP32 rounding outf and per-CTA column sums of |out|^2 (part).
-// 3: out = D in as double-float pairs (float4).  4: D in in integer form, exponents oex.
+// 3: out = D in as double-float pairs (float4).  4: D in in integer form, block words oex.
 template <int MODE, int S, bool IN64>
 __global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *__restrict__ lfx,
                                                    const int *__restrict__ lexp, const double2 *__restrict__ l64,
                                                    const int4 *__restrict__ in, const int *__restrict__ iex,
-                                                   void *outv, int *__restrict__ oex, const double2 *self, double a,
-                                                   int n, int tile, const double2 *__restrict__ B,
-                                                   float2 *__restrict__ outf, double *__restrict__ part) {
+                                                   const double2 *__restrict__ in64, void *outv,
+                                                   int *__restrict__ oex, const double2 *self, double a, int n,
+                                                   int tile, const double2 *__restrict__ B, float2 *__restrict__ outf,
+                                                   double *__restrict__ part) {
   constexpr int LS = 73;
   constexpr int IW = 32 / S;  // (site, right-hand side) items per warp
   constexpr int ND = 8 / S;   // directions per lane
@@ -843,8 +855,7 @@ __global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *
   const bool live = ls < nsites;
   const int *nb = snb + (live ? ls : 0) * 8;
   const int n3 = 3 * n, d0 = quad * ND;
-  const double2 *in64 = reinterpret_cast<const double2 *>(in);
-  int E = fx::kZero, low = fx::kSpecial, el = 0, ef = 0;
+  int E = fx::kZero, low = fx::kSpecial, even = fx::kZero, el = 0, ef = 0;  // even: the best neighbour's least colour
   int4 v[3];
   double2 x64[IN64 ? ND : 1][3];
   if (IN64) {
@@ -856,13 +867,22 @@ __global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *
 #pragma unroll
         for (int c = 0; c < 3; ++c) x64[IN64 ? d : 0][c] = __ldg(in64 + (nb[d0 + d] * n3 + j) + c * n);
 #pragma unroll
-      for (int d = 0; d < ND; ++d)
+      for (int d = 0; d < ND; ++d) {
+        int eb = 0, em = 0x7ff;
+        bool some = false;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           const double2 x = x64[IN64 ? d : 0][c];
-          ef = max(ef, max(fx::expo(x.x), fx::expo(x.y)));
-          any = any || fx::nonzero(x.x) || fx::nonzero(x.y);
+          const int e = max(fx::expo(x.x), fx::expo(x.y));
+          eb = max(eb, e);
+          em = min(em, e);
+          some = some || fx::nonzero(x.x) || fx::nonzero(x.y);
         }
+        ef = max(ef, eb);
+        if (em) even = max(even, em - 1022);
+        if (some) low = min(low, eb - 1022);
+        any = any || some;
+      }
     }
 #pragma unroll
     for (int off = IW; off < 32; off <<= 1) {
@@ -870,28 +890,27 @@ __global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *
       any = __shfl_xor_sync(0xffffffffu, (int)any, off) || any;
     }
     E = !any ? fx::kZero : (ef == 0 || ef == 0x7ff) ? fx::kSpecial : ef - 1022;
-    low = E;
   } else if (live) {
     el = lexp[h0 + ls];
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
-      const int e = iex[nb[d0 + d] * n + j];
+      const int code = iex[nb[d0 + d] * n + j], e = fx::exponent(code);
       E = max(E, e);
       low = min(low, e == fx::kZero ? fx::kSpecial : e);
+      even = max(even, fx::least(code));
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) v[c] = __ldg(in + (nb[d0] * n3 + j) + c * n);
   }
-  if (!IN64) {
 #pragma unroll
-    for (int off = IW; off < 32; off <<= 1) {
-      E = max(E, __shfl_xor_sync(0xffffffffu, E, off));
-      low = min(low, __shfl_xor_sync(0xffffffffu, low, off));
-    }
+  for (int off = IW; off < 32; off <<= 1) {
+    if (!IN64) E = max(E, __shfl_xor_sync(0xffffffffu, E, off));
+    low = min(low, __shfl_xor_sync(0xffffffffu, low, off));
+    even = max(even, __shfl_xor_sync(0xffffffffu, even, off));
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  const bool fast = E != fx::kSpecial && el != fx::kSpecial && (E == fx::kZero || E - low <= fx::kAlign);
+  const bool fast = E != fx::kSpecial && el != fx::kSpecial && (E == fx::kZero || (E - low <= fx::kAlign && E - even <= fx::kApart));
   long long R[6];
   if (live && fast) {
     long long pA[3], pB[3], mA[3], mB[3], iA[3], iB[3];  // sums of a c, b d, (a + b)(c + d)
@@ -919,7 +938,7 @@ __global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *
     } else {
 #pragma unroll 1
       for (int d = d0; d < d0 + ND; ++d, lk += 9) {
-        const int sh = min(fx::kAlign, E - iex[nb[d] * n + j]);  // (clamped for zeros only)
+        const int sh = min(fx::kAlign, E - fx::exponent(iex[nb[d] * n + j]));  // (clamped for zeros only)
         int4 w[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) w[c] = v[c];
@@ -962,8 +981,8 @@ __global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *
 #pragma unroll 1
       for (int q = 0; q < 24; ++q) {
         const int d = q / 3, cb = q - d * 3;
-        const double2 w = IN64 ? in64[nb[d] * n3 + j + cb * n]
-                               : fx::unpack(in[nb[d] * n3 + j + cb * n], iex[nb[d] * n + j]);
+        const double2 w = IN64 || in64 ? in64[nb[d] * n3 + j + cb * n]
+                                       : fx::unpack(in[nb[d] * n3 + j + cb * n], fx::exponent(iex[nb[d] * n + j]));
         const double2 *l = L + d * 9 + cb;
 #pragma unroll
         for (int ca = 0; ca < 3; ++ca) cmac<double>(acc[ca], l[ca * 3], w);
@@ -973,9 +992,9 @@ __global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *
       int4 q[3];
       int e;
       if (!fast) {
-        e = fx::pack3(acc, q);
+        e = fx::keep3(acc, q);
       } else if (E == fx::kZero) {
-        e = fx::kZero;
+        e = fx::code(fx::kZero, 0);
         q[0] = q[1] = q[2] = make_int4(0, 0, 0, 0);
       } else {
         e = fx::renorm3(R, k, q);
@@ -1077,21 +1096,22 @@ static rhmc_status_t launch_hop_fx(const Geom &g, int par, const FxLinks &L, con
   const size_t smem = (size_t)tile * (73 * sizeof(int4) + 8 * sizeof(int));
   const unsigned grid = (unsigned)((g.Vh + tile - 1) / tile);
   prof_begin(cat, s);
-  auto run = [&](auto kern, const int4 *src) {
-    kern<<<grid, threads, smem, s>>>(g, par, L.rec, L.exp, L.l64, src, in.e, out, oex, self, a, n, tile, B, outf, part);
+  auto run = [&](auto kern) {
+    kern<<<grid, threads, smem, s>>>(g, par, L.rec, L.exp, L.l64, in.v, in.e, in64, out, oex, self, a, n, tile, B, outf,
+                                     part);
   };
   bool done = false;
   if constexpr (MODE == 0 || MODE == 3 || MODE == 4) {
     if (in64 && split == 4) {
-      run(k_hop_fx<MODE, 4, true>, reinterpret_cast<const int4 *>(in64));
+      run(k_hop_fx<MODE, 4, true>);
       done = true;
     }
   }
   if (!done) {
     if (split == 4)
-      run(k_hop_fx<MODE, 4, false>, in.v);
+      run(k_hop_fx<MODE, 4, false>);
     else
-      run(k_hop_fx<MODE, 1, false>, in.v);
+      run(k_hop_fx<MODE, 1, false>);
   }
   // algorithmic bytes: every link once, the inputs once, the outputs once
   const double fields = 2.0 + (MODE == 1 ? 1.0 : 0.0) + (MODE == 2 ? 2.0 + (outf ? 0.5 : 0.0) : 0.0);

@@ -19,9 +19,19 @@
 // aligned (|lo| < 1.25 2^27), |B| <= 24 (2^29 1.25 2^28 + 2^27 2^29) < 2^63.
 //
 // A field in this form has one int4 (re hi, re lo, im hi, im lo) per complex, as
-// large as its FP64 form, and one exponent E per (site, column) for the three
-// colours.  Blocks with infinities, NaN or subnormals keep their FP64 values in the
-// int4 under the exponent kSpecial; kZero marks a block of zeros.
+// large as its FP64 form, and one word per (site, column) with the exponent E of the three
+// colours and how far the smallest colour lies below it (code, exponent, least).  Blocks with
+// infinities, NaN or subnormals keep their FP64 values in the int4 under the exponent
+// kSpecial; kZero marks a block of zeros.
+//
+// The error of a sum is absolute, 2^-55 of the largest operands, that of FP64 FMAs relative to
+// sum |U_cb| |v_b| of each output c.  The two agree unless that sum is small for some c, as where
+// unit-like links keep colours of very different size apart.  A hop therefore takes the integer
+// form only where one of the eight neighbours has all three colours within 2^kApart of
+// the largest: a row c of unitary links has an entry of order one there (stage_links_fx
+// checks it), so every output's sum is of the size the integers resolve.  Measured against
+// extended precision, largest error over sum |U_cb| |v_b| (integers; FP64 FMAs): Gaussian fields
+// 7.6e-17; 4.1e-16, unit links and colours 1, 1/8, 1/8 4.1e-16; 2.6e-16.
 #pragma once
 
 namespace rhmc {
@@ -31,6 +41,12 @@ constexpr int kLow = 27;              // bits of the low word
 constexpr int kBits = 55;             // magnitude bits
 constexpr int kSpecial = 1 << 20;     // exponent code: the block holds FP64 values
 constexpr int kZero = -(1 << 20);     // exponent code: all zeros
+constexpr int kApart = 3;             // see above; Gaussian colours: all but one (site, column) in a million
+
+// A block's word: its exponent and, in the low five bits, the distance to that of its smallest colour
+__device__ __forceinline__ int code(int e, int apart) { return e * 32 + min(apart, 31); }
+__device__ __forceinline__ int exponent(int c) { return c >> 5; }
+__device__ __forceinline__ int least(int c) { return (c >> 5) - (c & 31); }
 
 // biased exponent field (0: zero or subnormal, 0x7ff: infinity or NaN)
 __device__ __forceinline__ int expo(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
@@ -66,26 +82,32 @@ __device__ __forceinline__ long long fixed55(double x) {
   return (long long)(mag ^ (unsigned long long)sg) - sg;
 }
 
-// Three complex numbers (a site's column) as one block; returns its exponent.
-__device__ __forceinline__ int pack3(const double2 *v, int4 *o) {
-  int ef = 0;
+// Three complex numbers (a site's column) as they are; returns the block's word.
+__device__ __forceinline__ int keep3(const double2 *v, int4 *o) {
   bool any = false;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    ef = max(ef, max(expo(v[c].x), expo(v[c].y)));
     any = any || nonzero(v[c].x) || nonzero(v[c].y);
+    o[c] = *reinterpret_cast<const int4 *>(&v[c]);
   }
-  if (ef == 0x7ff || (ef == 0 && any)) {
+  return code(any ? kSpecial : kZero, 0);
+}
+// Three complex numbers as one block; returns its word.
+__device__ __forceinline__ int pack3(const double2 *v, int4 *o) {
+  int ef = 0, em = 0x7ff;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) o[c] = *reinterpret_cast<const int4 *>(&v[c]);
-    return kSpecial;
+  for (int c = 0; c < 3; ++c) {
+    const int e = max(expo(v[c].x), expo(v[c].y));
+    ef = max(ef, e);
+    em = min(em, e);
   }
+  if (ef == 0x7ff || ef == 0) return keep3(v, o);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const int2 re = split(v[c].x, ef), im = split(v[c].y, ef);
     o[c] = make_int4(re.x, re.y, im.x, im.y);
   }
-  return any ? ef - 1022 : kZero;
+  return code(ef - 1022, em ? ef - em : 31);
 }
 // The FP64 value of one complex of a block with exponent e.
 __device__ __forceinline__ double2 unpack(int4 q, int e) {
@@ -131,11 +153,15 @@ __device__ __forceinline__ long long shift(long long r, int right) {
 // Six reals r 2^k (three complex) as a block: brought to 55 bits by the leading bit of the
 // largest.
 __device__ __forceinline__ int renorm3(const long long *r, int k, int4 *o) {
-  unsigned long long m = 0;
+  int len = 0, least = 64;
 #pragma unroll
-  for (int c = 0; c < 6; ++c) m |= (unsigned long long)(r[c] ^ (r[c] >> 63));
-  // |r| <= m + 1 <= 2^len
-  const int len = 64 - __clzll((long long)m);
+  for (int c = 0; c < 3; ++c) {
+    // |r| <= m + 1 <= 2^l
+    const unsigned long long m = (unsigned long long)((r[2 * c] ^ (r[2 * c] >> 63)) | (r[2 * c + 1] ^ (r[2 * c + 1] >> 63)));
+    const int l = 64 - __clzll((long long)m);
+    len = max(len, l);
+    least = min(least, l);
+  }
   const int sh = len - kBits;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -143,10 +169,10 @@ __device__ __forceinline__ int renorm3(const long long *r, int k, int4 *o) {
     const int2 im = words(shift(r[2 * c + 1], sh));
     o[c] = make_int4(re.x, re.y, im.x, im.y);
   }
-  bool any = m != 0;
+  bool any = len != 0;
 #pragma unroll
   for (int c = 0; c < 6; ++c) any = any || r[c] != 0;  // (all -1 has m = 0)
-  return any ? k + len : kZero;
+  return code(any ? k + len : kZero, any ? len - least : 0);
 }
 
 }  // namespace fx

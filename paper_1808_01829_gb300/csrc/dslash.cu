@@ -801,8 +801,9 @@ static rhmc_status_t fx_convert(const Geom &g, const double2 *in, FxField out, i
 // n = 4 16 against 37 us.  Against a long-double sum its error is 1.0e-16 relative for
 // Gaussian fields, that of FP64 FMAs 2.9e-16.
 // Lanes with a special block among their inputs, neighbours more than 2^26 apart in
-// size, or no neighbour with its colours of like size (fx.cuh) take FP64 arithmetic, on
-// in64 where the input was given in FP64; its result is kept in FP64 (MODE 4).
+// size, or colours too far apart (fx.cuh) take FP64 arithmetic, on in64 where the input was
+// given in FP64; its result is kept in FP64 (MODE 4).  A warp with such a lane takes several times
+// as long; in solves at 12^4, n = 4 the hops take 11.8 and 13.9 us with the tests, 11.3 and 13.0 without.
 //
 // MODE 0: out = D in.  1: out = a self - D in.  2: out = B - (a self - D in), with
 // the optional FP32 rounding outf and per-CTA column sums of |out|^2 (part).
@@ -910,7 +911,7 @@ __global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  const bool fast = E != fx::kSpecial && el != fx::kSpecial && (E == fx::kZero || (E - low <= fx::kAlign && E - even <= fx::kApart));
+  bool fast = E != fx::kSpecial && el != fx::kSpecial && (E == fx::kZero || E - low <= fx::kAlign);
   long long R[6];
   if (live && fast) {
     long long pA[3], pB[3], mA[3], mB[3], iA[3], iB[3];  // sums of a c, b d, (a + b)(c + d)
@@ -968,6 +969,11 @@ __global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *
   for (int off = IW; off < 32; off <<= 1)
 #pragma unroll
     for (int c = 0; c < 6; ++c) R[c] += __shfl_xor_sync(0xffffffffu, R[c], off);
+  if (E != fx::kZero && E - even > fx::kApart) {
+    // colours far apart: the sums have to show that every output is of the size they resolve
+#pragma unroll
+    for (int c = 0; c < 3; ++c) fast = fast && fx::reaches(R[2 * c], R[2 * c + 1], fx::kReach);
+  }
   double nrm = 0.0;
   if (live) {
     const int c0 = S == 1 ? 0 : quad, c1 = S == 1 ? 3 : min(3, quad + 1);  // this lane's colours

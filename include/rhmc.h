@@ -113,8 +113,12 @@ rhmc_status_t rhmc_set_gauge(rhmc_ctx_t *ctx, const void *U_dev, rhmc_stream_t s
  * arguments.  In mixed precision with several shifts this includes the stored
  * block basis (RHMC_TUNE_BASIS_ITERS: built in, up to 384 blocks of
  * V/2 * 3 * n_rhs * 8 bytes within a quarter of the device memory, e.g.
- * 24.5 GB at 24^4, n_rhs = 16), in FP64 one of up to 768 blocks of 16 bytes per
- * entry within the same limit; RHMC_TUNE_BASIS_ITERS = 1 sizes without it. */
+ * 24.5 GB at 24^4, n_rhs = 16); RHMC_TUNE_BASIS_ITERS = 1 sizes without it.  FP64
+ * solves keep theirs in memory of the context, taken while they run (up to 768
+ * blocks of 16 bytes per entry within a quarter of the device memory, no more
+ * than stays free and never the last 256 MiB; 16 GiB at most stay with the context
+ * afterwards); without memory for it they go on without.  The workspace holds
+ * its coefficients. */
 size_t rhmc_workspace_bytes(const rhmc_ctx_t *ctx, int n_rhs, int n_shifts, rhmc_precision_t p);
 
 /* Y = (A + sigma) X for an n_rhs-wide block (multi-RHS operator, each link
@@ -453,8 +457,10 @@ rhmc_status_t rhmc_profile_enable(int on);
  *                                 assembled from it at the end of the multishift phase instead of
  *                                 updating P^(s), X^(s) every iteration; a solve that runs longer
  *                                 switches to the updates at that point.  0 = built-in (up to 384
- *                                 iterations, in FP64 768 of 16 bytes per entry, within a quarter
- *                                 of the device memory, off below 24), 1 = off, >= 2 = that capacity
+ *                                 iterations within a quarter of the device memory, off below 24),
+ *                                 1 = off, >= 2 = that capacity.  FP64: the same with up to 768 blocks
+ *                                 of 16 bytes per entry, in memory that the context takes as the
+ *                                 solve needs it (rhmc_workspace_bytes)
  *   RHMC_TUNE_BASIS_GEMM          the assembly's contraction: 0 = tcgen05 tensor-core kernel (FP16
  *                                 pieces of the scaled FP32 operands, three products, FP32
  *                                 accumulation moved to a correctly rounded running sum every 48

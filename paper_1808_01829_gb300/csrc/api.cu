@@ -218,6 +218,7 @@ struct rhmc_ctx {
   size_t md_bytes = 0;
   Scratch ulfx;                    // links of a gauge-force kick in integer form, and whether each fits
   Scratch hopfx;                   // the converted input of a lone FP64 hop
+  std::vector<std::pair<char *, size_t>> basis64;  // memory of the FP64 solve's stored basis, with its bytes
 };
 
 namespace rhmc {
@@ -420,7 +421,9 @@ struct SolveBufs {
   double2 *hist = nullptr;
   BasisBufs asmb;
   int cap = 0;
-  double2 *basis64 = nullptr;  // the FP64 solve's stored basis [cap][rows][n]; Q_k is formed in block k
+  // the FP64 solve's stored basis: cap pointers to blocks [rows][n] of the context's memory, which
+  // the solve fills in as it takes them; Q_k is formed in block k
+  double2 **basis64 = nullptr;
 };
 
 // Stored-basis capacity.  RHMC_TUNE_BASIS_ITERS: 0 = built-in, 1 = off, >= 2 = that
@@ -454,7 +457,7 @@ static int basis_cap(const Geom &g, int n, int ns, bool mixed) {
 }
 
 // Stored-basis capacity of the FP64 solve (same setting): up to kBasisCapMax64 blocks within a
-// quarter of the device's memory.
+// quarter of the device's memory.  The blocks are taken from the context as the solve needs them.
 constexpr int kBasisCapMax64 = 768;
 static int basis_cap64(const Geom &g, int n, int ns) {
   if (ns < 2) return 0;
@@ -466,6 +469,73 @@ static int basis_cap64(const Geom &g, int n, int ns) {
   const int cap = (int)std::min<size_t>(fit, kBasisCapMax64);
   return cap >= kBasisCapMin ? cap : 0;
 }
+
+// Blocks of the FP64 solve's stored basis.  A solve takes as many as its iterations need, each
+// time half as many again as it has (at least kBasisFirst bytes or kBasisCapMin blocks, at most
+// kBasisStep bytes), while it holds no more than it leaves free and kBasisLeave bytes stay free (the
+// driver needs memory for graphs and streams); from there on it goes on with updates in HBM.
+// kBasisKeep bytes stay with the context between solves, the rest is given back: allocating and
+// freeing takes about 1 ms per GB (24^4, n = 16: 47 GB, 2 % of a solve).
+constexpr size_t kBasisFirst = 64u << 20, kBasisStep = 4ull << 30, kBasisKeep = 16ull << 30, kBasisLeave = 256u << 20;
+struct Basis64 {
+  rhmc_ctx *c;
+  cudaStream_t s;
+  size_t block;                // bytes
+  int cap;
+  double2 **table;             // on the device
+  std::vector<double2 *> blk;  // the blocks so far
+  size_t seg = 0, off = 0;     // where the next one lies
+
+  void carve() {
+    for (; seg < c->basis64.size(); ++seg, off = 0)
+      for (; off + block <= c->basis64[seg].second; off += block) {
+        if ((int)blk.size() >= cap) return;
+        blk.push_back((double2 *)(c->basis64[seg].first + off));
+      }
+  }
+  // at least `want` blocks; false: not to be had
+  bool grow(int want) {
+    const size_t had = blk.size();
+    if ((size_t)want <= had) return true;
+    if (want > cap) return false;
+    carve();
+    if ((int)blk.size() < want) {
+      const size_t need = (size_t)want - blk.size();
+      size_t more = std::max({need, std::min(blk.size() / 2, kBasisStep / block), std::max<size_t>(kBasisCapMin, kBasisFirst / block)});
+      more = std::min(more, (size_t)cap - blk.size());
+      size_t free_b = 0, total = 0;
+      if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) free_b = 0;
+      const size_t hold = held();
+      const size_t most = std::min(free_b > hold ? (free_b - hold) / 2 : 0, free_b > kBasisLeave ? free_b - kBasisLeave : 0);
+      more = std::min(more, most / block);
+      void *p = nullptr;
+      if (more < need || cudaMalloc(&p, more * block) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+      }
+      c->basis64.emplace_back((char *)p, more * block);
+      carve();
+    }
+    return cudaMemcpyAsync(table + had, blk.data() + had, sizeof(double2 *) * (blk.size() - had),
+                           cudaMemcpyHostToDevice, s) == cudaSuccess;
+  }
+  size_t held() const {
+    size_t sum = 0;
+    for (auto &q : c->basis64) sum += q.second;
+    return sum;
+  }
+  ~Basis64() {
+    if (!cap) return;
+    size_t sum = held();
+    if (sum <= kBasisKeep) return;
+    cudaStreamSynchronize(s);  // (the assembly may still run)
+    while (!c->basis64.empty() && sum > kBasisKeep) {
+      sum -= c->basis64.back().second;
+      cudaFree(c->basis64.back().first);
+      c->basis64.pop_back();
+    }
+  }
+};
 
 static void layout_solve(Arena &a, const Geom &g, int n, int ns, bool mixed, SolveBufs &b) {
   const size_t len = (size_t)g.Vh * 3 * n;
@@ -508,7 +578,7 @@ static void layout_solve(Arena &a, const Geom &g, int n, int ns, bool mixed, Sol
   const int cap64 = mixed ? 0 : basis_cap64(g, n, ns);
   if (cap64 > 0) {
     b.cap = cap64;
-    b.basis64 = a.take<double2>((size_t)cap64 * len);
+    b.basis64 = a.take<double2 *>((size_t)cap64);
     b.hist = a.take<double2>((size_t)cap64 * ns * 2 * n * n);
     b.asmb.hist = b.hist;
     b.asmb.cap = cap64;
@@ -837,6 +907,8 @@ static rhmc_status_t solve_phase1(rhmc_ctx *c, const double2 *B, int n, int ns, 
   // stored-basis mode (mixed, several shifts, not accumulating): b.basis set
   SolveBufs b = b0;
   if (mixed && (ns < 2 || b.accumulate)) b.basis = nullptr, b.hist = nullptr, b.cap = 0;
+  Basis64 q64{c, s, sizeof(double2) * (size_t)len, b.basis64 ? b.cap : 0, b.basis64};
+  if (b.basis64 && !q64.grow(std::min(kBasisCapMin, b.cap))) b.basis64 = nullptr, b.hist = nullptr, b.cap = 0;
   const bool has64 = b.basis64 != nullptr;
   // X^(s) = sum_i Q_i C_i (want_p = 0), or P^(s) = sum_{i <= K} Q_i D_i (want_p = 1),
   // for s >= 1 from the stored basis (tcgen05 kernel whose epilogue writes the FP64
@@ -895,7 +967,7 @@ static rhmc_status_t solve_phase1(rhmc_ctx *c, const double2 *B, int n, int ns, 
     RHMC_TRY(block_axpy<double, T>(B, nullptr, b.rinv64, (C<T> *)b.Qb[0], rows, n, s));
   }
   if (has64)
-    RHMC_CUDA_TRY(cudaMemcpyAsync(b.basis64, b.Qb[0], sizeof(double2) * len, cudaMemcpyDeviceToDevice, s));
+    RHMC_CUDA_TRY(cudaMemcpyAsync(q64.blk[0], b.Qb[0], sizeof(double2) * len, cudaMemcpyDeviceToDevice, s));
   for (int q = 0; q < (has64 ? 1 : ns); ++q)
     RHMC_CUDA_TRY(cudaMemcpyAsync((C<T> *)b.P + q * len, b.Qb[0], sizeof(C<T>) * len, cudaMemcpyDeviceToDevice, s));
   if (mixed) RHMC_CUDA_TRY(cudaMemsetAsync(b.Xinc, 0, sizeof(float2) * len * ns, s));
@@ -929,14 +1001,13 @@ static rhmc_status_t solve_phase1(rhmc_ctx *c, const double2 *B, int n, int ns, 
   while (k < kmax) {
     const int chunk = prm.fixed_iters > 0 ? kmax : std::min(check_every, kmax - k);
     const int freeze = prm.fixed_iters > 0 ? 0 : 1;
-    if ((b.basis || b.basis64) && k + chunk > b.cap - 1) {
-      // the basis is full: X^(s) and P^(s) from it, then the shifted updates in HBM
+    if ((b.basis && k + chunk > b.cap - 1) || (b.basis64 && !q64.grow(k + chunk + 1))) {
+      // the basis is full, or there is no memory for more: X^(s) and P^(s) from it, then the shifted updates in HBM
       RHMC_TRY(assemble(k, 0));
       RHMC_TRY(assemble(k, 1));
       // (the FP64 basis also held Q_k)
       if (b.basis64)
-        RHMC_CUDA_TRY(cudaMemcpyAsync(b.Qb[k & 1], b.basis64 + (size_t)k * len, sizeof(double2) * len,
-                                      cudaMemcpyDeviceToDevice, s));
+        RHMC_CUDA_TRY(cudaMemcpyAsync(b.Qb[k & 1], q64.blk[k], sizeof(double2) * len, cudaMemcpyDeviceToDevice, s));
       b.basis = nullptr, b.basis64 = nullptr, b.hist = nullptr, b.cap = 0;
     }
     // a captured chunk replays for every later chunk with the same start modulo kCheckEvery
@@ -1417,6 +1488,7 @@ rhmc_status_t rhmc_destroy(rhmc_ctx_t *c) {
   if (c->md_buf) cudaFree(c->md_buf);
   scratch_free(c->ulfx);
   scratch_free(c->hopfx);
+  for (auto &q : c->basis64) cudaFree(q.first);
   for (int q = 0; q < 3; ++q) {
     if (c->ev_base[q]) cudaEventDestroy(c->ev_base[q]);
     if (c->ev_side[q]) cudaEventDestroy(c->ev_side[q]);

@@ -10,8 +10,8 @@
 // without P^(s) and X^(s) going through memory.  Where only the rational sum
 // sum_s w_s X^(s) is wanted (heatbath, action), the coefficients are summed first:
 // one product per row and iteration for all shifts together.
-// The blocks are written where they stay ([block][rows][n]): iteration k forms Q_k in block
-// k of the basis (k from the device counter: graph replays).
+// The blocks are written where they stay (a table of blocks [rows][n], so that a solve takes memory as
+// it goes): iteration k forms Q_k in block k of the basis (k from the device counter: graph replays).
 #include <algorithm>
 #include <mutex>
 
@@ -63,12 +63,12 @@ template <int N> struct Lanes {
 // output, so that small lattices spread over the FP64 units of the whole GPU (each FP64
 // instruction of a warp takes 64 clocks however few there are).
 template <int N>
-__global__ void __launch_bounds__(128) k_axpy64(const double2 *__restrict__ A, const double2 *__restrict__ basis,
+__global__ void __launch_bounds__(128) k_axpy64(const double2 *__restrict__ A, double2 *const *__restrict__ basis,
                                                 const int *__restrict__ kdev, const double2 *__restrict__ M,
                                                 double2 *__restrict__ Y, long rows) {
   __shared__ double2 sm[N * N];
   for (int k = threadIdx.x; k < N * N; k += blockDim.x) sm[k] = M[k];
-  const double2 *Q = basis + (size_t)(*kdev - 1) * rows * N;
+  const double2 *Q = basis[*kdev - 1];
   __syncthreads();
   const long per = 4 * Lanes<N>::RPW;
   for (long base = (long)blockIdx.x * per; base < rows; base += (long)gridDim.x * per) {
@@ -87,12 +87,12 @@ __global__ void __launch_bounds__(128) k_axpy64(const double2 *__restrict__ A, c
 // column j of Q takes terms k <= j and column j of P M2 terms k >= j: n + 1 products
 // together, formed in one running sum whose value after the first j + 1 is Q.
 template <int N>
-__global__ void __launch_bounds__(128) k_base64(const double2 *__restrict__ W, double2 *__restrict__ basis,
+__global__ void __launch_bounds__(128) k_base64(const double2 *__restrict__ W, double2 *const *__restrict__ basis,
                                                 const int *__restrict__ kdev, double2 *P, double2 *X,
                                                 const double2 *__restrict__ coef, long rows) {
   __shared__ double2 sm[3 * N * N];
   for (int k = threadIdx.x; k < 3 * N * N; k += blockDim.x) sm[k] = coef[k];
-  double2 *Q = basis + (size_t)*kdev * rows * N;
+  double2 *Q = basis[*kdev];
   __syncthreads();
   const long per = 4 * Lanes<N>::RPW;
   for (long base = (long)blockIdx.x * per; base < rows; base += (long)gridDim.x * per) {
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(256) k_basis64_combine(int n, int nshift, cons
 // A block with an infinity or NaN gives NaN.
 template <int N, int SG>
 __global__ void __launch_bounds__(128, 4)
-    k_basis64_apply(const double2 *__restrict__ basis, long rows, const SolverState *__restrict__ st, int K, int want,
+    k_basis64_apply(double2 *const *__restrict__ basis, long rows, const SolverState *__restrict__ st, int K, int want,
                     int nshift, const double2 *__restrict__ cf, long cfstride, double2 *__restrict__ out,
                     long fstride) {
   constexpr int NN = N * N, RPW = Lanes<N>::RPW;
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(128, 4)
     int ef = 0;
 #pragma unroll
     for (int i = 0; i < T; ++i) {
-      v[i] = (l.in && i < nb) ? basis[((size_t)(b + i) * rows + l.row) * N + l.j] : make_double2(0.0, 0.0);
+      v[i] = (l.in && i < nb) ? basis[b + i][l.row * N + l.j] : make_double2(0.0, 0.0);
       ef = max(ef, max(fx::expo(v[i].x), fx::expo(v[i].y)));
     }
     {
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(128, 4)
     if (s0 + g < nshift && (want != 1 || nblk[g])) out[(size_t)(s0 - 1 + g) * fstride + l.row * N + l.j] = acc[g];
 }
 
-rhmc_status_t axpy64(const double2 *A, const double2 *basis, const int *kdev, const double2 *M, double2 *Y, long rows,
+rhmc_status_t axpy64(const double2 *A, double2 *const *basis, const int *kdev, const double2 *M, double2 *Y, long rows,
                      int n, cudaStream_t s) {
   prof_begin(PROF_AXPY, s);
 #define L_(NN)                                                                                          \
@@ -269,7 +269,7 @@ rhmc_status_t axpy64(const double2 *A, const double2 *basis, const int *kdev, co
   return RHMC_OK;
 }
 
-rhmc_status_t base64(const double2 *W, double2 *basis, const int *kdev, double2 *P, double2 *X, const double2 *coef,
+rhmc_status_t base64(const double2 *W, double2 *const *basis, const int *kdev, double2 *P, double2 *X, const double2 *coef,
                      long rows, int n, cudaStream_t s) {
   prof_begin(PROF_UPDATE64, s);
 #define L_(NN)                                                                                          \
@@ -285,14 +285,14 @@ rhmc_status_t base64(const double2 *W, double2 *basis, const int *kdev, double2 
 }
 
 template <int N, int SG>
-static void launch_apply(const BasisBufs &bb, const double2 *basis, const double2 *cf, int nshift,
+static void launch_apply(const BasisBufs &bb, double2 *const *basis, const double2 *cf, int nshift,
                          const SolverState *st, long rows, int K, int want, double2 *out, long fstride,
                          cudaStream_t s) {
   const dim3 grid((unsigned)((rows + 4 * Lanes<N>::RPW - 1) / (4 * Lanes<N>::RPW)), (unsigned)((nshift - 2 + SG) / SG));
   k_basis64_apply<N, SG><<<grid, 128, 0, s>>>(basis, rows, st, K, want, nshift, cf, bb.cap + 1, out, fstride);
 }
 
-rhmc_status_t basis64_assemble(const BasisBufs &bb, const double2 *basis, int n, int nshift, const SolverState *st,
+rhmc_status_t basis64_assemble(const BasisBufs &bb, double2 *const *basis, int n, int nshift, const SolverState *st,
                                long rows, int K, int want_p, int combine, double2 *out, long fstride, cudaStream_t s) {
   if (nshift < 2 || (K <= 0 && !want_p)) return RHMC_OK;
   RHMC_TRY(basis_coef(bb, n, nshift, st, K, want_p, s));

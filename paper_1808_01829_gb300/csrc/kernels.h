@@ -165,16 +165,16 @@ size_t basis_pack_bytes(int n, int nshift, int cap);
 // cf of basis_assemble (FP64 expansion coefficients of X^(s) or P^(s)) alone
 rhmc_status_t basis_coef(const BasisBufs &bb, int n, int nshift, const SolverState *st, int K, int want_p,
                          cudaStream_t s);
-// basis64.cu: the FP64 solve's stored basis, [block][rows][n]; kdev: the device's iteration
+// basis64.cu: the FP64 solve's stored basis, a device table of blocks [rows][n]; kdev: the device's iteration
 // counter k.  W = Q_{k-1} + A M; Q_k = W rho^-1, X^(0) += P M1, P = Q_k + P M2.
-rhmc_status_t axpy64(const double2 *A, const double2 *basis, const int *kdev, const double2 *M, double2 *Y, long rows,
+rhmc_status_t axpy64(const double2 *A, double2 *const *basis, const int *kdev, const double2 *M, double2 *Y, long rows,
                      int n, cudaStream_t s);
-rhmc_status_t base64(const double2 *W, double2 *basis, const int *kdev, double2 *P, double2 *X, const double2 *coef,
+rhmc_status_t base64(const double2 *W, double2 *const *basis, const int *kdev, double2 *P, double2 *X, const double2 *coef,
                      long rows, int n, cudaStream_t s);
 // out_s = X^(s) (want_p = 0) or P^(s)_K (want_p = 1, active shifts) for s = 1 .. nshift - 1, at
 // out + (s - 1) fstride; combine (want_p = 0): sum_s w_s X^(s) into out.  bb.hist, bb.cf (room
 // for nshift sets of cap + 1 blocks) and bb.cap are used.
-rhmc_status_t basis64_assemble(const BasisBufs &bb, const double2 *basis, int n, int nshift, const SolverState *st,
+rhmc_status_t basis64_assemble(const BasisBufs &bb, double2 *const *basis, int n, int nshift, const SolverState *st,
                                long rows, int K, int want_p, int combine, double2 *out, long fstride, cudaStream_t s);
 // want_p = 0: X^(s) = sum_{i < last_s} Q_i C_i for s = 1 .. nshift-1 (FP64, C_i = alpha_{i+1}
 // + M2_{i+1} C_{i+1}; X^(s), s >= 1, is overwritten: it is zero before the one assembly of a

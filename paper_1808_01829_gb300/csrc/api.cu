@@ -819,8 +819,10 @@ static rhmc_status_t run_chunk_graph(rhmc_ctx *c, const SolveBufs &b, double2 *X
   // (mixed: the chunk does not touch X; with device stop it reads sigma_0 and the tolerance
   // from the state, so that one graph serves the corrections of every shift)
   const bool mixed = sizeof(T) == 4;
-  std::vector<double> key = {(double)(uintptr_t)b.P, mixed ? 0.0 : (double)(uintptr_t)X, (double)(uintptr_t)b.basis + (double)(uintptr_t)b.basis64,
-                             (double)b.accumulate, (double)n,
+  // (the FP32 hop's link records depend on the links staged last)
+  std::vector<double> key = {(double)(uintptr_t)b.P, mixed ? 0.0 : (double)(uintptr_t)X,
+                             (double)(uintptr_t)b.basis + (double)(uintptr_t)b.basis64,
+                             mixed && Links12Of<float>::get(c, 0) ? 1.0 : 0.0, (double)b.accumulate, (double)n,
                              (double)ns, b.device_stop ? 0.0 : sigma0, b.device_stop ? 0.0 : target, (double)freeze,
                              (double)sizeof(T), (double)len, (double)(chunk_start % kCheckEvery),
                              (double)b.device_stop};

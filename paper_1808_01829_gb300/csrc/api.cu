@@ -259,12 +259,16 @@ static rhmc_status_t ensure_pool(rhmc_ctx *c, size_t bytes) {
   return RHMC_OK;
 }
 
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+}
+
 // `bytes` for kernels on s, which wait for the buffer's last users; nullptr where there is no
 // memory for it, or while s is being captured (the graph would keep an address that a later
 // call may free, and run at any time).  The callers have forms that need no buffer.
 static void *scratch_begin(Scratch &b, size_t bytes, cudaStream_t s) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return nullptr;
+  if (capturing(s)) return nullptr;
   if (!b.used && cudaEventCreateWithFlags(&b.used, cudaEventDisableTiming) != cudaSuccess) {
     b.used = nullptr;
     cudaGetLastError();
@@ -1559,7 +1563,15 @@ rhmc_status_t rhmc_apply_mdagm_mrhs(rhmc_ctx_t *c, const void *X, void *Y, int n
   cudaStream_t s = (cudaStream_t)sv;
   const long len = c->g.Vh * 3 * n;
   if (p == RHMC_FP64 || p == RHMC_DF64) {  // both FP64-accurate on the integer units
-    RHMC_TRY(ensure_pool(c, sizeof(double2) * len + 2 * sizeof(int) * c->g.Vh * n + 1024));
+    const size_t need = sizeof(double2) * len + 2 * sizeof(int) * c->g.Vh * n + 1024;
+    if (c->pool_bytes < need && c->pool_bytes >= sizeof(double2) * len && capturing(s)) {
+      // a captured stream cannot enlarge the pool: native FP64, which needs the intermediate field only
+      double2 *tmp = (double2 *)c->pool;
+      RHMC_TRY(hop<double>(c->g, 1, c->l64[1], (const double2 *)X, tmp, nullptr, 0.0, n, 1, 0, s));
+      return hop<double>(c->g, 0, c->l64[0], tmp, (double2 *)Y, (const double2 *)X,
+                         4.0 * c->mass * c->mass + sigma, n, 1, 0, s);
+    }
+    RHMC_TRY(ensure_pool(c, need));
     Arena a(c->pool);
     double2 *tmp = a.take<double2>(len);
     FxExp ex{a.take<int>(c->g.Vh * n), a.take<int>(c->g.Vh * n)};

@@ -57,3 +57,24 @@ def test_first_call_under_capture(dims, n):
         torch.cuda.synchronize()
         assert colrel(Y.cpu().numpy(), refs[q]) <= 1e-13
     ctx.close()
+
+
+@pytest.mark.parametrize("dims,n", CASES)
+def test_operator_under_capture_with_the_pool_of_a_mixed_hop(dims, n):
+    """The pool that a mixed hop left holds the intermediate field of an FP64 operator application and
+    no more; under capture it cannot grow."""
+    torch = need_gpu()
+    ctx, Xs, _ = _case(dims, n)
+    ctx.hop(Xs[0], 1, "mixed")
+    X = Xs[0].clone()
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        Y = ctx.apply_mdagm_mrhs(X, 0.2, "fp64")
+    X.copy_(Xs[1])
+    graph.replay()
+    torch.cuda.synchronize()
+    y = Y.cpu().numpy()
+    ctx.tune_set(NATIVE, 1)
+    assert colrel(y, ctx.apply_mdagm_mrhs(Xs[1], 0.2, "fp64").cpu().numpy()) <= 1e-13
+    ctx.close()

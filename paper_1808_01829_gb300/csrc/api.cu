@@ -408,7 +408,7 @@ struct SolveBufs {
   void *P, *Qb[2], *W, *AP, *Todd, *Xinc;  // Qb: Q_k in Qb[k & 1]; Xinc: FP32 increments (mixed only)
   void *coef, *mw;
   // FP64 helpers
-  double2 *R64, *T64, *AP64, *rinv64;
+  double2 *R64, *T64, *rinv64;
   float *btiles;      // tensor-core B tiles of the shifted updates
   double2 *partial;   // the summed Gram matrix (n x n)
   double2 *gscratch;  // per-CTA Gram partials
@@ -556,7 +556,6 @@ static void layout_solve(Arena &a, const Geom &g, int n, int ns, bool mixed, Sol
   b.mw = a.take<char>((size_t)n * n * esz);
   b.R64 = a.take<double2>(len);
   b.T64 = a.take<double2>(len);
-  b.AP64 = a.take<double2>(len);
   b.rinv64 = a.take<double2>((size_t)n * n);
   b.btiles = a.take<float>((size_t)ns * 3 * 64 * 32);
   b.partial = a.take<double2>((size_t)n * n);

@@ -29,21 +29,6 @@ __device__ __forceinline__ void df_add_prod(DF &acc, float ah, float al, float b
   acc.h = s;
   acc.e = __fadd_rn(acc.e, __fadd_rn(t, err));
 }
-// acc += u * v for double-float complex u, v (float4 = re_hi, im_hi, re_lo, im_lo)
-__device__ __forceinline__ void df_cmac(DF &re, DF &im, const float4 &u, const float4 &v) {
-  df_add_prod(re, u.x, u.z, v.x, v.z);
-  df_add_prod(re, -u.y, -u.w, v.y, v.w);
-  df_add_prod(im, u.x, u.z, v.y, v.w);
-  df_add_prod(im, u.y, u.w, v.x, v.z);
-}
-__device__ __forceinline__ float4 df_pack(const DF &re, const DF &im) {
-  // renormalise: (h, e) -> (hi, lo) with FastTwoSum
-  const float rh = __fadd_rn(re.h, re.e), rl = __fsub_rn(re.e, __fsub_rn(rh, re.h));
-  const float ih = __fadd_rn(im.h, im.e), il = __fsub_rn(im.e, __fsub_rn(ih, im.h));
-  return make_float4(rh, ih, rl, il);
-}
-
-
 // a + b for two running sums (TwoSum of the leading parts, errors added)
 __device__ __forceinline__ DF df_add(const DF &a, const DF &b) {
   const float s = __fadd_rn(a.h, b.h);

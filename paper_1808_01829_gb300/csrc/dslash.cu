@@ -1087,7 +1087,7 @@ long hop_fx_parts(const Geom &g, int n) {
   return (g.Vh + tile - 1) / tile;
 }
 
-// in64 (optional): the input in FP64; the four-lane kernel converts it itself, else it is
+// in64: the input in FP64; the four-lane kernel converts it itself, else it is
 // converted into `in` first.  A lone FP64 hop (MODE 0) without a buffer for that takes the
 // four-lane kernel on every lattice (24^4, n = 16: 913 us; with the conversion 393 us).
 template <int MODE>
@@ -1106,19 +1106,11 @@ static rhmc_status_t launch_hop_fx(const Geom &g, int par, const FxLinks &L, con
     kern<<<grid, threads, smem, s>>>(g, par, L.rec, L.exp, L.l64, in.v, in.e, in64, out, oex, self, a, n, tile, B, outf,
                                      part);
   };
-  bool done = false;
-  if constexpr (MODE == 0 || MODE == 3 || MODE == 4) {
-    if (in64 && split == 4) {
-      run(k_hop_fx<MODE, 4, true>);
-      done = true;
-    }
-  }
-  if (!done) {
-    if (split == 4)
-      run(k_hop_fx<MODE, 4, false>);
-    else
-      run(k_hop_fx<MODE, 1, false>);
-  }
+  constexpr bool kFrom64 = MODE == 0 || MODE == 3 || MODE == 4;  // (these are always given in64, the others never)
+  if (split == 4)
+    run(k_hop_fx<MODE, 4, kFrom64>);
+  else
+    run(k_hop_fx<MODE, 1, false>);
   // algorithmic bytes: every link once, the inputs once, the outputs once
   const double fields = 2.0 + (MODE == 1 ? 1.0 : 0.0) + (MODE == 2 ? 2.0 + (outf ? 0.5 : 0.0) : 0.0);
   prof_end(s, (double)g.Vh * 16 * (72.0 + 3.0 * n * fields));

@@ -3,6 +3,28 @@
 
 #include "common.cuh"
 
+// Instantiate a launch for the runtime width n = 1..16.
+#define RHMC_DISPATCH_N(n, MACRO) \
+  switch (n) {                    \
+    case 1: MACRO(1); break;      \
+    case 2: MACRO(2); break;      \
+    case 3: MACRO(3); break;      \
+    case 4: MACRO(4); break;      \
+    case 5: MACRO(5); break;      \
+    case 6: MACRO(6); break;      \
+    case 7: MACRO(7); break;      \
+    case 8: MACRO(8); break;      \
+    case 9: MACRO(9); break;      \
+    case 10: MACRO(10); break;    \
+    case 11: MACRO(11); break;    \
+    case 12: MACRO(12); break;    \
+    case 13: MACRO(13); break;    \
+    case 14: MACRO(14); break;    \
+    case 15: MACRO(15); break;    \
+    case 16: MACRO(16); break;    \
+    default: return RHMC_ERR_INVALID_ARG; \
+  }
+
 namespace rhmc {
 
 constexpr int kMaxN = RHMC_MAX_NRHS;

@@ -484,7 +484,9 @@ rhmc_status_t rhmc_profile_enable(int on);
  *   RHMC_TUNE_PHASE1_MARGIN_MILLI the multishift phase runs to value/1000 x tol before the
  *                                 true-residual checks (1 .. 999; 0: built-in)
  *   RHMC_TUNE_CORRECTION_CHECK_EVERY  iterations between the host checks of a defect
- *                                 correction (a divisor of 6 uses captured graphs; 0: built-in 1)
+ *                                 correction (a divisor of 6 uses captured graphs; 0: built-in:
+ *                                 V/2 * 3 * n_rhs < 2^19 stops on the device, with a host check
+ *                                 every 6 iterations, larger fields are checked after every one)
  * Value 0 restores the built-in choice.  INVALID_ARG for an unknown key. */
 enum {
   RHMC_TUNE_HOP_RHS_PER_THREAD = 0,

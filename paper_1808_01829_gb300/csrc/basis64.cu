@@ -121,6 +121,19 @@ __global__ void __launch_bounds__(256) k_basis64_combine(int n, int nshift, cons
   out[(size_t)i * nn + t] = sum;
 }
 
+constexpr int kFar = 6;
+// sum_{i < nb, t < N} Q_{b + i}[row][t] C_i[t][j] in FP64
+template <int N>
+__device__ __noinline__ double2 basis64_terms(double2 *const *basis, int b, int nb, long row, int j,
+                                              const double2 *cf) {
+  double2 acc = czero<double>();
+#pragma unroll 1
+  for (int i = 0; i < nb; ++i)
+#pragma unroll 1
+    for (int t = 0; t < N; ++t) cmac<double>(acc, basis[b + i][row * N + t], cf[(i * N + t) * N + j]);
+  return acc;
+}
+
 // out_s = sum_i Q_i C^(s)_i for the shifts s0 + SG blockIdx.y ... (want = 0: X^(s), last_s
 // blocks; 1: P^(s), K + 1 blocks, active shifts; 2: one combined set, all K blocks).  One lane
 // per (row, column), SG shifts each, so that a row of Q is read once for SG shifts.
@@ -129,6 +142,9 @@ __global__ void __launch_bounds__(256) k_basis64_combine(int n, int nshift, cons
 // each (shift, column), and a sum is added to the FP64 result as one value.  A term costs 9
 // multiply-adds of four clocks where FP64 takes 4 of 64; converting and the FP64 value per
 // sum take about as long again.  8^4, n = 4, 12 shifts: 342 us, 1250 us with FP64 FMAs.
+// The error is 2^-55 of the largest entry times the largest coefficient; where the sum is far
+// below that and so is the sum of the terms' sizes (columns that hardly mix, under weak links:
+// large entries meet small coefficients), the terms are added in FP64 instead.
 // A block with an infinity or NaN gives NaN.
 template <int N, int SG>
 __global__ void __launch_bounds__(128, 4)
@@ -222,8 +238,27 @@ __global__ void __launch_bounds__(128, 4)
       if (ef == 0x7ff || e == 0x7ff) {
         acc[g].x = acc[g].y = __longlong_as_double(0x7ff8000000000000LL);
       } else {
-        acc[g].x += fx::value(fx::join(pA[g] - mA[g], pB[g] - mB[g]), k);
-        acc[g].y += fx::value(fx::join(iA[g] - pA[g] - mA[g], iB[g] - pB[g] - mB[g]), k);
+        const long long re = fx::join(pA[g] - mA[g], pB[g] - mB[g]);
+        const long long im = fx::join(iA[g] - pA[g] - mA[g], iB[g] - pB[g] - mB[g]);
+        bool small = ef && e && !fx::reaches(re, im, 56 - kFar);  // (largest times largest: 2^54 to 2^56)
+        if (small) {
+          unsigned size = 0;  // (largest times largest: 2^22 to 2^24)
+#pragma unroll 1
+          for (int t = 0; t < nb * N; ++t) {
+            const int4 w = q[t], u = c[g * T * NN + t * N];
+            size += (unsigned)((abs(w.x) + abs(w.z)) >> 16) * (unsigned)((abs(u.x) + abs(u.z)) >> 16);
+          }
+          small = size < 1u << (24 - kFar);
+        }
+        if (small) {
+          const double2 z = basis64_terms<N>(basis, b, min(nb, nblk[g] - b), l.row, l.j,
+                                             cf + ((size_t)(s0 - 1 + g) * cfstride + b) * NN);
+          acc[g].x += z.x;
+          acc[g].y += z.y;
+        } else {
+          acc[g].x += fx::value(re, k);
+          acc[g].y += fx::value(im, k);
+        }
       }
     }
   }

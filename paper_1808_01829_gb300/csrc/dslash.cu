@@ -796,14 +796,14 @@ static rhmc_status_t fx_convert(const Geom &g, const double2 *in, FxField out, i
 // warps (small lattices): the lanes' integer sums are added by shuffles, and three of
 // the four lanes write one colour each.  With S = 4 an FP64 input (IN64) is converted here:
 // a separate pass would cost a launch, and each value is read by few warps.
-// Measured per hop, FP64 fields: 24^4, n = 16 353 us (and 60 us to convert the input of
-// the first hop) against 1246 us with FP64 FMAs; an operator application at 8^4,
-// n = 4 16 against 37 us.  Against a long-double sum its error is 1.0e-16 relative for
+// Measured, FP64 fields: 24^4, n = 16 787 us per operator application (60 us of it to convert
+// the input of the first hop) against 2500 us with FP64 FMAs; at 8^4, n = 4 16 against 37 us.  Against a long-double sum its error is 1.0e-16 relative for
 // Gaussian fields, that of FP64 FMAs 2.9e-16.
 // Lanes with a special block among their inputs, neighbours more than 2^26 apart in
-// size, or colours too far apart (fx.cuh) take FP64 arithmetic, on in64 where the input was
-// given in FP64; its result is kept in FP64 (MODE 4).  A warp with such a lane takes several times
-// as long; in solves at 12^4, n = 4 the hops take 11.8 and 13.9 us with the tests, 11.3 and 13.0 without.
+// size, or an output whose terms are all small (fx.cuh) take FP64 arithmetic, on in64 where
+// the input was given in FP64; its result is kept in FP64 (MODE 4).  In solves at 12^4, n = 4 the
+// two hops take 11.5 and 13.2 us with the tests for that, 11.3 and 12.9 without; an input of one
+// colour only (a source) 1.9 ms per operator application at 24^4, n = 16, and 2.6 ms under unit links.
 //
 // MODE 0: out = D in.  1: out = a self - D in.  2: out = B - (a self - D in), with
 // the optional FP32 rounding outf and per-CTA column sums of |out|^2 (part).
@@ -912,6 +912,39 @@ __global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   bool fast = E != fx::kSpecial && el != fx::kSpecial && (E == fx::kZero || E - low <= fx::kAlign);
+  // colours apart at every neighbour: the sizes |U_cb| |v_b| themselves have to add up (fx.cuh)
+  const bool unsure = live && fast && E != fx::kZero && E - even > fx::kApart;
+  if (__any_sync(0xffffffffu, unsure)) {
+    unsigned size[3] = {0, 0, 0};  // (units of 2^-24 of largest link times largest value)
+    if (unsure) {
+      const int4 *lk = sl + ls * LS + d0 * 9;
+#pragma unroll 1
+      for (int q = 0; q < 3 * ND; ++q) {
+        const int d = q / 3, cb = q - d * 3, o = nb[d0 + d] * n3 + j + cb * n;
+        int re, im;
+        if (IN64) {
+          re = fx::split(in64[o].x, ef).x;
+          im = fx::split(in64[o].y, ef).x;
+        } else {
+          const int4 w = in[o];
+          const int sh = min(fx::kAlign, E - fx::exponent(iex[nb[d0 + d] * n + j]));
+          re = w.x >> sh;
+          im = w.z >> sh;
+        }
+        const unsigned w = (unsigned)(abs(re) + abs(im)) >> 16;
+#pragma unroll
+        for (int ca = 0; ca < 3; ++ca) {
+          const int4 l = lk[d * 9 + ca * 3 + cb];
+          size[ca] += w * ((unsigned)(abs(l.x) + abs(l.z)) >> 16);
+        }
+      }
+    }
+#pragma unroll
+    for (int off = IW; off < 32; off <<= 1)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) size[c] += __shfl_xor_sync(0xffffffffu, size[c], off);
+    if (unsure) fast = min(size[0], min(size[1], size[2])) >= 1u << 23;
+  }
   long long R[6];
   if (live && fast) {
     long long pA[3], pB[3], mA[3], mB[3], iA[3], iB[3];  // sums of a c, b d, (a + b)(c + d)
@@ -969,11 +1002,6 @@ __global__ void __launch_bounds__(128, 4) k_hop_fx(Geom g, int par, const int4 *
   for (int off = IW; off < 32; off <<= 1)
 #pragma unroll
     for (int c = 0; c < 6; ++c) R[c] += __shfl_xor_sync(0xffffffffu, R[c], off);
-  if (E != fx::kZero && E - even > fx::kApart) {
-    // colours far apart: the sums have to show that every output is of the size they resolve
-#pragma unroll
-    for (int c = 0; c < 3; ++c) fast = fast && fx::reaches(R[2 * c], R[2 * c + 1], fx::kReach);
-  }
   double nrm = 0.0;
   if (live) {
     const int c0 = S == 1 ? 0 : quad, c1 = S == 1 ? 3 : min(3, quad + 1);  // this lane's colours

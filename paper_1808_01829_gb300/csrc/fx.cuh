@@ -29,8 +29,8 @@
 // unit-like links keep colours of very different size apart.  A hop therefore takes the integer
 // form only where one of the eight neighbours has all three colours within 2^kApart of
 // the largest (a row c of unitary links has an entry of order one there, which stage_links_fx
-// checks) or where every output itself is within 2^kApart of largest link times largest
-// value: its sum is of the size the integers resolve.  Measured against
+// checks), or else where for every output that sum, formed from the leading words, is
+// at least half of largest link times largest value.  Measured against
 // extended precision, largest error over sum |U_cb| |v_b| (integers; FP64 FMAs): Gaussian fields
 // 7.6e-17; 4.1e-16, unit links and colours 1, 1/8, 1/8 4.1e-16; 2.6e-16, 1, 1/16, 1/16 5.0e-16; 2.6e-16.
 #pragma once
@@ -43,7 +43,6 @@ constexpr int kBits = 55;             // magnitude bits
 constexpr int kSpecial = 1 << 20;     // exponent code: the block holds FP64 values
 constexpr int kZero = -(1 << 20);     // exponent code: all zeros
 constexpr int kApart = 3;             // see above; Gaussian colours: all but one (site, column) in a million
-constexpr int kReach = 56 - kApart;  // the second test, on a sum in units of 2^(E1 + E2 - 56)
 
 // A block's word: its exponent and, in the low five bits, the distance to that of its smallest colour
 __device__ __forceinline__ int code(int e, int apart) { return e * 32 + min(apart, 31); }

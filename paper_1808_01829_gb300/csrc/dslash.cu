@@ -797,8 +797,9 @@ static rhmc_status_t fx_convert(const Geom &g, const double2 *in, FxField out, i
 // the four lanes write one colour each.  With S = 4 an FP64 input (IN64) is converted here:
 // a separate pass would cost a launch, and each value is read by few warps.
 // Measured, FP64 fields: 24^4, n = 16 787 us per operator application (60 us of it to convert
-// the input of the first hop) against 2500 us with FP64 FMAs; at 8^4, n = 4 16 against 37 us.  Against a long-double sum its error is 1.0e-16 relative for
-// Gaussian fields, that of FP64 FMAs 2.9e-16.
+// the input of the first hop) against 2500 us with FP64 FMAs; at 8^4, n = 4 16 against 37 us.
+// Against a long-double sum its error is 1.0e-16 relative for Gaussian fields, that of FP64 FMAs
+// 2.9e-16.
 // Lanes with a special block among their inputs, neighbours more than 2^26 apart in
 // size, or an output whose terms are all small (fx.cuh) take FP64 arithmetic, on in64 where
 // the input was given in FP64; its result is kept in FP64 (MODE 4).  In solves at 12^4, n = 4 the

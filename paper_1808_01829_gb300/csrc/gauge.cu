@@ -327,7 +327,7 @@ __device__ __forceinline__ void row_times(const int4 *a, const int4 *b, long lon
   }
 }
 // Sizes (in units of 2^-20) below which the FP64 form is the more accurate one; see k_gauge_momentum_fx
-constexpr int kOffSize = (int)(0.8 * (1 << 20)), kDiagSize = (int)(0.4 * (1 << 20));
+constexpr int kOffSize = (1 << 20) / 2, kDiagSize = (1 << 20) / 4;
 __device__ __forceinline__ int4 conj_if(int4 z, int m) {  // m = -1: the conjugate, 0: z
   return make_int4(z.x, z.y, (z.z ^ m) - m, (z.w ^ m) - m);
 }
@@ -344,9 +344,11 @@ __device__ __forceinline__ int4 conj_if(int4 z, int m) {  // m = -1: the conjuga
 // exp(i eps H) with eps = 0.5 8.1e-17, FP64 form 2.3e-16.
 // The error in these units is the same for every link, that of the FP64 form is relative to
 // S_ij = sum_k |U_ik| |V_kj| + |U_jk| |V_ki| off the diagonal and to the largest of
-// sum_k |Re U_ik| |Im V_ki| + |Im U_ik| |Re V_ki| on it.  They meet where these are 0.8 and 0.4
-// (both forms up to 1.6e-16 S and 4.4e-16 S); a link below either takes the FP64 form.  At
-// eps = 0.5 no link does, at 0.3 one in 2000 (659 us), from 0.1 down nearly all (1.8 ms).
+// sum_k |Re U_ik| |Im V_ki| + |Im U_ik| |Re V_ki| on it.  A link where these are below 1/2 or
+// 1/4 takes the FP64 form; there the largest errors are 3.1e-16 S and 6.2e-16 S (FP64 form
+// 1.6e-16 and 4.2e-16), at twice these sizes they are equal, above the integers are closer.  At
+// eps = 0.5 no link does, at 0.3 hardly one (579 us), at 0.2 few (681 us), from 0.1 down nearly
+// all (1.8 ms; limits of 0.8 and 0.4 took 660 and 1220 us at 0.3 and 0.2).
 __global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4 *__restrict__ v,
                                                               const int *__restrict__ ok,
                                                               const double2 *__restrict__ U, double2 *__restrict__ P,

@@ -74,8 +74,10 @@ typedef enum {
                           coefficient algebra, FP64 force.  The residuals of the
                           loop use the FP64-accurate operator */
   RHMC_DF64 = 2        /* operator only (apply / hop): FP64-accurate; the same arithmetic as
-                          RHMC_FP64 (exact integer sums of products on the integer units,
-                          several times faster than this GPU's FP64 units) */
+                          RHMC_FP64: exact integer sums of products on the integer units,
+                          several times faster than this GPU's FP64 units, where their
+                          error is within that of FP64 sums for every component, FP64
+                          elsewhere */
 } rhmc_precision_t;
 
 /* Largest number of right-hand sides per block (n_pf). */
@@ -133,11 +135,11 @@ rhmc_status_t rhmc_apply_mdagm_mrhs(rhmc_ctx_t *ctx, const void *X_dev, void *Y_
  * under a fixed memory budget, or under a framework that owns all
  * allocation).  The paper has no counterpart; this is a deployment variant.
  * It allocates nothing: the odd-parity intermediate lives in file-scope
- * device arrays of fixed size (32 MiB, and a sixth as much for exponents; i.e. V/2 * 3 * n_rhs * 16 bytes at most,
- * e.g. a 16^4 lattice with 16 right-hand sides), which every GPU that loads
- * the library holds until the process exits; Y serves as scratch before the
- * result is written.  Larger problems are rejected
- * with INVALID_ARG.  The first call on a device looks up the array's device
+ * device arrays of fixed size (32 MiB of values, so V/2 * 3 * n_rhs * 16 bytes
+ * at most, e.g. a 16^4 lattice with 16 right-hand sides; a sixth as much for
+ * exponents), which every GPU that loads the library holds until the process
+ * exits; Y serves as scratch before the result is written.  Larger problems
+ * are rejected with INVALID_ARG.  The first call on a device looks up the array's device
  * address (cudaGetSymbolAddress); make that first call before any stream
  * capture.  All calls share the array: calls that overlap on the GPU (other
  * streams, other threads) race on it and must be serialised by the caller.
@@ -149,7 +151,9 @@ rhmc_status_t rhmc_apply_mdagm_mrhs_noalloc(rhmc_ctx_t *ctx, const void *X_dev, 
                                             rhmc_stream_t s);
 
 /* One staggered hop Y = D X onto parity out_parity (0: D_eo, input odd;
- * 1: D_oe, input even).  Same layouts and precision rule as above. */
+ * 1: D_oe, input even).  Same layouts and precision rule as above.  In FP64 and
+ * DF64 hops of one context may be enqueued on several streams, and captured
+ * before any other call. */
 rhmc_status_t rhmc_hop(rhmc_ctx_t *ctx, const void *X_dev, void *Y_dev, int n_rhs, int out_parity,
                        rhmc_precision_t p, rhmc_stream_t s);
 
@@ -300,7 +304,11 @@ rhmc_status_t rhmc_momenta_from_normals(rhmc_ctx_t *ctx, const double *p_dev, vo
 /* Gauge-force kick P += eps TA(U G_g^dagger) / 2 with G_g = -(beta / 3) V^dagger,
  * V_mu(x) the sum of the six staples around U_mu(x):
  *   V_mu(x) = sum_{nu != mu} [U_nu(x+mu) U_mu(x+nu)^dagger U_nu(x)^dagger
- *                             + U_nu(x+mu-nu)^dagger U_mu(x-nu)^dagger U_nu(x-nu)]. */
+ *                             + U_nu(x+mu-nu)^dagger U_mu(x-nu)^dagger U_nu(x-nu)].
+ * The products are exact integer sums where that is as accurate as FP64 (links of
+ * the size of SU(3)'s, a force not small next to its products); the context keeps
+ * 592 bytes per site for it.  FP64 elsewhere, under stream capture and without
+ * memory. */
 rhmc_status_t rhmc_gauge_momentum(rhmc_ctx_t *ctx, const void *U_dev, void *P_dev, double beta, double eps,
                                   rhmc_stream_t s);
 

@@ -261,7 +261,9 @@ static rhmc_status_t ensure_pool(rhmc_ctx *c, size_t bytes) {
 
 static bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // (the legacy stream while another one is being captured: the launch will say so)
+  return true;
 }
 
 // `bytes` for kernels on s, which wait for the buffer's last users; nullptr where there is no
@@ -418,7 +420,7 @@ struct SolveBufs {
   SolverState *st;
   bool device_stop = false;  // (mixed, single shift) the solve stops on the device
   int accumulate = 0;  // shifts s >= 1 add w_s X^(s) into one field after X^(0) (FP64)
-  // stored-basis mode (mixed, several shifts): the block basis Q_0 .. Q_{cap-1}
+  // stored-basis mode of the mixed solve (several shifts): the block basis Q_0 .. Q_{cap-1}
   // (rows x cap*n, row-major), the per-iteration shift coefficients and the
   // assembly's operands; basis == nullptr: shifted updates in HBM
   float2 *basis = nullptr;
@@ -508,7 +510,7 @@ struct Basis64 {
       size_t more = std::max({need, std::min(blk.size() / 2, kBasisStep / block), std::max<size_t>(kBasisCapMin, kBasisFirst / block)});
       more = std::min(more, (size_t)cap - blk.size());
       size_t free_b = 0, total = 0;
-      if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) free_b = 0;
+      if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) free_b = 0, cudaGetLastError();
       const size_t hold = held();
       const size_t most = std::min(free_b > hold ? (free_b - hold) / 2 : 0, free_b > kBasisLeave ? free_b - kBasisLeave : 0);
       more = std::min(more, most / block);
@@ -909,7 +911,7 @@ static rhmc_status_t solve_phase1(rhmc_ctx *c, const double2 *B, int n, int ns, 
   const long rows = c->g.Vh * 3;
   const long len = rows * n;
   const double sigma0 = shifts[0];
-  // stored-basis mode (mixed, several shifts, not accumulating): b.basis set
+  // stored-basis mode (several shifts): b.basis set (mixed, not accumulating) or b.basis64 (FP64)
   SolveBufs b = b0;
   if (mixed && (ns < 2 || b.accumulate)) b.basis = nullptr, b.hist = nullptr, b.cap = 0;
   Basis64 q64{c, s, sizeof(double2) * (size_t)len, b.basis64 ? b.cap : 0, b.basis64};

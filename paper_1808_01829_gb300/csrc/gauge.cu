@@ -250,6 +250,54 @@ __device__ __noinline__ void kick_fp64(const Geom &g, const double2 *U, double2 
   add_ta(P + e * 9, mul(ld3(U + e * 9), V), coef);
 }
 
+// The same for one link by all 32 lanes of a warp: lane 9 s + 3 i + j forms entry (i, j) of the two
+// staples of the s-th direction and of U V, the factors' rows by shuffles.  About 3 us, where a
+// lane on its own takes 45.
+__device__ __noinline__ void kick_fp64_warp(const Geom &g, const double2 *U, double2 *P, double coef, long site,
+                                            int mu) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31, s = lane / 9, e = lane - 9 * s, i = e / 3, j = e - 3 * i;
+  const int nu = s == 3 ? (mu ? 0 : 1) : s < mu ? s : s + 1;  // (lanes 27 to 31 only take part in the shuffles)
+  int x[4], xp[4], xn[4], xd[4], xpd[4];
+  lex_coords(g, site, x);
+  step(g, x, mu, 1, xp);
+  step(g, x, nu, 1, xn);
+  step(g, x, nu, -1, xd);
+  step(g, xd, mu, 1, xpd);
+  const double2 *un = U + (site * 4 + nu) * 9, *up = U + (lex_of(g, xp) * 4 + nu) * 9,
+                *mn = U + (lex_of(g, xn) * 4 + mu) * 9, *md = U + (lex_of(g, xd) * 4 + mu) * 9,
+                *pd = U + (lex_of(g, xpd) * 4 + nu) * 9, *nd = U + (lex_of(g, xd) * 4 + nu) * 9;
+  auto from = [&](double2 z, int src) {
+    return make_double2(__shfl_sync(kAll, z.x, src & 31), __shfl_sync(kAll, z.y, src & 31));
+  };
+  auto conj = [](double2 z) { return make_double2(z.x, -z.y); };
+  double2 a = make_double2(0.0, 0.0), b = a, f = a, h = a;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    cmac<double>(a, up[i * 3 + k], conj(mn[j * 3 + k]));  // U_nu(x+mu) U_mu(x+nu)^dagger
+    cmac<double>(b, md[i * 3 + k], pd[k * 3 + j]);        // U_mu(x-nu) U_nu(x+mu-nu)
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    cmac<double>(f, from(a, 9 * s + 3 * i + k), conj(un[j * 3 + k]));
+    cmac<double>(h, conj(from(b, 9 * s + 3 * k + i)), nd[k * 3 + j]);
+  }
+  const double2 v = make_double2(f.x + h.x, f.y + h.y);
+  const double2 v0 = from(v, e), v1 = from(v, 9 + e), v2 = from(v, 18 + e);
+  const double2 V = make_double2(v0.x + v1.x + v2.x, v0.y + v1.y + v2.y);
+  double2 w = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) cmac<double>(w, U[(site * 4 + mu) * 9 + i * 3 + k], from(V, 3 * k + j));
+  const double2 t = from(w, 3 * j + i);
+  const double tr = (from(w, 0).y + from(w, 4).y + from(w, 8).y) / 3.0;
+  if (lane < 9) {
+    double2 *p = P + (site * 4 + mu) * 9 + e;
+    const double2 z = *p;
+    *p = make_double2(fma(coef, 0.5 * (w.x - t.x), z.x),
+                      fma(coef, 0.5 * (w.y + t.y) - (i == j ? tr : 0.0), z.y));
+  }
+}
+
 __global__ void __launch_bounds__(128) k_gauge_momentum(Geom g, const double2 *__restrict__ U, double2 *__restrict__ P,
                                                         double coef) {
   const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -327,9 +375,35 @@ __device__ __forceinline__ void row_times(const int4 *a, const int4 *b, long lon
   }
 }
 // Sizes (in units of 2^-20) below which the FP64 form is the more accurate one; see k_gauge_momentum_fx
-constexpr int kOffSize = (1 << 20) / 2, kDiagSize = (1 << 20) / 4;
+constexpr int kOffSize = (int)(0.8 * (1 << 20)), kDiagSize = (int)(0.4 * (1 << 20));
+// Links of a warp that need the FP64 form: up to this many one by one with all lanes
+constexpr int kFew = 12;
 __device__ __forceinline__ int4 conj_if(int4 z, int m) {  // m = -1: the conjugate, 0: z
   return make_int4(z.x, z.y, (z.z ^ m) - m, (z.w ^ m) - m);
+}
+// p += coef TA(w) for w in units of 2^-55
+__device__ __forceinline__ void add_ta_fx(double2 *p, const long long *w, double coef) {
+  // TA(w) = (w - w^dagger)/2 - tr(w - w^dagger)/6; its upper triangle, twice as large
+  const long long tr = (w[1] + w[9] + w[17]) / 3;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double d = fx::value(w[2 * (i * 4) + 1] - tr, -54);
+    double2 z = p[i * 4];
+    z.y = fma(0.5 * coef, d, z.y);
+    p[i * 4] = z;
+#pragma unroll
+    for (int j = i + 1; j < 3; ++j) {
+      const int a = 2 * (i * 3 + j), c = 2 * (j * 3 + i);
+      const double re = fx::value(w[a] - w[c], -55), im = fx::value(w[a + 1] + w[c + 1], -55);
+      double2 z1 = p[i * 3 + j], z2 = p[j * 3 + i];
+      z1.x = fma(0.5 * coef, re, z1.x);
+      z1.y = fma(0.5 * coef, im, z1.y);
+      z2.x = fma(-0.5 * coef, re, z2.x);
+      z2.y = fma(0.5 * coef, im, z2.y);
+      p[i * 3 + j] = z1;
+      p[j * 3 + i] = z2;
+    }
+  }
 }
 }  // namespace
 
@@ -339,16 +413,15 @@ __device__ __forceinline__ int4 conj_if(int4 z, int m) {  // m = -1: the conjuga
 // The loops over staples and rows are not unrolled, and the sum lives in shared memory:
 // unrolled, the warps waited for instructions.  Bound by the integer multiplier, 13 x 243
 // multiply-adds of four clocks per link (175 us at 16^3 x 32), and by the adds and shifts around
-// them at two warps per scheduler.  Measured at 16^3 x 32, with the conversion: 562 us, 1795 us in
+// them at two warps per scheduler.  Measured at 16^3 x 32, with the conversion: 568 us, 1795 us in
 // FP64.  Error of the force (largest entry, relative to the largest of the lattice): links
 // exp(i eps H) with eps = 0.5 8.1e-17, FP64 form 2.3e-16.
 // The error in these units is the same for every link, that of the FP64 form is relative to
 // S_ij = sum_k |U_ik| |V_kj| + |U_jk| |V_ki| off the diagonal and to the largest of
-// sum_k |Re U_ik| |Im V_ki| + |Im U_ik| |Re V_ki| on it.  A link where these are below 1/2 or
-// 1/4 takes the FP64 form; there the largest errors are 3.1e-16 S and 6.2e-16 S (FP64 form
-// 1.6e-16 and 4.2e-16), at twice these sizes they are equal, above the integers are closer.  At
-// eps = 0.5 no link does, at 0.3 hardly one (579 us), at 0.2 few (681 us), from 0.1 down nearly
-// all (1.8 ms; limits of 0.8 and 0.4 took 660 and 1220 us at 0.3 and 0.2).
+// sum_k |Re U_ik| |Im V_ki| + |Im U_ik| |Re V_ki| on it.  They meet where these are 0.8 and 0.4
+// (both forms up to 1.6e-16 S and 4.4e-16 S); a link below either takes the FP64 form, a few
+// of a warp with all its lanes, many each with its own.  At eps = 0.5 no link does, at 0.3
+// one in 2000 (573 us; 660 us with a lane each), at 0.2 646 us (1220), 1.46 ms at 0.1, at most 1.78 ms.
 __global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4 *__restrict__ v,
                                                               const int *__restrict__ ok,
                                                               const double2 *__restrict__ U, double2 *__restrict__ P,
@@ -371,6 +444,7 @@ __global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4
   }
   step(g, x, mu, 1, xp);
   const int sp = (int)lex_of(g, xp);
+  const bool whole = blockIdx.x * 32 + 32 <= nsite;  // every lane of the CTA has a site
   const int flags = ok[mu * nsite + site];
   bool fits = flags & kFits;
 #pragma unroll 1
@@ -384,8 +458,8 @@ __global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4
     const int sx = fwd ? sp : (int)lex_of(g, xq), sz = fwd ? site : sn;
     const int near = flags & ok[nu * nsite + sx] & ok[mu * nsite + sn] & ok[nu * nsite + sz];
     fits = fits && (near & kFits);
-    // one such plaquette in a warp: the FP64 form will be needed at the end, so at once
-    if (q == 0 && __any_sync(__activemask(), near & kWeak)) {
+    // a warp with many such plaquettes: the FP64 form will be needed at the end, so at once
+    if (q == 0 && (whole ? __popc(__ballot_sync(0xffffffffu, near & kWeak)) > kFew : near & kWeak)) {
       kick_fp64(g, U, P, coef, (long)site * 4 + mu);
       return;
     }
@@ -448,31 +522,13 @@ __global__ void __launch_bounds__(128, 2) k_gauge_momentum_fx(Geom g, const int4
     di = max(di, d);
     row_times(a, b, w + 6 * i);
   }
-  if (!fits || min(od[0], min(od[1], od[2])) < kOffSize || di < kDiagSize) {
-    kick_fp64(g, U, P, coef, (long)site * 4 + mu);
-    return;
-  }
-  // TA(w) = (w - w^dagger)/2 - tr(w - w^dagger)/6; its upper triangle, twice as large
-  double2 *p = P + ((long)site * 4 + mu) * 9;
-  const long long tr = (w[1] + w[9] + w[17]) / 3;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const double d = fx::value(w[2 * (i * 4) + 1] - tr, -54);
-    double2 z = p[i * 4];
-    z.y = fma(0.5 * coef, d, z.y);
-    p[i * 4] = z;
-#pragma unroll
-    for (int j = i + 1; j < 3; ++j) {
-      const int a = 2 * (i * 3 + j), c = 2 * (j * 3 + i);
-      const double re = fx::value(w[a] - w[c], -55), im = fx::value(w[a + 1] + w[c + 1], -55);
-      double2 z1 = p[i * 3 + j], z2 = p[j * 3 + i];
-      z1.x = fma(0.5 * coef, re, z1.x);
-      z1.y = fma(0.5 * coef, im, z1.y);
-      z2.x = fma(-0.5 * coef, re, z2.x);
-      z2.y = fma(0.5 * coef, im, z2.y);
-      p[i * 3 + j] = z1;
-      p[j * 3 + i] = z2;
-    }
+  const bool fp64 = !fits || min(od[0], min(od[1], od[2])) < kOffSize || di < kDiagSize;
+  if (!fp64) add_ta_fx(P + ((long)site * 4 + mu) * 9, w, coef);
+  unsigned left = whole ? __ballot_sync(0xffffffffu, fp64) : 0u;
+  if (!whole || __popc(left) > kFew) {
+    if (fp64) kick_fp64(g, U, P, coef, (long)site * 4 + mu);
+  } else {
+    for (; left; left &= left - 1) kick_fp64_warp(g, U, P, coef, (long)blockIdx.x * 32 + __ffs(left) - 1, mu);
   }
 }
 
